@@ -496,6 +496,46 @@ cudaError_t launch_conv(const ConvSrc& s, const __nv_bfloat16* Wt, int Kpad, int
 
 size_t wpart_floats(long long V, int Kpad, int N) { return (size_t)blocks_for(V, kWChunk) * Kpad * N; }
 
+// The bias gradient's partial sums: N per chunk, or kBiasT (k_wgrad_lin).
+size_t bpart_floats(long long V, int N) { return (size_t)blocks_for(V, kWChunk) * std::max(N, kBiasT); }
+
+template <int CL, int BN, int MODE>
+cudaError_t launch_wgrad_lin(const ConvSrc& s, const __nv_bfloat16* g, int N, int Kpad, unsigned chunks, float* wpart,
+                             float* bpart, cudaStream_t st)
+{
+    const size_t smem = LinSmem<BN>::bytes();
+    static bool attr_dev[64] = {};   // the attribute belongs to the current device: set once per device
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    if (!attr_dev[dev]) {
+        const cudaError_t e =
+            cudaFuncSetAttribute(k_wgrad_lin<CL, BN, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        attr_dev[dev] = true;
+    }
+    const dim3 grid(chunks, (unsigned)(3 * (s.C / CL) + kBiasY), (unsigned)((N + BN - 1) / BN));
+    k_wgrad_lin<CL, BN, MODE><<<grid, kLT, smem, st>>>(s, g, N, Kpad, FastDiv(s.W), FastDiv(s.H), wpart, bpart);
+    return cudaGetLastError();
+}
+template <int BN>
+cudaError_t launch_wgrad_lin_c(const ConvSrc& s, const __nv_bfloat16* g, int N, int Kpad, unsigned chunks,
+                               float* wpart, float* bpart, cudaStream_t st)
+{
+    if (s.C == 1) {
+        const dim3 grid(chunks, 2, (unsigned)((N + BN - 1) / BN));
+        k_wgrad_lin1<BN><<<grid, kC1T, 0, st>>>(s, g, N, Kpad, FastDiv(s.W), FastDiv(s.H), wpart, bpart);
+        return cudaGetLastError();
+    }
+    if (s.C % 16 == 0) {
+        if (s.b) return launch_wgrad_lin<16, BN, 2>(s, g, N, Kpad, chunks, wpart, bpart, st);
+        if (s.up) return launch_wgrad_lin<16, BN, 1>(s, g, N, Kpad, chunks, wpart, bpart, st);
+        return launch_wgrad_lin<16, BN, 0>(s, g, N, Kpad, chunks, wpart, bpart, st);
+    }
+    if (s.b) return launch_wgrad_lin<8, BN, 2>(s, g, N, Kpad, chunks, wpart, bpart, st);
+    if (s.up) return launch_wgrad_lin<8, BN, 1>(s, g, N, Kpad, chunks, wpart, bpart, st);
+    return launch_wgrad_lin<8, BN, 0>(s, g, N, Kpad, chunks, wpart, bpart, st);
+}
+
 // gW [N][27 C] and gb [N] of a convolution with input s and output gradient
 // g ([V][N] bfloat16), through the partial buffers.
 cudaError_t launch_wgrad(const ConvSrc& s, const __nv_bfloat16* g, int N, float* wpart, float* bpart, float* gW,
@@ -504,6 +544,20 @@ cudaError_t launch_wgrad(const ConvSrc& s, const __nv_bfloat16* g, int N, float*
     const long long V = (long long)s.D * s.H * s.W;
     const int Kpad = round_up(27 * s.C, kBK);
     const unsigned chunks = blocks_for(V, kWChunk);
+    // staged rows for one-channel sources and multiples of 8 channels (the
+    // same bits as the gather kernel, which keeps the others); at most 32
+    // outputs a CTA, so that the coarse levels' few chunks still spread
+    if (!tiles_disabled() && (s.C == 1 || (s.C % 8 == 0 && !s.f32)) && N <= kBiasT &&
+        !(s.b && s.up) && V < (1LL << 30)) {
+        const cudaError_t e = N <= 8    ? launch_wgrad_lin_c<8>(s, g, N, Kpad, chunks, wpart, bpart, st)
+                              : N <= 16 ? launch_wgrad_lin_c<16>(s, g, N, Kpad, chunks, wpart, bpart, st)
+                                        : launch_wgrad_lin_c<32>(s, g, N, Kpad, chunks, wpart, bpart, st);
+        if (e != cudaSuccess) return e;
+        const int Kvalid = 27 * s.C;
+        k_wgrad_lin_reduce<<<blocks_for((long long)Kvalid * N, 256) + 1, 256, 0, st>>>(wpart, (int)chunks, Kpad,
+                                                                                       Kvalid, N, bpart, gW, gbias);
+        return cudaGetLastError();
+    }
     const int bn = tile_n(N);
     dim3 grid(blocks_for(Kpad, kBM), chunks, (unsigned)((N + bn - 1) / bn));
     if (bn == 16)
@@ -756,7 +810,7 @@ mh3d_status mh3d_unet_create_levels(int nx, int ny, int nz, int levels, const in
         wp = std::max(wp, wpart_floats(n->V[lv], l.Kf, l.cout));
         skn = std::max(skn, std::max(splitk_floats(n->V[lv], l.Nf, l.cout, l.Kf),
                                      splitk_floats(n->V[lv], l.Nb, l.cin, l.Kb)));
-        bp = std::max(bp, (size_t)blocks_for(n->V[lv], kWChunk) * l.cout);
+        bp = std::max(bp, bpart_floats(n->V[lv], l.cout));
         cm = std::max(cm, std::max(l.cin, l.cout));
     }
     n->nparam = off;
@@ -1098,7 +1152,7 @@ mh3d_status mh3d_unet_conv_weight_grad(const mh3d_unet_conv_desc* c, const void*
     const long long V = (long long)c->nx * c->ny * c->nz;
     const int K = round_up(27 * c->cin, kBK);
     Tmp wp(sizeof(float) * wpart_floats(V, K, c->cout));
-    Tmp bp(sizeof(float) * (size_t)blocks_for(V, kWChunk) * c->cout);
+    Tmp bp(sizeof(float) * bpart_floats(V, c->cout));
     if (!wp.p || !bp.p) return MH3D_ERR_OOM;
     if (launch_wgrad(src_from(c), (const __nv_bfloat16*)g, c->cout, (float*)wp.p, (float*)bp.p, gW, gb, st) !=
         cudaSuccess)

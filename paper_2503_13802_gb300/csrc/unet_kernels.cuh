@@ -592,6 +592,458 @@ __global__ void __launch_bounds__(kThreads) k_conv_wgrad(ConvSrc src, const __nv
         }
 }
 
+// ---------------------------------------------------------------------------
+// Weight gradient from staged rows, for sources of 8 n channels.  The sums
+// are the gather kernel's, product for product (chunks of kWChunk
+// consecutive voxels, 16 voxels per mma in ascending order, chunks added in
+// order), so the two give the same bits; what changes is how the operands
+// reach the tensor cores.  One CTA takes a chunk, one dz, one slice of CL
+// channels and BN outputs.  Blocks of 128 voxels (linear index) and their
+// source voxels for the three dy -- 130 consecutive ones each, the linear
+// shift of the tap -- are copied to shared memory once (cp.async, the next
+// block under this block's products), and the three dx taps read the same
+// rows: an A slice (16 weight rows x 16 voxels) is one ldmatrix.trans whose
+// lanes point at their voxel's 16-byte row, or at a zero row where the tap
+// leaves the volume (a 9-bit mask per voxel, formed with the block).  Warp =
+// dy; a warp multiplies its three dx taps (CL = 8: two taps a slice).
+// blockIdx.y past the slices sums the bias.
+//
+// What bounds it: a chunk is 256 dependent mma steps, so the instructions of
+// a step times 256 on one warp per scheduler, whatever the layer; offsets
+// and masks are therefore formed once per thread or block, not per step.
+// The gather form spent that many block barriers and 27 gathers per voxel:
+// at 64x64x64, channels (16, 32, 64), a layer took 270-460 us with it and
+// takes 38-78 us here (a whole training step 5.51 -> 1.81 ms).
+constexpr int kLV = 128;            // voxels per staged block
+constexpr int kLR = kLV + 2;        // staged source voxels per dy
+constexpr int kLS = 24;             // elements per staged voxel (16 + 8: eight rows hit distinct banks)
+constexpr int kLT = 96;             // threads: one warp per dy
+constexpr int kBiasT = 256;         // summands in flight of a bias chunk (k_bias_part's threads)
+constexpr int kBiasY = (kBiasT + kLT - 1) / kLT;   // CTAs per chunk that carry them
+
+// n / d for 0 <= n < 2^31 by a multiplication (d >= 1): m = ceil(2^(31+l) / d),
+// l = ceil(log2 d), has an error below 1, so n m / 2^(31+l) is off by less
+// than 2^-l <= 1/d.
+struct FastDiv {
+    uint32_t d = 1, m = 0, s = 0;
+    FastDiv() = default;
+    explicit FastDiv(int div) : d((uint32_t)div)
+    {
+        uint32_t l = 0;
+        while ((1ull << l) < d) ++l;
+        if (d > 1) {
+            m = (uint32_t)(((1ull << (31 + l)) + d - 1) / d);
+            s = l - 1;
+        }
+    }
+    __device__ __forceinline__ uint32_t div(uint32_t n) const { return d == 1 ? n : __umulhi(n, m) >> s; }
+};
+
+template <int BN>
+struct LinSmem {   // one of the two buffers, elements
+    static constexpr int kSrc = 3 * kLR * kLS;
+    static constexpr int kGrad = kLV * (BN + 8);
+    static constexpr int kBuf = kSrc + kGrad + kLV;   // and the block's masks
+    static constexpr size_t bytes() { return sizeof(__nv_bfloat16) * (2 * (size_t)kBuf + 8); }
+};
+
+__device__ __forceinline__ void lin_cp16(void* sdst, const void* gsrc, bool in)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr(sdst)), "l"(gsrc), "r"(in ? 16u : 0u)
+                 : "memory");
+}
+
+__device__ __forceinline__ void ldsm_x2_t(uint32_t r[2], const void* p)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];"
+                 : "=r"(r[0]), "=r"(r[1])
+                 : "r"(smem_addr(p)));
+}
+
+// The block's output gradients into sG [128][BN + 8]: zero past v1 and N.
+template <int BN, int T>
+__device__ __forceinline__ void lin_stage_grad(__nv_bfloat16* sG, const __nv_bfloat16* __restrict__ dY, int N, int n0,
+                                               int vb, int v1)
+{
+    constexpr int CH = BN / 8;
+#pragma unroll
+    for (int i0 = 0; i0 < kLV * CH; i0 += T) {
+        const int i = i0 + threadIdx.x;
+        if (kLV * CH % T != 0 && i >= kLV * CH) break;
+        const int j = i / CH, c = n0 + (i % CH) * 8;
+        __nv_bfloat16* d = sG + j * (BN + 8) + (i % CH) * 8;
+        const bool in = vb + j < v1 && c < N;
+        const __nv_bfloat16* g = dY + (in ? (size_t)(vb + j) * N + c : 0);
+        if ((N & 7) == 0) {
+            lin_cp16(d, g, in);
+        } else {
+            uint32_t w[4] = {0, 0, 0, 0};
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                if (in && c + e < N) w[e / 2] |= (uint32_t)(*reinterpret_cast<const uint16_t*>(g + e)) << (16 * (e & 1));
+            *reinterpret_cast<uint4*>(d) = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+    }
+}
+
+// The B fragments (all BN outputs) of voxels kk .. kk + 15.
+template <int BN>
+__device__ __forceinline__ void grad_frags(uint32_t (&b)[BN / 8][2], const __nv_bfloat16* sG, int kk, int lane)
+{
+    const int row = kk + (lane & 7) + ((lane >> 3) & 1) * 8;
+    if constexpr (BN == 8) {
+        ldsm_x2_t(b[0], sG + row * (BN + 8));
+    } else {
+#pragma unroll
+        for (int j = 0; j < BN / 16; ++j) {
+            uint32_t r[4];
+            ldsm_x4_t(r, sG + row * (BN + 8) + j * 16 + (lane >> 4) * 8);
+            b[2 * j][0] = r[0];
+            b[2 * j][1] = r[1];
+            b[2 * j + 1][0] = r[2];
+            b[2 * j + 1][1] = r[3];
+        }
+    }
+}
+
+// The bias gradient's chunk sums as k_bias_part forms them: summand t
+// (< per, the largest multiple of N within kBiasT) adds the chunk's elements
+// t, t + per, ... in order; k_wgrad_lin_reduce combines them.
+__device__ __forceinline__ void lin_bias(const __nv_bfloat16* __restrict__ dY, int N, int v0, int v1, int t,
+                                         float* __restrict__ bvs)
+{
+    const int per = (kBiasT / N) * N;
+    if (t >= kBiasT) return;
+    float s = 0.f;
+    if (t < per) {
+        constexpr int U = 32;   // loads in flight
+        const __nv_bfloat16* p = dY + (size_t)v0 * N + t;
+        int left = ((v1 - v0) * N - t + per - 1) / per;
+        for (; left >= U; left -= U, p += U * per) {
+            __nv_bfloat16 q[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) q[u] = p[u * per];
+#pragma unroll
+            for (int u = 0; u < U; ++u) s += bf2f(q[u]);
+        }
+        for (; left > 0; --left, p += per) s += bf2f(*p);
+    }
+    bvs[(size_t)blockIdx.x * kBiasT + t] = s;
+}
+
+// MODE: 0 a plain source, 1 a half-resolution source read by nearest x2
+// upsampling, 2 the rounded sum of two sources (loaded to registers before
+// a block's products and summed into the other buffer after them).
+template <int CL, int BN, int MODE>
+__global__ void __launch_bounds__(kLT) k_wgrad_lin(ConvSrc src, const __nv_bfloat16* __restrict__ dY, int N, int Kpad,
+                                                   FastDiv fw, FastDiv fh, float* __restrict__ part,
+                                                   float* __restrict__ bvs)
+{
+    static_assert(CL == 8 || CL == 16, "channel slice");
+    extern __shared__ __align__(16) unsigned char wl_raw[];
+    constexpr int NT = BN / 8, U = CL == 16 ? 3 : 2, CH = CL / 8;
+    constexpr int SG = LinSmem<BN>::kSrc, SM = SG + LinSmem<BN>::kGrad, BUF = LinSmem<BN>::kBuf;
+    constexpr int IT = (3 * kLR * CH + kLT - 1) / kLT;
+    __nv_bfloat16* sm = reinterpret_cast<__nv_bfloat16*>(wl_raw);
+    __nv_bfloat16* sZ = sm + 2 * BUF;   // 8 zeros
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int D = src.D, H = src.H, W = src.W, C = src.C, V = D * H * W;
+    const int v0 = blockIdx.x * kWChunk, v1 = min(v0 + kWChunk, V);
+    const int nsl = C / CL;
+    if ((int)blockIdx.y >= 3 * nsl) {
+        if (blockIdx.z == 0) lin_bias(dY, N, v0, v1, ((int)blockIdx.y - 3 * nsl) * kLT + threadIdx.x, bvs);
+        return;
+    }
+    const int slice = (int)blockIdx.y / 3, dz = (int)blockIdx.y % 3 - 1;
+    const int n0 = blockIdx.z * BN;
+    if (threadIdx.x < 8) sZ[threadIdx.x] = __float2bfloat16(0.f);
+
+    // this thread's staged units: for dy the source voxels vb - 1 + (dz H +
+    // dy) W + j, j < 130 (zero outside [0, V); a shift that crosses a face is
+    // replaced by the zero row where it is read)
+    int rel[IT], dst[IT];
+#pragma unroll
+    for (int i = 0; i < IT; ++i) {
+        const int q = threadIdx.x + i * kLT, c8 = q % CH, dyi = q / CH / kLR, j = q / CH - dyi * kLR;
+        rel[i] = -1 + j + (dz * H + dyi - 1) * W;
+        dst[i] = q < 3 * kLR * CH ? (dyi * kLR + j) * kLS + c8 * 8 : -1;
+    }
+    const int ch0 = slice * CL + (CH == 2 ? (threadIdx.x & 1) * 8 : 0);   // kLT is even: c8 = thread parity
+    const __nv_bfloat16* sa = src.a + ch0;
+    uint4 ra[MODE == 2 ? IT : 1], rb[MODE == 2 ? IT : 1];
+    auto stage = [&](int vb, __nv_bfloat16* buf) {
+#pragma unroll
+        for (int i = 0; i < IT; ++i) {
+            const int u = vb + rel[i];
+            const bool in = dst[i] >= 0 && (unsigned)u < (unsigned)V;
+            if constexpr (MODE == 2) {
+                ra[i] = rb[i] = make_uint4(0, 0, 0, 0);
+                if (in) {
+                    ra[i] = *reinterpret_cast<const uint4*>(sa + (size_t)u * C);
+                    rb[i] = *reinterpret_cast<const uint4*>(src.b + ch0 + (size_t)u * C);
+                }
+            } else if (dst[i] >= 0) {
+                size_t off = 0;
+                if (MODE == 1 && in) {
+                    const int yz = (int)fw.div(u), x = u - yz * W, z = (int)fh.div(yz), y = yz - z * H;
+                    off = (size_t)(((z >> 1) * (H >> 1) + (y >> 1)) * (W >> 1) + (x >> 1)) * C;
+                } else if (in) {
+                    off = (size_t)u * C;
+                }
+                lin_cp16(buf + dst[i], sa + off, in);
+            }
+        }
+        lin_stage_grad<BN, kLT>(buf + SG, dY, N, n0, vb, v1);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        // the voxels' masks: bit 3 dy + dx set where the tap stays inside
+        for (int j = threadIdx.x; j < kLV; j += kLT) {
+            const int v = vb + j, yz = (int)fw.div(v), x = v - yz * W, z = (int)fh.div(yz), y = yz - z * H;
+            uint32_t m = 0;
+            if (v < v1 && (unsigned)(z + dz) < (unsigned)D) {
+                const uint32_t mx = (x > 0 ? 1u : 0u) | 2u | (x < W - 1 ? 4u : 0u);
+                m = (y > 0 ? mx : 0u) | mx << 3 | (y < H - 1 ? mx << 6 : 0u);
+            }
+            reinterpret_cast<uint16_t*>(buf + SM)[j] = (uint16_t)m;
+        }
+    };
+    auto finish = [&](__nv_bfloat16* buf) {   // MODE 2: the rounded sums into the buffer
+        if constexpr (MODE == 2) {
+#pragma unroll
+            for (int i = 0; i < IT; ++i) {
+                if (dst[i] < 0) continue;
+                __nv_bfloat162* pr = reinterpret_cast<__nv_bfloat162*>(&ra[i]);
+                const __nv_bfloat162* pq = reinterpret_cast<const __nv_bfloat162*>(&rb[i]);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float2 a = __bfloat1622float2(pr[e]), b = __bfloat1622float2(pq[e]);
+                    pr[e] = __floats2bfloat162_rn(a.x + b.x, a.y + b.y);
+                }
+                *reinterpret_cast<uint4*>(buf + dst[i]) = ra[i];
+            }
+        }
+    };
+
+    float acc[U][NT][4];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int t = 0; t < NT; ++t) acc[u][t][0] = acc[u][t][1] = acc[u][t][2] = acc[u][t][3] = 0.f;
+    // this lane's voxel of an A slice: rr of its 16; mh: its 8-row half
+    const int rr = (lane & 7) + 8 * (lane >> 4), mh = (lane >> 3) & 1;
+    const uint32_t zrow = smem_addr(sZ);
+
+    stage(v0, sm);
+    finish(sm);
+    int cur = 0;
+    for (int vb = v0; vb < v1; vb += kLV, cur ^= 1) {
+        const bool more = vb + kLV < v1;
+        if (more) {
+            stage(vb + kLV, sm + (cur ^ 1) * BUF);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        __syncthreads();
+        const __nv_bfloat16* buf = sm + cur * BUF;
+        const uint32_t row = smem_addr(buf + (warp * kLR + rr + 1) * kLS + (CL == 16 ? mh * 8 : 0));   // dx = 0
+        const uint16_t* msk = reinterpret_cast<const uint16_t*>(buf + SM) + rr;
+#pragma unroll
+        for (int ks = 0; ks < kLV / 16; ++ks) {
+            uint32_t b[NT][2];
+            grad_frags<BN>(b, buf + SG, 16 * ks, lane);
+            const uint32_t mk = ((uint32_t)msk[16 * ks] >> (3 * warp)) & 7u;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int dxi = CL == 16 ? u : 2 * u + mh;   // CL = 8: the halves carry two taps (3: none)
+                const uint32_t p = (mk >> dxi) & 1u ? row + (16 * ks + dxi - 1) * kLS * 2 : zrow;
+                uint32_t a[4];
+                asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                             : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3])
+                             : "r"(p));
+#pragma unroll
+                for (int t = 0; t < NT; ++t) mma_bf16(acc[u][t], a, b[t][0], b[t][1]);
+            }
+        }
+        if (more) finish(sm + (cur ^ 1) * BUF);
+        __syncthreads();
+    }
+    // fragment (row lane / 4 [+ 8], columns 2 (lane % 4) + {0, 1})
+    float* P = part + (size_t)blockIdx.x * Kpad * N;
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int t = 0; t < NT; ++t)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int half = e >> 1, r = (lane >> 2);
+                const int dxi = CL == 16 ? u : 2 * u + half;
+                if (dxi > 2) continue;
+                const int k = (9 * (dz + 1) + 3 * warp + dxi) * C + slice * CL + (CL == 16 ? r + 8 * half : r);
+                const int n = n0 + t * 8 + 2 * (lane & 3) + (e & 1);
+                if (n < N) P[(size_t)k * N + n] = acc[u][t][e];
+            }
+}
+
+// The same for one-channel sources (the FP32 network input): the nine
+// (dz, dy) rows of a block are staged as scalars, two threads build a
+// voxel's 27 taps as one row of the operand (16 each), and warp w multiplies
+// taps 16 (w & 1) .. + 15 with outputs 8 (w / 2) .. + 7.
+constexpr int kC1T = 256;
+template <int BN>
+__global__ void __launch_bounds__(kC1T) k_wgrad_lin1(ConvSrc src, const __nv_bfloat16* __restrict__ dY, int N, int Kpad,
+                                                     FastDiv fw, FastDiv fh, float* __restrict__ part,
+                                                     float* __restrict__ bvs)
+{
+    constexpr int NT = BN / 8, IT = (9 * kLR + kC1T - 1) / kC1T;
+    static_assert(2 * NT <= kC1T / 32, "a warp per (tap half, output tile)");
+    __shared__ __align__(16) __nv_bfloat16 sS[9 * kLR + 6];
+    __shared__ __align__(16) __nv_bfloat16 sA[kLV * (kBK + 8)];
+    __shared__ __align__(16) __nv_bfloat16 sG[2][kLV * (BN + 8)];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int D = src.D, H = src.H, W = src.W, V = D * H * W;
+    const int v0 = blockIdx.x * kWChunk, v1 = min(v0 + kWChunk, V);
+    if (blockIdx.y > 0) {
+        if (blockIdx.z == 0) lin_bias(dY, N, v0, v1, threadIdx.x, bvs);
+        return;
+    }
+    const int n0 = blockIdx.z * BN;
+    const float fsc = src.f32_scale ? *src.f32_scale : 1.f;
+    float f[IT];
+    auto fetch = [&](int vb) {
+#pragma unroll
+        for (int i = 0; i < IT; ++i) {
+            const int q = threadIdx.x + i * kC1T, r = q / kLR, j = q - r * kLR;
+            const int u = vb - 1 + j + ((r / 3 - 1) * H + (r % 3 - 1)) * W;
+            float val = 0.f;
+            if (q < 9 * kLR && (unsigned)u < (unsigned)V) {
+                if (src.f32) {
+                    val = src.f32[u] * fsc;
+                } else {
+                    int o = u;
+                    if (src.up) {
+                        const int yz = (int)fw.div(u), x = u - yz * W, z = (int)fh.div(yz), y = yz - z * H;
+                        o = ((z >> 1) * (H >> 1) + (y >> 1)) * (W >> 1) + (x >> 1);
+                    }
+                    val = bf2f(src.a[o]);
+                    if (src.b) val = bf2f(__float2bfloat16(val + bf2f(src.b[o])));
+                }
+            }
+            f[i] = val;
+        }
+    };
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    fetch(v0);
+    lin_stage_grad<BN, kC1T>(sG[0], dY, N, n0, v0, v1);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    int cur = 0;
+    const int un = warp & 1, nt = warp >> 1, jv = threadIdx.x & (kLV - 1), half = threadIdx.x / kLV;
+    for (int vb = v0; vb < v1; vb += kLV, cur ^= 1) {
+#pragma unroll
+        for (int i = 0; i < IT; ++i) {
+            const int q = threadIdx.x + i * kC1T;
+            if (q < 9 * kLR) sS[q] = __float2bfloat16(f[i]);
+        }
+        __syncthreads();
+        if (vb + kLV < v1) {
+            fetch(vb + kLV);
+            lin_stage_grad<BN, kC1T>(sG[cur ^ 1], dY, N, n0, vb + kLV, v1);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        {   // taps 16 half .. + 15 of this thread's voxel, zero where they leave the volume
+            const int v = vb + jv, yz = (int)fw.div(v), x = v - yz * W, z = (int)fh.div(yz), y = yz - z * H;
+            uint32_t m = 0;
+            if (v < v1) {
+                const uint32_t mx = (x > 0 ? 1u : 0u) | 2u | (x < W - 1 ? 4u : 0u);
+                const uint32_t my = (y > 0 ? mx : 0u) | mx << 3 | (y < H - 1 ? mx << 6 : 0u);
+                m = (z > 0 ? my : 0u) | my << 9 | (z < D - 1 ? my << 18 : 0u);
+            }
+            const uint16_t* sp = reinterpret_cast<const uint16_t*>(sS) + jv;
+            uint32_t w[8];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                // tap 16 half + i: its row (tap / 3) and dx + 1 (tap % 3); taps past 26 read row 8
+                const int o0 = (i / 3) * kLR + i % 3, k1 = 16 + i < 27 ? 16 + i : 26, o1 = (k1 / 3) * kLR + k1 % 3;
+                const uint32_t t = sp[half ? o1 : o0];
+                const uint32_t b = (m >> (16 * half + i)) & 1u ? t : 0u;
+                if (i & 1) w[i / 2] |= b << 16;
+                else w[i / 2] = b;
+            }
+            uint4* d = reinterpret_cast<uint4*>(sA + jv * (kBK + 8) + 16 * half);
+            d[0] = make_uint4(w[0], w[1], w[2], w[3]);
+            d[1] = make_uint4(w[4], w[5], w[6], w[7]);
+        }
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncthreads();
+        if (nt < NT) {
+#pragma unroll
+            for (int ks = 0; ks < kLV / 16; ++ks) {
+                uint32_t b[2], a[4];
+                ldsm_x2_t(b, sG[cur] + (16 * ks + (lane & 15)) * (BN + 8) + nt * 8);
+                ldsm_x4_t(a, sA + (16 * ks + (lane & 7) + (lane >> 4) * 8) * (kBK + 8) + un * 16 + ((lane >> 3) & 1) * 8);
+                mma_bf16(acc, a, b[0], b[1]);
+            }
+        }
+        __syncthreads();
+    }
+    if (nt >= NT) return;
+    float* P = part + (size_t)blockIdx.x * Kpad * N;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const int k = 16 * un + (lane >> 2) + 8 * (e >> 1);
+        const int n = n0 + nt * 8 + 2 * (lane & 3) + (e & 1);
+        if (k < 27 && n < N) P[(size_t)k * N + n] = acc[e];
+    }
+}
+
+// gW[n][k] = sum over chunks, in order, of part[chunk][k][n] (as
+// k_wgrad_reduce); the last block's sums gb[n] over
+// the chunks of the bias summands, each chunk's in k_bias_part's order.
+__global__ void __launch_bounds__(256) k_wgrad_lin_reduce(const float* __restrict__ part, int chunks, int Kpad,
+                                                          int Kvalid, int N, const float* __restrict__ bvs,
+                                                          float* __restrict__ gW, float* __restrict__ gb)
+{
+    if (blockIdx.x == gridDim.x - 1) {
+        __shared__ float t_s[2048];   // [chunks of a round][N]
+        const int per = (kBiasT / N) * N, cr = 2048 / N;
+        float s = 0.f;
+        for (int c0 = 0; c0 < chunks; c0 += cr) {
+            const int nc = chunks - c0 < cr ? chunks - c0 : cr;
+            for (int i = threadIdx.x; i < nc * N; i += 256) {
+                const float* q = bvs + (size_t)(c0 + i / N) * kBiasT;
+                float t = 0.f;
+#pragma unroll 8
+                for (int j = i % N; j < per; j += N) t += q[j];
+                t_s[i] = t;
+            }
+            __syncthreads();
+            if ((int)threadIdx.x < N) {
+#pragma unroll 8
+                for (int c = 0; c < nc; ++c) s += t_s[c * N + threadIdx.x];
+            }
+            __syncthreads();
+        }
+        if ((int)threadIdx.x < N) gb[threadIdx.x] = s;
+        return;
+    }
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= Kvalid * N) return;
+    const int k = i / N, n = i % N;
+    const float* q = part + i;   // (c Kpad + k) N + n
+    const size_t cs = (size_t)Kpad * N;
+    float s = 0.f;
+    int c = 0;
+    constexpr int U = 16;   // loads in flight
+    for (; c + U <= chunks; c += U) {
+        float w[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) w[u] = q[(c + u) * cs];
+#pragma unroll
+        for (int u = 0; u < U; ++u) s += w[u];
+    }
+    for (; c < chunks; ++c) s += q[c * cs];
+    gW[(size_t)n * Kvalid + k] = s;
+}
+
 // grad[n][k] (k < Kvalid: the parameter layout W[co][tap][ci]) = sum over
 // chunks, in chunk order, of part[chunk][k][n].
 __global__ void k_wgrad_reduce(const float* __restrict__ part, int chunks, int Kpad, int Kvalid, int N,
