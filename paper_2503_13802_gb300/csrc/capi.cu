@@ -303,7 +303,19 @@ XArgs xpass_args(const Plan& P)
     a.s = P.s;
     a.K = P.K;
     a.rows = P.ny * P.nz;
+    a.dny = FastDiv(P.ny);
     a.M = (long long)a.rows * P.mx;
+    if (P.windowed) {
+        a.M = P.Mf;
+        a.win.on = 1;
+        a.win.pz = P.pad[2];
+        a.win.py = P.pad[1];
+        a.win.pm = P.pad[0] / P.s;
+        a.win.fnz = P.fnz;
+        a.win.fny = P.fny;
+        a.win.fmx = P.fmx;
+        a.win.dny = a.dny;
+    }
     a.pairs = P.tile.xpass_pairs;
     a.kg = P.tile.xpass_kgroup;
     a.vec4 = (P.nx % 4 == 0 && ((uintptr_t)P.sens % 16) == 0) ? 1 : 0;
@@ -338,13 +350,13 @@ cudaError_t launch_forward(const Plan& P, const float* rho, float2* d, float* t1
     xw.vin = t2;
     xw.dout = d;
     xw.ks = P.tile.xw_ks_fwd;
-    if (xw_available(xw, true, P.tile.fwd_path == 2)) {
+    if (!P.windowed && xw_available(xw, true, P.tile.fwd_path == 2)) {
         // T_z, then the warp-centric drive-axis forward
         TArgs tz = tpass_args(P, 2, t1, t2, P.Zhat);
         if ((e = run_tpass(tz, tpass_outer(P, 2), st)) != cudaSuccess) return e;
         return run_xfwd_w(xw, st);
     }
-    if (ct_zxfwd_available(P.nx, P.nz, P.s) && ((uintptr_t)t1 & 15u) == 0) {
+    if (!P.windowed && ct_zxfwd_available(P.nx, P.nz, P.s) && ((uintptr_t)t1 & 15u) == 0) {
         // T_z and the drive-axis forward in one launch (a cluster of CTAs per y-slab)
         ZXArgs z;
         z.x = xpass_args(P);
@@ -371,8 +383,8 @@ cudaError_t launch_adjoint(const Plan& P, const float2* d, float* rho, float* t1
     xw.din = d;
     xw.vout = t1;
     // the plan's tuned path (adj_path: 1 warp fused, 2 warp then T_z^T, 3 CTA-level; 0 the default)
-    const bool warp = P.tile.adj_path != 3 && xw_available(xw, false);
-    const bool fused = !warp && ct_xzadj_available(P.nx, P.nz, P.s) && ((uintptr_t)d & 15u) == 0 &&
+    const bool warp = !P.windowed && P.tile.adj_path != 3 && xw_available(xw, false);
+    const bool fused = !P.windowed && !warp && ct_xzadj_available(P.nx, P.nz, P.s) && ((uintptr_t)d & 15u) == 0 &&
                        ((uintptr_t)t2 & 15u) == 0 && P.mx % 2 == 0 && P.M % 2 == 0;
     if (warp && P.tile.adj_path != 2 && xzw_available(xw, P.nz) && ((uintptr_t)t2 & 15u) == 0) {
         // the warp-centric drive-axis adjoint and T_z^T in one launch (a
@@ -504,12 +516,13 @@ cudaError_t launch_normal(const Plan& P, int mode, const RegArgs& reg, const flo
     xf.dout = portrait;
     if ((e = run_xfwd(xf, st)) != cudaSuccess) return e;
     // a padded plan's data cover the field of view only: A^T A becomes
-    // A^T M A with M the field-of-view mask of the portraits
-    if (P.padded && (e = mask_portraits(P, portrait, st)) != cudaSuccess) return e;
+    // A^T M A with M the field-of-view mask of the portraits (windowed passes
+    // exchange the field of view's portraits only)
+    if (P.padded && !P.windowed && (e = mask_portraits(P, portrait, st)) != cudaSuccess) return e;
     XArgs xa = xpass_args(P);
     xa.din = portrait;
     xa.vout = t1;
-    if ((e = xw_available(xa, false) ? run_xadj_w(xa, st) : run_xadj(xa, st)) != cudaSuccess) return e;
+    if ((e = !P.windowed && xw_available(xa, false) ? run_xadj_w(xa, st) : run_xadj(xa, st)) != cudaSuccess) return e;
     TArgs tz2 = tpass_args(P, 2, t1, t2, P.Zhat_adj);
     if (cg) tz2.cg = cgp;
     if ((e = run_tpass(tz2, tpass_outer(P, 2), st)) != cudaSuccess) return e;
@@ -623,12 +636,17 @@ mh3d_status mh3d_plan_create(const mh3d_geometry* g, void* stream, mh3d_plan* ou
     P->ay.n = ny;
     P->az.n = nz;
     P->am.n = mx;
-    if (!radix_plan(nx, P->ax.rp, 0) || !radix_plan(ny, P->ay.rp, 0) || !radix_plan(nz, P->az.rp, 0) ||
-        !radix_plan(mx, P->am.rp, 0)) {
+    if (!radix_plan(nx, P->ax.rp) || !radix_plan(ny, P->ay.rp) || !radix_plan(nz, P->az.rp) ||
+        !radix_plan(mx, P->am.rp, xpass_max_last(P->s))) {
         delete P;
         return MH3D_ERR_UNSUPPORTED_SIZE;
     }
     choose_tiles(*P);
+    // where no specialised drive-axis pass serves the extended length, the
+    // run-time ones read and write the field of view's portraits directly
+    // (144 x 144 x 72 with 128 x 128 x 64 inside, K = 8: the mask took 23 us
+    // an application, padding 30 us, and the passes moved the padding too)
+    P->windowed = P->padded && xpass_windowed(nx, mx, P->s, P->tile.xpass_pairs);
     if (xfwd_smem_bytes(nx, mx, P->tile.xpass_pairs, P->tile.xpass_kgroup) > kSmemBudget ||
         tpass_smem_bytes(std::max(ny, nz), P->tile.tpass_cols) > kSmemBudget) {
         delete P;
@@ -718,7 +736,7 @@ mh3d_status mh3d_forward(mh3d_plan P, const float* rho, void* d, void* stream)
         return MH3D_ERR_INVALID_ARG;
     }
     P->err.clear();
-    if (P->padded) {   // forward on the extended grid, then the field of view's portraits
+    if (P->padded && !P->windowed) {   // forward on the extended grid, then the field of view's portraits
         mh3d_status s = ensure_portrait(*P);
         if (s != MH3D_OK) return s;
         MH3D_TRY(P, launch_forward(*P, rho, P->w.portrait, P->w.t1, P->w.t2, (cudaStream_t)stream));
@@ -737,7 +755,7 @@ mh3d_status mh3d_adjoint(mh3d_plan P, const void* d, float* rho, void* stream)
         return MH3D_ERR_INVALID_ARG;
     }
     P->err.clear();
-    if (P->padded) {   // the field of view's portraits zero-padded, then the adjoint on the extended grid
+    if (P->padded && !P->windowed) {   // the field of view's portraits zero-padded, then the adjoint on the extended grid
         mh3d_status s = ensure_portrait(*P);
         if (s != MH3D_OK) return s;
         MH3D_TRY(P, pad_portraits(*P, (const float2*)d, P->w.portrait, (cudaStream_t)stream));

@@ -23,47 +23,6 @@
 
 namespace mh3d {
 
-// Radix 16 as 4 x 4: y_{q1 + 4 q2} = sum_{m2} W4^{q2 m2} [W16^{q1 m2} sum_{m1} W4^{q1 m1} v_{4 m1 + m2}].
-template <bool INV>
-__device__ __forceinline__ void dft16(float2* v)
-{
-    constexpr float kH = 0.70710678118654752440f;   // cos(pi/4)
-    constexpr float kC = 0.92387953251128675613f;   // cos(pi/8)
-    constexpr float kS = 0.38268343236508977173f;   // sin(pi/8)
-    float2 a[4][4];
-#pragma unroll
-    for (int m2 = 0; m2 < 4; ++m2) {
-        float2 t[4] = {v[m2], v[4 + m2], v[8 + m2], v[12 + m2]};
-        dft4<INV>(t);
-#pragma unroll
-        for (int q1 = 0; q1 < 4; ++q1) a[q1][m2] = t[q1];
-    }
-    // twiddles W16^{q1 m2} (forward e^{-2 pi i q1 m2 / 16})
-    const float sg = INV ? 1.f : -1.f;
-    // q1 = 1: m2 = 1, 2, 3 -> angles pi/8, pi/4, 3pi/8
-    a[1][1] = c_mul(a[1][1], make_float2(kC, sg * kS));
-    a[1][2] = c_mul(a[1][2], make_float2(kH, sg * kH));
-    a[1][3] = c_mul(a[1][3], make_float2(kS, sg * kC));
-    // q1 = 2: angles pi/4, pi/2, 3pi/4
-    a[2][1] = c_mul(a[2][1], make_float2(kH, sg * kH));
-    a[2][2] = c_rot<INV>(a[2][2]);
-    a[2][3] = c_mul(a[2][3], make_float2(-kH, sg * kH));
-    // q1 = 3: angles 3pi/8, 3pi/4, 9pi/8
-    a[3][1] = c_mul(a[3][1], make_float2(kS, sg * kC));
-    a[3][2] = c_mul(a[3][2], make_float2(-kH, sg * kH));
-    a[3][3] = c_mul(a[3][3], make_float2(-kC, -sg * kS));
-#pragma unroll
-    for (int q1 = 0; q1 < 4; ++q1) {
-        dft4<INV>(a[q1]);
-#pragma unroll
-        for (int q2 = 0; q2 < 4; ++q2) v[q1 + 4 * q2] = a[q1][q2];
-    }
-}
-template <>
-__device__ __forceinline__ void dft<16, false>(float2* v) { dft16<false>(v); }
-template <>
-__device__ __forceinline__ void dft<16, true>(float2* v) { dft16<true>(v); }
-
 namespace ct {
 
 // ---------------------------------------------------------------------------

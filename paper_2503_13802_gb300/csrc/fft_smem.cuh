@@ -1,6 +1,7 @@
 // Shared-memory Stockham FFT engine for batches of short pencils (sm_103a).
 //
-// A batch is P pencils of one length n (2^a 3^b, n <= 1024).  Element e of
+// A batch is P pencils of one length n (2^a 3^b, n <= 1024; P a power of
+// two).  Element e of
 // pencil p lives at buf[e * ld + p] (pencil index fastest), so consecutive
 // threads touch consecutive float2 words: a half warp covers 128 contiguous
 // bytes, which is bank-conflict free for 64-bit accesses.  ld = P + 1 keeps
@@ -22,8 +23,8 @@
 // global memory.
 //
 // Twiddle tables (W_n^t, t < n) come from the host, computed in FP64 and
-// rounded once; the DFT kernels use only the exact constants 1/2, sqrt(3)/2
-// and sqrt(1/2).
+// rounded once; the DFT kernels' constants are the sines and cosines of
+// multiples of pi / 8, pi / 9 and pi / 6.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -133,100 +134,320 @@ __device__ __forceinline__ void dft<8, false>(float2* v) { dft8<false>(v); }
 template <>
 __device__ __forceinline__ void dft<8, true>(float2* v) { dft8<true>(v); }
 
-// Plain shared-memory buffer access.
+// Radix 9 as 3 x 3: y_{q1 + 3 q2} = sum_{m2} W3^{q2 m2} [W9^{q1 m2} sum_{m1} W3^{q1 m1} v_{3 m1 + m2}].
+template <bool INV>
+__device__ __forceinline__ void dft9(float2* v)
+{
+    constexpr float kC1 = 0.76604444311897803520f, kS1 = 0.64278760968653932632f;   // 2 pi / 9
+    constexpr float kC2 = 0.17364817766693034885f, kS2 = 0.98480775301220805937f;   // 4 pi / 9
+    constexpr float kC4 = -0.93969262078590838405f, kS4 = 0.34202014332566873304f;  // 8 pi / 9
+    const float sg = INV ? 1.f : -1.f;
+    float2 a[3][3];
+#pragma unroll
+    for (int m2 = 0; m2 < 3; ++m2) {
+        float2 t[3] = {v[m2], v[3 + m2], v[6 + m2]};
+        dft3<INV>(t);
+#pragma unroll
+        for (int q1 = 0; q1 < 3; ++q1) a[q1][m2] = t[q1];
+    }
+    a[1][1] = c_mul(a[1][1], make_float2(kC1, sg * kS1));
+    a[1][2] = c_mul(a[1][2], make_float2(kC2, sg * kS2));
+    a[2][1] = c_mul(a[2][1], make_float2(kC2, sg * kS2));
+    a[2][2] = c_mul(a[2][2], make_float2(kC4, sg * kS4));
+#pragma unroll
+    for (int q1 = 0; q1 < 3; ++q1) {
+        dft3<INV>(a[q1]);
+#pragma unroll
+        for (int q2 = 0; q2 < 3; ++q2) v[q1 + 3 * q2] = a[q1][q2];
+    }
+}
+template <>
+__device__ __forceinline__ void dft<9, false>(float2* v) { dft9<false>(v); }
+template <>
+__device__ __forceinline__ void dft<9, true>(float2* v) { dft9<true>(v); }
+
+// Radix A B for coprime A, B by the prime-factor map (Good 1958): with
+// n = B n1 + A n2 (mod A B) and k = k1 e1 + k2 e2 (mod A B), e1 = 1 (mod A),
+// 0 (mod B) and e2 the other way round, W^{n k} = W_A^{n1 k1} W_B^{n2 k2}:
+// no twiddles.  2 x 3 (e = 3, 4) and 3 x 4 (e = 4, 9).
+template <int A, int B, int E1, int E2, bool INV>
+__device__ __forceinline__ void dft_pf(float2* v)
+{
+    float2 t[A][B];
+#pragma unroll
+    for (int n1 = 0; n1 < A; ++n1) {
+#pragma unroll
+        for (int n2 = 0; n2 < B; ++n2) t[n1][n2] = v[(B * n1 + A * n2) % (A * B)];
+        dft<B, INV>(t[n1]);
+    }
+#pragma unroll
+    for (int k2 = 0; k2 < B; ++k2) {
+        float2 u[A];
+#pragma unroll
+        for (int n1 = 0; n1 < A; ++n1) u[n1] = t[n1][k2];
+        dft<A, INV>(u);
+#pragma unroll
+        for (int k1 = 0; k1 < A; ++k1) v[(k1 * E1 + k2 * E2) % (A * B)] = u[k1];
+    }
+}
+template <>
+__device__ __forceinline__ void dft<6, false>(float2* v) { dft_pf<2, 3, 3, 4, false>(v); }
+template <>
+__device__ __forceinline__ void dft<6, true>(float2* v) { dft_pf<2, 3, 3, 4, true>(v); }
+template <>
+__device__ __forceinline__ void dft<12, false>(float2* v) { dft_pf<3, 4, 4, 9, false>(v); }
+template <>
+__device__ __forceinline__ void dft<12, true>(float2* v) { dft_pf<3, 4, 4, 9, true>(v); }
+
+// Radix 16 as 4 x 4: y_{q1 + 4 q2} = sum_{m2} W4^{q2 m2} [W16^{q1 m2} sum_{m1} W4^{q1 m1} v_{4 m1 + m2}].
+template <bool INV>
+__device__ __forceinline__ void dft16(float2* v)
+{
+    constexpr float kH = 0.70710678118654752440f;   // cos(pi/4)
+    constexpr float kC = 0.92387953251128675613f;   // cos(pi/8)
+    constexpr float kS = 0.38268343236508977173f;   // sin(pi/8)
+    float2 a[4][4];
+#pragma unroll
+    for (int m2 = 0; m2 < 4; ++m2) {
+        float2 t[4] = {v[m2], v[4 + m2], v[8 + m2], v[12 + m2]};
+        dft4<INV>(t);
+#pragma unroll
+        for (int q1 = 0; q1 < 4; ++q1) a[q1][m2] = t[q1];
+    }
+    // twiddles W16^{q1 m2} (forward e^{-2 pi i q1 m2 / 16})
+    const float sg = INV ? 1.f : -1.f;
+    // q1 = 1: m2 = 1, 2, 3 -> angles pi/8, pi/4, 3pi/8
+    a[1][1] = c_mul(a[1][1], make_float2(kC, sg * kS));
+    a[1][2] = c_mul(a[1][2], make_float2(kH, sg * kH));
+    a[1][3] = c_mul(a[1][3], make_float2(kS, sg * kC));
+    // q1 = 2: angles pi/4, pi/2, 3pi/4
+    a[2][1] = c_mul(a[2][1], make_float2(kH, sg * kH));
+    a[2][2] = c_rot<INV>(a[2][2]);
+    a[2][3] = c_mul(a[2][3], make_float2(-kH, sg * kH));
+    // q1 = 3: angles 3pi/8, 3pi/4, 9pi/8
+    a[3][1] = c_mul(a[3][1], make_float2(kS, sg * kC));
+    a[3][2] = c_mul(a[3][2], make_float2(-kH, sg * kH));
+    a[3][3] = c_mul(a[3][3], make_float2(-kC, -sg * kS));
+#pragma unroll
+    for (int q1 = 0; q1 < 4; ++q1) {
+        dft4<INV>(a[q1]);
+#pragma unroll
+        for (int q2 = 0; q2 < 4; ++q2) v[q1 + 4 * q2] = a[q1][q2];
+    }
+}
+template <>
+__device__ __forceinline__ void dft<16, false>(float2* v) { dft16<false>(v); }
+template <>
+__device__ __forceinline__ void dft<16, true>(float2* v) { dft16<true>(v); }
+
+// Plain shared-memory buffer access.  Loaders and storers of the run-time
+// stages give at(p), the access to one pencil's elements, so that what
+// depends on the pencil only is formed once per butterfly.
 struct BufLd {
     const float2* b;
     int ld;
     __device__ __forceinline__ float2 operator()(int e, int p) const { return b[e * ld + p]; }
+    struct At {
+        const float2* b;
+        int ld;
+        __device__ __forceinline__ float2 operator()(int e) const { return b[e * ld]; }
+    };
+    __device__ __forceinline__ At at(int p) const { return At{b + p, ld}; }
 };
 struct BufSt {
     float2* b;
     int ld;
     __device__ __forceinline__ void operator()(int e, int p, float2 v) const { b[e * ld + p] = v; }
+    struct At {
+        float2* b;
+        int ld;
+        __device__ __forceinline__ void operator()(int e, float2 v) const { b[e * ld] = v; }
+    };
+    __device__ __forceinline__ At at(int p) const { return At{b + p, ld}; }
 };
 
-// One radix-R Stockham stage over P pencils of length n.
-template <int R, bool INV, bool PFAST, class LD, class ST>
-__device__ __forceinline__ void fft_stage(const LD& ld, const ST& st, int n, int Ns, int P,
-                                          const float2* __restrict__ tw)
+// ---------------------------------------------------------------------------
+// Run-time schedules.  A stage's radix is a template parameter (one switch
+// per stage), its length, strides and divisions are uniform values; the
+// pencil count is a power of two, 1 << lgP.
+// ---------------------------------------------------------------------------
+// Geometry of stage s of a schedule: butterflies nb = n / R, Ns = product
+// of the earlier radices, and the divisions by both.
+struct StageGeom {
+    int n, nb, Ns, R;
+    FastDiv dnb, dns;
+};
+__device__ __forceinline__ StageGeom stage_fwd(const RadixPlan& pl, int s)
 {
-    const int nb = n / R;
-    const int total = nb * P;
-    const int tstep = n / (Ns * R);
+    return StageGeom{pl.n, (int)pl.dnb[s].d, pl.ns[s], pl.radix[s], pl.dnb[s], pl.dns[s]};
+}
+// Stage i of the reversed schedule (the inverse transforms).
+__device__ __forceinline__ StageGeom stage_rev(const RadixPlan& pl, int i)
+{
+    const int s = pl.nst - 1 - i;
+    return StageGeom{pl.n, (int)pl.dnb[s].d, pl.nsr[s], pl.radix[s], pl.dnb[s], pl.dnsr[s]};
+}
+
+// Butterfly idx of a stage: pencil and butterfly number, pencils fastest
+// (PFAST) or butterflies fastest.
+template <bool PFAST>
+__device__ __forceinline__ void stage_index(int idx, const StageGeom& g, int lgP, int& p, int& j)
+{
+    if (PFAST) {
+        p = idx & ((1 << lgP) - 1);
+        j = idx >> lgP;
+    } else {
+        p = (int)g.dnb.div((uint32_t)idx);
+        j = idx - p * g.nb;
+    }
+}
+
+// The twiddles W_{Ns R}^{r k} of a butterfly (k = j mod Ns) applied to v.
+template <int R, bool INV>
+__device__ __forceinline__ void stage_twiddle(float2* v, int k, const StageGeom& g, const float2* __restrict__ tw)
+{
+    // table step n / (Ns R) = nb / Ns; a stage past the first has k < Ns
+    const int step = k * (g.Ns == g.nb ? 1 : (int)g.dns.div((uint32_t)g.nb));
+#pragma unroll
+    for (int r = 1; r < R; ++r) {
+        float2 w = tw[r * step];
+        if (INV) w.y = -w.y;
+        v[r] = c_mul(v[r], w);
+    }
+}
+
+// One radix-R Stockham stage over 1 << lgP pencils.
+template <int R, bool INV, bool PFAST, class LD, class ST>
+__device__ __forceinline__ void rt_stage(const LD& ld, const ST& st, const StageGeom& g, int lgP,
+                                         const float2* __restrict__ tw)
+{
+    const int total = g.nb << lgP;
     for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
         int p, j;
-        if (PFAST) {
-            p = idx % P;
-            j = idx / P;
-        } else {
-            j = idx % nb;
-            p = idx / nb;
-        }
-        const int k = j % Ns;
+        stage_index<PFAST>(idx, g, lgP, p, j);
         float2 v[R];
+        const auto lp = ld.at(p);
 #pragma unroll
-        for (int r = 0; r < R; ++r) v[r] = ld(j + r * nb, p);
-        if (Ns > 1) {
-#pragma unroll
-            for (int r = 1; r < R; ++r) {
-                float2 w = tw[r * k * tstep];
-                if (INV) w.y = -w.y;
-                v[r] = c_mul(v[r], w);
-            }
+        for (int r = 0; r < R; ++r) v[r] = lp(j + r * g.nb);
+        int dst;
+        if (g.Ns == 1) {
+            dst = j * R;
+        } else if (g.Ns == g.nb) {
+            dst = j;
+            stage_twiddle<R, INV>(v, j, g, tw);
+        } else {
+            const int q = (int)g.dns.div((uint32_t)j), k = j - q * g.Ns;
+            dst = q * g.Ns * R + k;
+            stage_twiddle<R, INV>(v, k, g, tw);
         }
         dft<R, INV>(v);
-        const int dst = (j - k) * R + k;
+        const auto sp = st.at(p);
 #pragma unroll
-        for (int r = 0; r < R; ++r) st(dst + r * Ns, p, v[r]);
+        for (int r = 0; r < R; ++r) sp(dst + r * g.Ns, v[r]);
     }
 }
 
 template <bool INV, bool PFAST, class LD, class ST>
-__device__ __forceinline__ void fft_stage_dispatch(int R, const LD& ld, const ST& st, int n, int Ns, int P,
-                                                   const float2* tw)
+__device__ __forceinline__ void rt_stage_any(const LD& ld, const ST& st, const StageGeom& g, int lgP,
+                                             const float2* __restrict__ tw)
 {
-    switch (R) {
-        case 8: fft_stage<8, INV, PFAST>(ld, st, n, Ns, P, tw); break;
-        case 4: fft_stage<4, INV, PFAST>(ld, st, n, Ns, P, tw); break;
-        case 2: fft_stage<2, INV, PFAST>(ld, st, n, Ns, P, tw); break;
-        case 3: fft_stage<3, INV, PFAST>(ld, st, n, Ns, P, tw); break;
+    switch (g.R) {
+        case 16: rt_stage<16, INV, PFAST>(ld, st, g, lgP, tw); break;
+        case 12: rt_stage<12, INV, PFAST>(ld, st, g, lgP, tw); break;
+        case 9: rt_stage<9, INV, PFAST>(ld, st, g, lgP, tw); break;
+        case 8: rt_stage<8, INV, PFAST>(ld, st, g, lgP, tw); break;
+        case 6: rt_stage<6, INV, PFAST>(ld, st, g, lgP, tw); break;
+        case 4: rt_stage<4, INV, PFAST>(ld, st, g, lgP, tw); break;
+        case 3: rt_stage<3, INV, PFAST>(ld, st, g, lgP, tw); break;
+        case 2: rt_stage<2, INV, PFAST>(ld, st, g, lgP, tw); break;
         default: break;
     }
 }
 
-// Full transform of P pencils: first stage reads `first`, last stage writes
-// `last`, intermediate stages use scratch buffers s0 (written by stage 0,
-// 2, ...) and s1 (stage 1, 3, ...), both with leading dimension lds >= P.
-// `last` may target either scratch buffer only if that buffer is not read by
-// the last stage: the caller guarantees it (see fft_result_buf).
-// FIRST_PFAST / LAST_PFAST choose the mapping of the first / last stage
-// (a single-stage transform uses LAST_PFAST).  Length 1 copies.
+// A stage between shared-memory buffers, pencils fastest: one copy of the
+// code per kernel file (the stages between a transform's first and last).
+template <bool INV>
+__device__ __noinline__ void rt_stage_buf(const float2* src, float2* dst, int lds, const StageGeom& g, int lgP,
+                                          const float2* __restrict__ tw)
+{
+    rt_stage_any<INV, true>(BufLd{src, lds}, BufSt{dst, lds}, g, lgP, tw);
+}
+
+// The last forward stage, a multiplication by mu (element e by mu[e]) and the
+// first inverse stage on the same butterflies, in registers.
+template <int R, class LD, class ST>
+__device__ __forceinline__ void rt_conv(const LD& ld, const ST& st, const float2* __restrict__ mu, const StageGeom& g, int lgP,
+                                        const float2* __restrict__ tw)
+{
+    const int total = g.nb << lgP;
+    for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
+        const int p = idx & ((1 << lgP) - 1), j = idx >> lgP;
+        float2 v[R];
+        const auto lp = ld.at(p);
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = lp(j + r * g.nb);
+        if (g.Ns > 1) {
+#pragma unroll
+            for (int r = 1; r < R; ++r) v[r] = c_mul(v[r], tw[r * j]);
+        }
+        dft<R, false>(v);
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = c_mul(v[r], mu[j + r * g.nb]);
+        dft<R, true>(v);
+        const auto sp = st.at(p);
+#pragma unroll
+        for (int r = 0; r < R; ++r) sp(j * R + r, v[r]);
+    }
+}
+template <class LD, class ST>
+__device__ __forceinline__ void rt_conv_any(const LD& ld, const ST& st, const float2* __restrict__ mu,
+                                            const StageGeom& g, int lgP, const float2* __restrict__ tw)
+{
+    switch (g.R) {
+        case 16: rt_conv<16>(ld, st, mu, g, lgP, tw); break;
+        case 12: rt_conv<12>(ld, st, mu, g, lgP, tw); break;
+        case 9: rt_conv<9>(ld, st, mu, g, lgP, tw); break;
+        case 8: rt_conv<8>(ld, st, mu, g, lgP, tw); break;
+        case 6: rt_conv<6>(ld, st, mu, g, lgP, tw); break;
+        case 4: rt_conv<4>(ld, st, mu, g, lgP, tw); break;
+        case 3: rt_conv<3>(ld, st, mu, g, lgP, tw); break;
+        case 2: rt_conv<2>(ld, st, mu, g, lgP, tw); break;
+        default: break;
+    }
+}
+
+// Full transform of P (a power of two) pencils: first stage reads `first`,
+// last stage writes `last`, intermediate stages use scratch buffers s0
+// (written by stage 0, 2, ...) and s1 (stage 1, 3, ...), both with leading
+// dimension lds >= P.  `last` may target either scratch buffer only if that
+// buffer is not read by the last stage: the caller guarantees it (see
+// fft_result_index).  FIRST_PFAST / LAST_PFAST choose the mapping of the
+// first / last stage (a single-stage transform uses LAST_PFAST).  The
+// inverse runs the schedule reversed.  Length 1 copies.
 template <bool INV, bool FIRST_PFAST, bool LAST_PFAST, class LD, class ST>
 __device__ __forceinline__ void fft_run(const RadixPlan& pl, const LD& first, const ST& last, float2* s0,
                                         float2* s1, int lds, int P, const float2* tw)
 {
-    const int n = pl.n;
+    const int lgP = 31 - __clz(P);
     if (pl.nst == 0) {
-        for (int p = threadIdx.x; p < P; p += blockDim.x) last(0, p, first(0, p));
+        for (int p = threadIdx.x; p < P; p += blockDim.x) last.at(p)(0, first.at(p)(0));
         __syncthreads();
         return;
     }
-    int Ns = 1;
     for (int s = 0; s < pl.nst; ++s) {
-        const int R = pl.radix[s];
+        const StageGeom g = INV ? stage_rev(pl, s) : stage_fwd(pl, s);
         const bool isFirst = (s == 0), isLast = (s == pl.nst - 1);
         float2* dstb = (s & 1) ? s1 : s0;
         const float2* srcb = (s & 1) ? s0 : s1;   // buffer written by stage s-1
         if (isFirst && isLast) {
-            fft_stage_dispatch<INV, LAST_PFAST>(R, first, last, n, Ns, P, tw);
+            rt_stage_any<INV, LAST_PFAST>(first, last, g, lgP, tw);
         } else if (isFirst) {
-            fft_stage_dispatch<INV, FIRST_PFAST>(R, first, BufSt{dstb, lds}, n, Ns, P, tw);
+            rt_stage_any<INV, FIRST_PFAST>(first, BufSt{dstb, lds}, g, lgP, tw);
         } else if (isLast) {
-            fft_stage_dispatch<INV, LAST_PFAST>(R, BufLd{srcb, lds}, last, n, Ns, P, tw);
+            rt_stage_any<INV, LAST_PFAST>(BufLd{srcb, lds}, last, g, lgP, tw);
         } else {
-            fft_stage_dispatch<INV, true>(R, BufLd{srcb, lds}, BufSt{dstb, lds}, n, Ns, P, tw);
+            rt_stage_buf<INV>(srcb, dstb, lds, g, lgP, tw);
         }
-        Ns *= R;
         __syncthreads();
     }
 }

@@ -39,7 +39,7 @@
 namespace mh3d {
 namespace {
 
-constexpr int kGP = 8;      // pencils per CTA
+constexpr int kGPMin = 8, kGPMax = 32;   // pencils per CTA of k_gen_line (gen_pencils)
 constexpr int kGT = 128;    // threads per CTA
 constexpr int kGB = 256;    // threads per CTA of the pointwise kernels
 
@@ -81,6 +81,19 @@ struct GenLd {
         const long long b = base[p];
         return b < 0 ? make_float2(0.f, 0.f) : v[b + e * stride];
     }
+    struct At {
+        const float2* v;   // the pencil, or null
+        long long stride;
+        __device__ __forceinline__ float2 operator()(int e) const
+        {
+            return v ? v[e * stride] : make_float2(0.f, 0.f);
+        }
+    };
+    __device__ __forceinline__ At at(int p) const
+    {
+        const long long b = base[p];
+        return At{b < 0 ? nullptr : v + b, stride};
+    }
 };
 struct GenSt {
     float2* v;
@@ -91,24 +104,40 @@ struct GenSt {
         const long long b = base[p];
         if (b >= 0) v[b + e * stride] = x;
     }
+    struct At {
+        float2* v;
+        long long stride;
+        __device__ __forceinline__ void operator()(int e, float2 x) const
+        {
+            if (v) v[e * stride] = x;
+        }
+    };
+    __device__ __forceinline__ At at(int p) const
+    {
+        const long long b = base[p];
+        return At{b < 0 ? nullptr : v + b, stride};
+    }
 };
 
-// One transform along an axis, in place: every CTA owns kGP whole pencils;
+// One transform along an axis, in place: every CTA owns 1 << lgP whole pencils;
 // the first stage reads all of them before the last stage writes.  PF: the
-// first and last stages walk pencils fastest (axes y and z, where the kGP
-// pencils are neighbours in memory); along x they walk elements fastest.
+// first and last stages walk pencils fastest (axes y and z, where the
+// pencils are neighbours in memory); along x they walk elements fastest, on a
+// padded pencil stride (no bank conflicts).
 template <bool INV, bool PF>
-__global__ void __launch_bounds__(kGT) k_gen_line(float2* v, Pencils g, RadixPlan pl, const float2* __restrict__ tw)
+__global__ void __launch_bounds__(kGT) k_gen_line(float2* v, Pencils g, RadixPlan pl, int lgP,
+                                                   const float2* __restrict__ tw)
 {
     extern __shared__ float2 gsm[];
-    __shared__ long long sbase[kGP];
+    __shared__ long long sbase[kGPMax];
+    const int P = 1 << lgP, lds = P + (PF ? 0 : 1);
     float2* s0 = gsm;
-    float2* s1 = gsm + (size_t)pl.n * kGP;
-    const long long p0 = (long long)blockIdx.x * kGP, np = g.count();
-    if (threadIdx.x < kGP) sbase[threadIdx.x] = p0 + threadIdx.x < np ? g.base(p0 + threadIdx.x) : -1;
+    float2* s1 = gsm + (size_t)pl.n * lds;
+    const long long p0 = (long long)blockIdx.x * P, np = g.count();
+    if (threadIdx.x < P) sbase[threadIdx.x] = p0 + threadIdx.x < np ? g.base(p0 + threadIdx.x) : -1;
     __syncthreads();
     const long long sd = g.stride();
-    fft_run<INV, PF, PF>(pl, GenLd{v, sbase, sd}, GenSt{v, sbase, sd}, s0, s1, kGP, kGP, tw);
+    fft_run<INV, PF, PF>(pl, GenLd{v, sbase, sd}, GenSt{v, sbase, sd}, s0, s1, lds, P, tw);
 }
 
 // Fused pre- and post-steps of the compile-time pencil kernel (MODE):
@@ -490,7 +519,7 @@ cudaError_t gen_set_attributes()
     if (dev < 0 || dev >= kGenMaxDevices) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lk(g_gen_attr_mu);
     if (g_gen_attr_done[dev]) return cudaSuccess;
-    const int smem = (int)(sizeof(float2) * 2 * (size_t)kMaxLen * kGP);
+    const int smem = (int)(sizeof(float2) * 2 * (size_t)kMaxLen * (kGPMin + 1));
     e = cudaFuncSetAttribute(k_gen_line<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_gen_line<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -533,6 +562,20 @@ void gen_line_ct(int grid, float2* v, const Pencils& g, const float2* tw, bool i
     else gen_line_ct_launch<L, false, false>(grid, v, g, tw, mode, io, st);
 }
 
+// log2 of the pencils a CTA of k_gen_line takes: 8, doubled while the stage
+// with the fewest butterflies has less than one per thread (36 = 6 x 6: 48
+// butterflies for 128 threads on 8 pencils) and a CTA per SM remains, up to 32.
+// The shared memory stays below that of 1024-element pencils, 8 at a time:
+// a stage of radix R <= 16 has n / R >= n / 16 butterflies a pencil, so P > 8
+// takes n P <= 16 x 128 x 2.
+int gen_lg_pencils(const RadixPlan& rp, long long np)
+{
+    int nb = rp.n, lg = 3;
+    for (int s = 0; s < rp.nst; ++s) nb = std::min(nb, rp.n / rp.radix[s]);
+    while ((1 << lg) < kGPMax && (nb << lg) < kGT && (np >> (lg + 1)) >= 152) ++lg;
+    return lg;
+}
+
 // Transform of every pencil of `vols` volumes (rows of width W, vstride
 // float2 apart) along `axis`, in place, or with a fused step (mode, io: see
 // GenIO; modes other than 0 need gen_ct_length(ap.n)).
@@ -550,13 +593,14 @@ cudaError_t gen_line(float2* v, int axis, int W, int ny, int nz, int vols, long 
         return cudaGetLastError();
     }
     if (mode != 0) return cudaErrorInvalidValue;
-    const size_t smem = sizeof(float2) * 2 * (size_t)ap.n * kGP;
-    const int grid = (int)((np + kGP - 1) / kGP);
     const bool pf = axis != 0;
-    if (inv && pf) k_gen_line<true, true><<<grid, kGT, smem, st>>>(v, g, ap.rp, ap.tw);
-    else if (inv) k_gen_line<true, false><<<grid, kGT, smem, st>>>(v, g, ap.rp, ap.tw);
-    else if (pf) k_gen_line<false, true><<<grid, kGT, smem, st>>>(v, g, ap.rp, ap.tw);
-    else k_gen_line<false, false><<<grid, kGT, smem, st>>>(v, g, ap.rp, ap.tw);
+    const int lgP = gen_lg_pencils(ap.rp, np), P = 1 << lgP;
+    const size_t smem = sizeof(float2) * 2 * (size_t)ap.n * (P + (pf ? 0 : 1));
+    const int grid = (int)((np + P - 1) / P);
+    if (inv && pf) k_gen_line<true, true><<<grid, kGT, smem, st>>>(v, g, ap.rp, lgP, ap.tw);
+    else if (inv) k_gen_line<true, false><<<grid, kGT, smem, st>>>(v, g, ap.rp, lgP, ap.tw);
+    else if (pf) k_gen_line<false, true><<<grid, kGT, smem, st>>>(v, g, ap.rp, lgP, ap.tw);
+    else k_gen_line<false, false><<<grid, kGT, smem, st>>>(v, g, ap.rp, lgP, ap.tw);
     return cudaGetLastError();
 }
 

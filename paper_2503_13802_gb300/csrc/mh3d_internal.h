@@ -10,20 +10,29 @@
 #include <cuda_runtime.h>
 
 #include "../../include/mh3d.h"
+#include "fastdiv.h"
 
 namespace mh3d {
 
 using cplx = std::complex<double>;
 
-constexpr int kMaxStages = 8;     // radix stages per 1D length (2^a 3^b <= 1024)
+constexpr int kMaxStages = 4;     // radix stages per 1D length (2^a 3^b <= 1024 takes at most 3)
 constexpr int kMaxLen = 1024;     // longest supported axis
 constexpr int kMaxK = 31;         // harmonics per plan
 
-// Radix schedule of one 1D length; passed to kernels by value.
+// Radix schedule of one 1D length; passed to kernels by value.  Stage s of
+// a forward transform has radix[s]; an inverse runs the schedule reversed
+// (radix[nst - 1] first), so that the last forward and the first inverse
+// stage share their butterflies.
 struct RadixPlan {
-    int n;
-    int nst;
-    int radix[kMaxStages];
+    int n = 1;
+    int nst = 0;
+    int radix[kMaxStages] = {1, 1, 1, 1};
+    int ns[kMaxStages] = {1, 1, 1, 1};    // product of the radices before stage s
+    int nsr[kMaxStages] = {1, 1, 1, 1};   // product of the radices after stage s (those before it in the reverse)
+    FastDiv dnb[kMaxStages];              // by n / radix[s]
+    FastDiv dns[kMaxStages];              // by ns[s]
+    FastDiv dnsr[kMaxStages];             // by nsr[s]
 };
 
 // One axis of the plan: length, radix schedule, twiddle table (device).
@@ -122,6 +131,9 @@ struct Plan {
     int fnx = 1, fny = 1, fnz = 1, fmx = 1;
     long long Mf = 1;
     bool padded = false;
+    // the padded plan's drive-axis passes read and write field-of-view
+    // portraits themselves (run-time kernels): no extended portraits, no mask
+    bool windowed = false;
     double vox[3] = {1, 1, 1};
     double gamma = 1, gammaA = 1, tratio = 0.5;
     std::vector<double> theta;
@@ -190,7 +202,12 @@ std::vector<cplx> drive_spectrum(int n, double dx, int k, double gamma, double g
 std::vector<cplx> transverse_spectrum(int n, double d, double gt);
 std::vector<cplx> twiddles(int n);
 double hermitian_lambda_max(const std::vector<cplx>& H, int s);
-bool radix_plan(int n, RadixPlan& pl, int variant);
+// Largest last radix of the portrait length's schedule: the run-time
+// drive-axis passes keep the s aliases of a butterfly in registers (s R <= 24
+// complex values; 0: any, those passes do not run).
+inline int xpass_max_last(int s) { return s == 1 ? 16 : (s == 2 ? 12 : (s == 3 ? 8 : (s == 4 ? 6 : 0))); }
+// max_last: largest radix of the schedule's last stage (0: any)
+bool radix_plan(int n, RadixPlan& pl, int max_last = 0);
 
 // ops.cu: operator launches (all asynchronous on `st`)
 struct OpCtx;

@@ -135,8 +135,8 @@ extern "C" mh3d_status mh3d_forward_noalloc(const mh3d_geometry* g, const float*
     P.ay.n = ny;
     P.az.n = nz;
     P.am.n = mx;
-    if (!radix_plan(nx, P.ax.rp, 0) || !radix_plan(ny, P.ay.rp, 0) || !radix_plan(nz, P.az.rp, 0) ||
-        !radix_plan(mx, P.am.rp, 0))
+    if (!radix_plan(nx, P.ax.rp) || !radix_plan(ny, P.ay.rp) || !radix_plan(nz, P.az.rp) ||
+        !radix_plan(mx, P.am.rp, xpass_max_last(P.s)))
         return MH3D_ERR_UNSUPPORTED_SIZE;
     // launch shape: the same shared-memory budget rule as planned operators
     const size_t budget = 200 * 1024;

@@ -24,40 +24,104 @@
 //   X normal: the drive-axis part of A^T A, sum_k X_k^T P^T P X_k, which in
 //     the Fourier domain couples only the s aliases of each frequency:
 //     an s x s block per alias class, precomputed in FP64.
+#include <algorithm>
+#include <cstdint>
 #include <cstdio>
 
 #include "ops_kernels.cuh"
 #include "ops_functors.cuh"
+#include "ops_xrt.cuh"
 
 namespace mh3d {
 
-__global__ void __launch_bounds__(256) k_tpass(const TArgs a)
+// The T pass of any length.  What bounds it: latency -- a CTA's load,
+// transform and store run in turn -- so the first stage reads its operands
+// from global memory straight into registers (its radix in flight per
+// thread), the last stage writes from registers, the spectral product sits
+// between the last forward and first inverse stage, and a length of two
+// radices (up to 144, most up to 256) crosses shared memory twice, with two
+// barriers and one butterfly per thread and stage.  Against the former
+// kernel (radices 2, 3, 4, 8; up to ten stages and barriers, run-time
+// divisions per butterfly): 162 x 108 x 81, a y pass 29 us before.
+template <int MODE, bool EPI>
+__global__ void __launch_bounds__(256, 2) k_tpass(const __grid_constant__ TArgs a)
 {
     extern __shared__ float2 sm[];
     __shared__ double red[34];
     __shared__ float cgs[3];
     float beta = 0.f, alpha = 0.f;
     if (a.cg.flags && !cg_enter_cta(a.cg, a.pupdate != 0, &beta, &alpha, cgs)) return;
-    const int n = a.n, P = a.cols / 2, ld = P + 1;
+    const int n = a.n, P = a.cols / 2, lgP = 31 - __clz(P), nst = a.rp.nst;
     float2* tw = sm;
     float2* mu = tw + n;
     float2* s0 = mu + n;
-    float2* s1 = s0 + n * ld;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        tw[i] = a.tw[i];
-        mu[i] = a.mult[i];
-    }
-    __syncthreads();
+    float2* s1 = s0 + n * P;
+    cp_table(tw, a.tw, n);
+    cp_table(mu, a.mult, n);
     const int x0 = blockIdx.x * a.cols;
-    const long long base = (long long)blockIdx.y * a.os;
-    const int res = fft_result_index(a.rp.nst);
-    float2* sr = res ? s1 : s0;
-    float2* so = res ? s0 : s1;
+    const int base = (int)((long long)blockIdx.y * a.os);
     DotAcc acc, acc2;
-    fft_run<false, true, true>(a.rp, TLoad{&a, base, x0, beta, alpha}, BufSt{sr, ld}, s0, s1, ld, P, tw);
-    fft_run<true, true, true>(a.rp, MulLd{sr, ld, mu}, TStore{&a, base, x0, &acc, a.part2 ? &acc2 : nullptr}, so,
-                              sr, ld, P, tw);
-    if (a.epilogue && a.part) {
+    const TLoad ld{&a, base, x0};
+    const TStore st{&a, base, x0};
+    float2* src = s0;
+    float2* dst = s1;
+    auto flip = [&]() {
+        float2* t = src;
+        src = dst;
+        dst = t;
+    };
+    if constexpr (MODE != 0) {
+        t_update<MODE>(a, base, x0, lgP, beta, alpha, s1);
+        cp_table_wait();
+        __syncthreads();
+    }
+    if (nst < 2) {
+        // one butterfly is the whole convolution (length 1: a product)
+        if constexpr (MODE == 0) {
+            cp_table_wait();
+            __syncthreads();
+        }
+        if (nst == 0) {
+            for (int p = threadIdx.x; p < P; p += blockDim.x) {
+                const float2 v = c_mul(MODE != 0 ? s1[p] : ld.at(p)(0), mu[0]);
+                if constexpr (EPI) s0[p] = v;
+                else st.at(p)(0, v);
+            }
+        } else if constexpr (EPI) {
+            rt_conv_any(ld, BufSt{s0, P}, mu, stage_fwd(a.rp, 0), lgP, tw);
+        } else if constexpr (MODE != 0) {
+            rt_conv_any(BufLd{s1, P}, st, mu, stage_fwd(a.rp, 0), lgP, tw);
+        } else {
+            rt_conv_any(ld, st, mu, stage_fwd(a.rp, 0), lgP, tw);
+        }
+    } else {
+        if constexpr (MODE != 0) {
+            rt_stage_buf<false>(s1, s0, P, stage_fwd(a.rp, 0), lgP, tw);
+        } else {
+            rt_stage_any<false, true>(ld, BufSt{s0, P}, stage_fwd(a.rp, 0), lgP, tw);
+            cp_table_wait();
+        }
+        __syncthreads();
+        for (int s = 1; s < nst - 1; ++s, flip()) {
+            rt_stage_buf<false>(src, dst, P, stage_fwd(a.rp, s), lgP, tw);
+            __syncthreads();
+        }
+        rt_conv_any(BufLd{src, P}, BufSt{dst, P}, mu, stage_fwd(a.rp, nst - 1), lgP, tw);
+        __syncthreads();
+        for (int s = 1; s < nst - 1; ++s) {
+            flip();
+            rt_stage_buf<true>(src, dst, P, stage_rev(a.rp, s), lgP, tw);
+            __syncthreads();
+        }
+        flip();
+        if constexpr (EPI) rt_stage_buf<true>(src, dst, P, stage_rev(a.rp, nst - 1), lgP, tw);
+        else rt_stage_any<true, true>(BufLd{src, P}, st, stage_rev(a.rp, nst - 1), lgP, tw);
+    }
+    if constexpr (EPI) {
+        __syncthreads();
+        t_epilogue(a, base, x0, lgP, nst < 2 ? s0 : dst, &acc, a.part2 ? &acc2 : nullptr);
+    }
+    if (EPI && a.part) {
         const int bid = blockIdx.y * gridDim.x + blockIdx.x, nb = gridDim.x * gridDim.y;
         float2 t, t2;
         block_pair_acc2(acc, a.part2 ? &acc2 : nullptr, reinterpret_cast<float*>(red), &t, &t2);
@@ -73,96 +137,120 @@ cudaError_t run_tpass(const TArgs& a, int nouter, cudaStream_t st)
 {
     if (ct_tpass_available(a)) return run_tpass_ct(a, nouter, st);
     dim3 grid((a.nx + a.cols - 1) / a.cols, nouter);
-    const size_t smem = tpass_smem_bytes(a.n, a.cols);
-    k_tpass<<<grid, 256, smem, st>>>(a);
+    const int P = a.cols / 2;
+    const size_t smem = sizeof(float2) * (size_t)(2 * a.n + 2 * a.n * P);
+    const int T = std::min(256, std::max(64, round32(max_nb(a.rp) * P)));
+    if (a.epilogue) k_tpass<0, true><<<grid, T, smem, st>>>(a);
+    else if (a.pupdate == 2) k_tpass<2, false><<<grid, T, smem, st>>>(a);
+    else if (a.pupdate) k_tpass<1, false><<<grid, T, smem, st>>>(a);
+    else k_tpass<0, false><<<grid, T, smem, st>>>(a);
     return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
-// X pass kernels
+// X pass kernels (s = 1..4: ops_xrt.cuh)
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_xfwd(const XArgs a)
+// Any s and any length (one included), one harmonic at a time: the aliases
+// folded, or the harmonics summed, in shared memory.
+__global__ void __launch_bounds__(256) k_xfwd(const __grid_constant__ XArgs a)
 {
     extern __shared__ float2 sm[];
-    const int nx = a.nx, mx = a.mx, P = a.pairs, ldA = P + 1;
-    const int PB = a.kg * P, ldB = PB + 1;
+    const int nx = a.nx, mx = a.mx, P = 1 << a.lgP, ld = P + 1;
     float2* twx = sm;
     float2* twm = twx + nx;
     float2* A0 = twm + mx;
-    float2* A1 = A0 + nx * ldA;
-    float2* B0 = A1 + nx * ldA;
-    float2* B1 = B0 + mx * ldB;
+    float2* A1 = A0 + nx * ld;
+    float2* B0 = A1 + nx * ld;
+    float2* B1 = B0 + mx * ld;
     for (int i = threadIdx.x; i < nx; i += blockDim.x) twx[i] = a.twx[i];
     for (int i = threadIdx.x; i < mx; i += blockDim.x) twm[i] = a.twm[i];
     __syncthreads();
     const int row0 = blockIdx.x * 2 * P;
     const int res = fft_result_index(a.rpx.nst);
     float2* Ar = res ? A1 : A0;
-    fft_run<false, false, true>(a.rpx, RowPairLd{a.vin, nx, row0, a.rows}, BufSt{Ar, ldA}, A0, A1, ldA, P, twx);
-    for (int k0 = 0; k0 < a.K; k0 += a.kg) {
-        const int kn = min(a.kg, a.K - k0);
-        fft_run<true, true, false>(a.rpm, FoldLd{Ar, ldA, a.Xhat + (long long)k0 * nx, nx, mx, a.s, P},
-                                   PortraitSt{a.dout + (long long)k0 * a.M, a.phase + k0, a.M, mx, row0, a.rows, P},
-                                   B0, B1, ldB, kn * P, twm);
-    }
+    fft_run<false, false, true>(a.rpx, RowPairLd{a.vin, nx, row0, a.rows}, BufSt{Ar, ld}, A0, A1, ld, P, twx);
+    for (int k = 0; k < a.K; ++k)
+        fft_run<true, true, false>(a.rpm, FoldLd{Ar, ld, a.Xhat + (long long)k * nx, mx, a.s},
+                                   PortraitSt{a.dout + (long long)k * a.M, __ldg(a.phase + k),
+                                              PortraitRows{row0, a.rows, mx, a.win}},
+                                   B0, B1, ld, P, twm);
 }
 
-__global__ void __launch_bounds__(256) k_xadj(const XArgs a)
+__global__ void __launch_bounds__(256) k_xadj(const __grid_constant__ XArgs a)
 {
     extern __shared__ float2 sm[];
-    const int nx = a.nx, mx = a.mx, P = a.pairs, ldA = P + 1;
-    const int PB = a.kg * P, ldB = PB + 1;
+    const int nx = a.nx, mx = a.mx, P = 1 << a.lgP, ld = P + 1;
     float2* twx = sm;
     float2* twm = twx + nx;
-    float2* acc = twm + mx;            // [nx][ldA]
-    float2* S0 = acc + nx * ldA;       // scratch region (max of both uses)
-    float2* B1 = S0 + mx * ldB;
-    float2* S1 = S0 + nx * ldA;
+    float2* acc = twm + mx;            // [nx][ld]
+    float2* S0 = acc + nx * ld;        // two buffers of nx ld (the transforms of mx use their starts)
+    float2* S1 = S0 + nx * ld;
     for (int i = threadIdx.x; i < nx; i += blockDim.x) twx[i] = a.twx[i];
     for (int i = threadIdx.x; i < mx; i += blockDim.x) twm[i] = a.twm[i];
     __syncthreads();
     const int row0 = blockIdx.x * 2 * P;
-    const int resm = fft_result_index(a.rpm.nst);
-    float2* Fr = resm ? B1 : S0;
-    for (int k0 = 0; k0 < a.K; k0 += a.kg) {
-        const int kn = min(a.kg, a.K - k0);
+    float2* Fr = fft_result_index(a.rpm.nst) ? S1 : S0;
+    for (int k = 0; k < a.K; ++k) {
         fft_run<false, false, true>(a.rpm,
-                                    PortraitLd{a.din + (long long)k0 * a.M, a.phase + k0, a.M, mx, row0, a.rows, P},
-                                    BufSt{Fr, ldB}, S0, B1, ldB, kn * P, twm);
-        // acc[w][p] (+)= sum_kk conj(Xhat_k[w]) F_kk[w mod mx][p]
+                                    PortraitKLd{a.din + (long long)k * a.M, __ldg(a.phase + k),
+                                                PortraitRows{row0, a.rows, mx, a.win}},
+                                    BufSt{Fr, ld}, S0, S1, ld, P, twm);
+        // acc[w][p] (+)= conj(Xhat_k[w]) F[w mod mx][p]
         for (int idx = threadIdx.x; idx < nx * P; idx += blockDim.x) {
-            const int p = idx % P, w = idx / P;
+            const int p = idx & (P - 1), w = idx >> a.lgP;
             const int m = w % mx;
-            float2 v = (k0 == 0) ? make_float2(0.f, 0.f) : acc[w * ldA + p];
-            for (int kk = 0; kk < kn; ++kk)
-                v = c_add(v, c_mulc(Fr[m * ldB + kk * P + p], __ldg(a.Xhat + (long long)(k0 + kk) * nx + w)));
-            acc[w * ldA + p] = v;
+            const float2 v = c_mulc(Fr[m * ld + p], __ldg(a.Xhat + (long long)k * nx + w));
+            acc[w * ld + p] = (k == 0) ? v : c_add(acc[w * ld + p], v);
         }
         __syncthreads();
     }
-    fft_run<true, true, false>(a.rpx, BufLd{acc, ldA}, RowPairSt{a.vout, nx, row0, a.rows}, S0, S1, ldA, P, twx);
+    fft_run<true, true, false>(a.rpx, BufLd{acc, ld}, RowPairSt{a.vout, nx, row0, a.rows}, S0, S1, ld, P, twx);
 }
 
-__global__ void __launch_bounds__(256) k_xnrm(const XArgs a)
+__global__ void __launch_bounds__(256) k_xnrm(const __grid_constant__ XArgs a)
 {
     extern __shared__ float2 sm[];
     __shared__ double red[34];
     float dummy;
     if (a.cg_active && !cg_enter(a.cg, false, &dummy, red)) return;
-    const int nx = a.nx, P = a.pairs, ldA = P + 1;
+    const int nx = a.nx, lgP = a.lgP, P = 1 << lgP, ld = P + 1, nst = a.rpx.nst;
     float2* twx = sm;
     float2* A0 = twx + nx;
-    float2* A1 = A0 + nx * ldA;
-    for (int i = threadIdx.x; i < nx; i += blockDim.x) twx[i] = a.twx[i];
-    __syncthreads();
+    float2* A1 = A0 + nx * ld;
+    cp_table(twx, a.twx, nx);
     const int row0 = blockIdx.x * 2 * P;
-    const int res = fft_result_index(a.rpx.nst);
-    float2* Ar = res ? A1 : A0;
-    float2* Ao = res ? A0 : A1;
     DotAcc dacc, dacc2;
-    fft_run<false, false, true>(a.rpx, RowPairLd{a.vin, nx, row0, a.rows}, BufSt{Ar, ldA}, A0, A1, ldA, P, twx);
-    fft_run<true, true, false>(a.rpx, QLd{Ar, ldA, a.Q, a.mx, a.s},
-                               NrmEpiSt{&a, row0, &dacc, a.part2 ? &dacc2 : nullptr}, Ao, Ar, ldA, P, twx);
+    const RowPairLd rows{a.vin, nx, row0, a.rows};
+    float2* src = A0;
+    float2* dst = A1;
+    auto flip = [&]() {
+        float2* t = src;
+        src = dst;
+        dst = t;
+    };
+    if (nst == 0) {
+        for (int p = threadIdx.x; p < P; p += blockDim.x) A0[p] = rows.at(p)(0);
+        __syncthreads();
+        for (int p = threadIdx.x; p < P; p += blockDim.x) A1[p] = QLd{A0, ld, a.Q, a.mx, a.s, a.dmx}.at(p)(0);
+        cp_table_wait();
+    } else {
+        rt_stage_any<false, false>(rows, BufSt{A0, ld}, stage_fwd(a.rpx, 0), lgP, twx);
+        cp_table_wait();
+        __syncthreads();
+        for (int s = 1; s < nst; ++s, flip()) {
+            rt_stage_buf<false>(src, dst, ld, stage_fwd(a.rpx, s), lgP, twx);
+            __syncthreads();
+        }
+        // the alias blocks on the first inverse stage's loads
+        rt_stage_any<true, true>(QLd{src, ld, a.Q, a.mx, a.s, a.dmx}, BufSt{dst, ld}, stage_rev(a.rpx, 0), lgP, twx);
+        for (int s = 1; s < nst; ++s) {
+            __syncthreads();
+            flip();
+            rt_stage_buf<true>(src, dst, ld, stage_rev(a.rpx, s), lgP, twx);
+        }
+    }
+    __syncthreads();
+    nrm_epilogue_rt(a, row0, P, dst, ld, &dacc, a.part2 ? &dacc2 : nullptr);
     if (a.part) {
         float2 t, t2;
         block_pair_acc2(dacc, a.part2 ? &dacc2 : nullptr, reinterpret_cast<float*>(red), &t, &t2);
@@ -174,22 +262,124 @@ __global__ void __launch_bounds__(256) k_xnrm(const XArgs a)
 
 int xpass_blocks(int rows, int pairs) { return (rows + 2 * pairs - 1) / (2 * pairs); }
 
-cudaError_t run_xfwd(const XArgs& a, cudaStream_t st)
+namespace {
+
+constexpr size_t kXSmemMax = 200 * 1024;
+
+// Launch shape of the run-time forward and adjoint: 8 row pairs (16 left
+// 144 x 144 x 72 with 324 CTAs, two an SM: a second wave nearly empty), fewer
+// where they leave SMs without a CTA; then as many harmonics a round (1, 2
+// or 4: the adjoint adds their sums one after another) as 256 threads hold, one thread per (harmonic, butterfly,
+// pair), while two CTAs fit an SM's shared memory.
+struct XShape {
+    int lgP = 3, lgK = 0, threads = 0, pitch = 0;
+    size_t smem = 0;
+    bool ok = false;
+};
+XShape x_rt_shape(const RadixPlan& rpx, const RadixPlan& rpm, int s, int K, int rows, bool adj)
 {
-    if (ct_xpass_available(a.nx, a.s, a.pairs)) return run_xfwd_ct(a, st);
-    k_xfwd<<<xpass_blocks(a.rows, a.pairs), 256, xfwd_smem_bytes(a.nx, a.mx, a.pairs, a.kg), st>>>(a);
+    XShape h;
+    if (s < 1 || s > 4 || rpx.nst < 1 || rpm.nst < 1 || rpm.nst > 3) return h;
+    const int nx = rpx.n, mx = rpm.n, R = rpm.radix[rpm.nst - 1], NB = mx / R;
+    if (s * R > kXRegs) return h;
+    // the adjoint's staged rows: an odd pitch spreads a half-warp's rows over the banks
+    h.pitch = mx | 1;
+    auto smem = [&](int lgP, int lgK) {
+        const size_t P = (size_t)1 << lgP, KG = (size_t)1 << lgK, a = 2 * (size_t)nx * (P + 1);
+        const size_t b = 2 * (size_t)mx * (KG * P + 1) + (adj ? 2 * KG * 2 * P * h.pitch : 0);
+        return sizeof(float2) * (nx + mx + (adj ? 2 : 3) * KG * nx + std::max(a, b));
+    };
+    while (h.lgP > 1 && xpass_blocks(rows, 1 << h.lgP) < 152) --h.lgP;
+    while (h.lgP > 0 && ((NB << h.lgP) > 256 || smem(h.lgP, 0) > kXSmemMax)) --h.lgP;
+    if ((NB << h.lgP) > 256 || smem(h.lgP, 0) > kXSmemMax) return h;
+    while (h.lgK < 2 && (1 << h.lgK) < K && (NB << (h.lgP + h.lgK + 1)) <= 256 && smem(h.lgP, h.lgK + 1) <= kXSmemMax / 2) ++h.lgK;
+    const int want = std::max(std::max(max_nb(rpx) << h.lgP, max_nb(rpm) << (h.lgP + h.lgK)), NB << (h.lgP + h.lgK));
+    h.threads = std::min(256, std::max(64, round32(want)));
+    h.smem = smem(h.lgP, h.lgK);
+    h.ok = true;
+    return h;
+}
+
+// Row pairs of the any-s kernels: as many as fit, at most 16.
+int x_any_lgP(size_t per_pair, size_t fixed)
+{
+    int lgP = 4;
+    while (lgP > 0 && fixed + per_pair * ((1 << lgP) + 1) > kXSmemMax) --lgP;
+    return lgP;
+}
+
+template <class F>
+cudaError_t launch_x(F* f, XArgs& a, int lgP, int threads, size_t smem, cudaStream_t st)
+{
+    a.lgP = lgP;
+    f<<<xpass_blocks(a.rows, 1 << lgP), threads, smem, st>>>(a);
     return cudaGetLastError();
 }
-cudaError_t run_xadj(const XArgs& a, cudaStream_t st)
+
+}  // namespace
+
+bool xpass_windowed(int nx, int mx, int s, int pairs)
 {
-    if (ct_xpass_available(a.nx, a.s, a.pairs)) return run_xadj_ct(a, st);
-    k_xadj<<<xpass_blocks(a.rows, a.pairs), 256, xadj_smem_bytes(a.nx, a.mx, a.pairs, a.kg), st>>>(a);
-    return cudaGetLastError();
+    (void)mx;
+    return !ct_xpass_available(nx, s, pairs);
 }
-cudaError_t run_xnrm(const XArgs& a, cudaStream_t st)
+
+int xnrm_rt_pairs(const RadixPlan& rpx)
 {
-    if (ct_xpass_available(a.nx, a.s, a.pairs)) return run_xnrm_ct(a, st);
-    k_xnrm<<<xpass_blocks(a.rows, a.pairs), 256, xnrm_smem_bytes(a.nx, a.pairs), st>>>(a);
+    int lgP = 4;
+    while (lgP > 0 && ((rpx.n / (rpx.nst ? rpx.radix[0] : 1)) << lgP > 256 ||
+                       sizeof(float2) * (size_t)(rpx.n + 2 * rpx.n * ((1 << lgP) + 1)) > kXSmemMax))
+        --lgP;
+    return 1 << lgP;
+}
+
+cudaError_t run_xfwd(const XArgs& a0, cudaStream_t st)
+{
+    if (!a0.win.on && ct_xpass_available(a0.nx, a0.s, a0.pairs)) return run_xfwd_ct(a0, st);
+    XArgs a = a0;
+    const XShape h = x_rt_shape(a.rpx, a.rpm, a.s, a.K, a.rows, false);
+    if (h.ok) {
+        a.lgP = h.lgP;
+        a.lgK = h.lgK;
+        const int grid = xpass_blocks(a.rows, 1 << h.lgP);
+        if (a.s == 1) return XRt<1>::fwd(a, grid, h.threads, h.smem, st);
+        if (a.s == 2) return XRt<2>::fwd(a, grid, h.threads, h.smem, st);
+        if (a.s == 3) return XRt<3>::fwd(a, grid, h.threads, h.smem, st);
+        return XRt<4>::fwd(a, grid, h.threads, h.smem, st);
+    }
+    const size_t per = sizeof(float2) * 2 * ((size_t)a.nx + a.mx), fixed = sizeof(float2) * ((size_t)a.nx + a.mx);
+    const int lgP = x_any_lgP(per, fixed);
+    return launch_x(k_xfwd, a, lgP, 256, fixed + per * ((1 << lgP) + 1), st);
+}
+cudaError_t run_xadj(const XArgs& a0, cudaStream_t st)
+{
+    if (!a0.win.on && ct_xpass_available(a0.nx, a0.s, a0.pairs)) return run_xadj_ct(a0, st);
+    XArgs a = a0;
+    const XShape h = x_rt_shape(a.rpx, a.rpm, a.s, a.K, a.rows, true);
+    a.pitch = h.pitch;
+    if (h.ok) {
+        a.lgP = h.lgP;
+        a.lgK = h.lgK;
+        const int grid = xpass_blocks(a.rows, 1 << h.lgP);
+        if (a.s == 1) return XRt<1>::adj(a, grid, h.threads, h.smem, st);
+        if (a.s == 2) return XRt<2>::adj(a, grid, h.threads, h.smem, st);
+        if (a.s == 3) return XRt<3>::adj(a, grid, h.threads, h.smem, st);
+        return XRt<4>::adj(a, grid, h.threads, h.smem, st);
+    }
+    const size_t per = sizeof(float2) * 3 * (size_t)a.nx, fixed = sizeof(float2) * ((size_t)a.nx + a.mx);
+    const int lgP = x_any_lgP(per, fixed);
+    return launch_x(k_xadj, a, lgP, 256, fixed + per * ((1 << lgP) + 1), st);
+}
+cudaError_t run_xnrm(const XArgs& a0, cudaStream_t st)
+{
+    if (ct_xpass_available(a0.nx, a0.s, a0.pairs)) return run_xnrm_ct(a0, st);
+    XArgs a = a0;
+    a.dmx = FastDiv(a.mx);
+    const int P = xnrm_rt_pairs(a.rpx);
+    a.lgP = 0;
+    while ((1 << a.lgP) < P) ++a.lgP;
+    const size_t smem = sizeof(float2) * (size_t)(a.nx + 2 * a.nx * (P + 1));
+    k_xnrm<<<xpass_blocks(a.rows, P), std::min(256, std::max(64, round32(max_nb(a.rpx) * P))), smem, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -210,8 +400,15 @@ cudaError_t ops_set_attributes()
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e != cudaSuccess) return e;
-    if ((e = opt_in_smem(k_tpass, optin)) != cudaSuccess) return e;
+    if ((e = opt_in_smem(k_tpass<0, false>, optin)) != cudaSuccess) return e;
+    if ((e = opt_in_smem(k_tpass<0, true>, optin)) != cudaSuccess) return e;
+    if ((e = opt_in_smem(k_tpass<1, false>, optin)) != cudaSuccess) return e;
+    if ((e = opt_in_smem(k_tpass<2, false>, optin)) != cudaSuccess) return e;
     if ((e = opt_in_smem(k_xfwd, optin)) != cudaSuccess) return e;
+    if ((e = XRt<1>::set_attributes(optin)) != cudaSuccess) return e;
+    if ((e = XRt<2>::set_attributes(optin)) != cudaSuccess) return e;
+    if ((e = XRt<3>::set_attributes(optin)) != cudaSuccess) return e;
+    if ((e = XRt<4>::set_attributes(optin)) != cudaSuccess) return e;
     if ((e = opt_in_smem(k_xadj, optin)) != cudaSuccess) return e;
     if ((e = opt_in_smem(k_xnrm, optin)) != cudaSuccess) return e;
     if ((e = xw_set_attributes()) != cudaSuccess) return e;

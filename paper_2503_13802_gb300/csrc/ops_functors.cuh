@@ -179,93 +179,194 @@ __device__ __forceinline__ void cg_count_iteration(const CgCtl& c)
 // ---------------------------------------------------------------------------
 // T pass
 // ---------------------------------------------------------------------------
+// Column pair p of a tile (run-time kernels).  nx even: columns x0 + 2p and
+// x0 + 2p + 1, one 8-byte access; nx odd (rows not 8-byte aligned): columns
+// x0 + p and x0 + p + P, so that consecutive lanes take consecutive columns
+// of either access.
+struct TCols {
+    int x, second;       // first column, distance to the second
+    bool has1, has2;
+    __device__ __forceinline__ TCols(const TArgs& a, int x0, int p)
+    {
+        second = a.vec2 ? 1 : a.cols / 2;
+        x = x0 + (a.vec2 ? 2 * p : p);
+        has1 = x < a.nx;
+        has2 = x + second < a.nx;
+    }
+    __device__ __forceinline__ float2 ld(const float* __restrict__ p, int i, int vec2) const
+    {
+        if (vec2) return *reinterpret_cast<const float2*>(p + i);
+        return make_float2(p[i], has2 ? p[i + second] : 0.f);
+    }
+    __device__ __forceinline__ void st(float* __restrict__ p, int i, int vec2, float2 v) const
+    {
+        if (vec2) {
+            *reinterpret_cast<float2*>(p + i) = v;
+        } else {
+            p[i] = v.x;
+            if (has2) p[i + second] = v.y;
+        }
+    }
+};
+
+// Tile loader of a plain pass (in, times b).
 struct TLoad {
     const TArgs* a;
-    long long base;
+    int base;            // voxel index of element 0, column 0 (grids hold at most 2^30 voxels)
     int x0;
-    float beta;
-    float alpha = 0.f;
-    __device__ __forceinline__ float2 operator()(int e, int p) const
+    struct At {
+        const TArgs* a;
+        TCols c;
+        int base, es;
+        __device__ __forceinline__ float2 operator()(int e) const
+        {
+            if (!c.has1) return make_float2(0.f, 0.f);
+            const int i = base + e * es, w = a->vec2;
+            float2 v = c.ld(a->in, i, w);
+            if (a->bin) {
+                const float2 bb = c.ld(a->bin, i, w);
+                v.x *= bb.x;
+                v.y *= bb.y;
+            }
+            return v;
+        }
+    };
+    __device__ __forceinline__ At at(int p) const
     {
-        const int x = x0 + 2 * p;
-        if (x >= a->nx) return make_float2(0.f, 0.f);
-        const long long i = base + (long long)e * a->es + x;
-        const bool has2 = x + 1 < a->nx;
-        float2 v;
-        if (a->pupdate == 2) {
-            const float2 rr = ld2(a->rvec, i, has2, a->vec2);
-            const float2 ss = ld2(a->svec, i, has2, a->vec2);
-            const float2 pp = ld2(a->pvec, i, has2, a->vec2);
-            const float2 qq = ld2(a->qdir, i, has2, a->vec2);
-            const float2 xx = ld2(a->xvec, i, has2, a->vec2);
-            const float2 pn = make_float2(fmaf(beta, pp.x, rr.x), fmaf(beta, pp.y, rr.y));
-            const float2 qn = make_float2(fmaf(beta, qq.x, ss.x), fmaf(beta, qq.y, ss.y));
-            st2(a->pvec, i, has2, a->vec2, pn);
-            st2(a->qdir, i, has2, a->vec2, qn);
-            st2(a->xvec, i, has2, a->vec2, make_float2(fmaf(alpha, pn.x, xx.x), fmaf(alpha, pn.y, xx.y)));
-            v = make_float2(fmaf(-alpha, qn.x, rr.x), fmaf(-alpha, qn.y, rr.y));
-            st2(a->rvec_w, i, has2, a->vec2, v);
-        } else if (a->pupdate) {
-            const float2 rr = ld2(a->rvec, i, has2, a->vec2);
-            const float2 pp = ld2(a->pvec, i, has2, a->vec2);
-            v = make_float2(fmaf(beta, pp.x, rr.x), fmaf(beta, pp.y, rr.y));
-            st2(a->pvec, i, has2, a->vec2, v);
-        } else {
-            v = ld2(a->in, i, has2, a->vec2);
-        }
-        if (a->bin) {
-            const float2 bb = ld2(a->bin, i, has2, a->vec2);
-            v.x *= bb.x;
-            v.y *= bb.y;
-        }
-        return v;
+        const TCols c(*a, x0, p);
+        return At{a, c, base + c.x, (int)a->es};
     }
 };
 
-struct MulLd {
-    const float2* b;
-    int ld;
-    const float2* mu;
-    __device__ __forceinline__ float2 operator()(int e, int p) const { return c_mul(b[e * ld + p], mu[e]); }
-};
+// The CG vector updates of a tile (TArgs.pupdate: MODE 1 p = r + beta p, 2
+// the single-reduction form), the first stage's input into buf [n][P].  Four
+// elements a step with every load before the stores, so that a thread keeps
+// up to 24 loads in flight.
+template <int MODE>
+__device__ __forceinline__ void t_update(const TArgs& a, int base, int x0, int lgP, float beta, float alpha, float2* buf)
+{
+    constexpr int U = 4;
+    const int w = a.vec2, de = (int)blockDim.x >> lgP, n = a.n;   // a thread keeps its column pair
+    const TCols c(a, x0, (int)threadIdx.x & ((1 << lgP) - 1));
+    const int es = (int)a.es, b0 = base + c.x;
+    for (int e0 = (int)threadIdx.x >> lgP; e0 < n; e0 += U * de) {
+        float2 rr[U], ss[U], pp[U], qq[U], xx[U], bb[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int e = e0 + u * de, i = b0 + e * es;
+            if (e >= n || !c.has1) continue;
+            rr[u] = c.ld(a.rvec, i, w);
+            pp[u] = c.ld(a.pvec, i, w);
+            if constexpr (MODE == 2) {
+                ss[u] = c.ld(a.svec, i, w);
+                qq[u] = c.ld(a.qdir, i, w);
+                xx[u] = c.ld(a.xvec, i, w);
+            }
+            bb[u] = a.bin ? c.ld(a.bin, i, w) : make_float2(1.f, 1.f);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int e = e0 + u * de, i = b0 + e * es;
+            if (e >= n) continue;
+            float2 v = make_float2(0.f, 0.f);
+            if (c.has1) {
+                const float2 pn = make_float2(fmaf(beta, pp[u].x, rr[u].x), fmaf(beta, pp[u].y, rr[u].y));
+                c.st(a.pvec, i, w, pn);
+                v = pn;
+                if constexpr (MODE == 2) {
+                    const float2 qn = make_float2(fmaf(beta, qq[u].x, ss[u].x), fmaf(beta, qq[u].y, ss[u].y));
+                    c.st(a.qdir, i, w, qn);
+                    c.st(a.xvec, i, w, make_float2(fmaf(alpha, pn.x, xx[u].x), fmaf(alpha, pn.y, xx[u].y)));
+                    v = make_float2(fmaf(-alpha, qn.x, rr[u].x), fmaf(-alpha, qn.y, rr[u].y));
+                    c.st(a.rvec_w, i, w, v);
+                }
+                if (a.bin) {
+                    v.x *= bb[u].x;
+                    v.y *= bb[u].y;
+                }
+            }
+            buf[(e << lgP) + ((int)threadIdx.x & ((1 << lgP) - 1))] = v;
+        }
+    }
+}
 
+// Tile storer of a plain pass (times b).
 struct TStore {
     const TArgs* a;
-    long long base;
+    int base;
     int x0;
-    DotAcc* acc;
-    DotAcc* acc2 = nullptr;   // input . input (single-reduction CG)
-    __device__ __forceinline__ void operator()(int e, int p, float2 v) const
-    {
-        const int x = x0 + 2 * p;
-        if (x >= a->nx) return;
-        const long long i = base + (long long)e * a->es + x;
-        const bool has2 = x + 1 < a->nx;
-        if (a->bout) {
-            const float2 bb = ld2(a->bout, i, has2, a->vec2);
-            v.x *= bb.x;
-            v.y *= bb.y;
-        }
-        if (a->epilogue) {
-            const RegArgs& g = a->reg;
-            const long long sz = (long long)g.nx * g.ny;
-            const int z = (int)(i / sz), y = (int)((i - (long long)z * sz) / g.nx);
-            v.x += reg_term(g, a->pin, i, x, y, z);
-            if (has2) v.y += reg_term(g, a->pin, i + 1, x + 1, y, z);
-            st2(a->qvec, i, has2, a->vec2, v);
-            const float p0 = a->pin[i];
-            acc->add(p0, v.x);
-            if (acc2) acc2->add(p0, p0);
-            if (has2) {
-                const float p1 = a->pin[i + 1];
-                acc->add(p1, v.y);
-                if (acc2) acc2->add(p1, p1);
+    struct At {
+        const TArgs* a;
+        TCols c;
+        int base, es;
+        __device__ __forceinline__ void operator()(int e, float2 v) const
+        {
+            if (!c.has1) return;
+            const int i = base + e * es, w = a->vec2;
+            if (a->bout) {
+                const float2 bb = c.ld(a->bout, i, w);
+                v.x *= bb.x;
+                v.y *= bb.y;
             }
-        } else {
-            st2(a->out, i, has2, a->vec2, v);
+            c.st(a->out, i, w, v);
         }
+    };
+    __device__ __forceinline__ At at(int p) const
+    {
+        const TCols c(*a, x0, p);
+        return At{a, c, base + c.x, (int)a->es};
     }
 };
+
+// The explicit normal operator's epilogue over a transformed tile buf [n][P]:
+// q = b w + lambda R p, with p^T q (and p^T p for acc2); four elements a step
+// with the loads of R = I first.
+__device__ __forceinline__ void t_epilogue(const TArgs& a, int base, int x0, int lgP, const float2* buf, DotAcc* acc,
+                                           DotAcc* acc2)
+{
+    constexpr int U = 4;
+    const int w = a.vec2, de = (int)blockDim.x >> lgP, n = a.n;   // a thread keeps its column pair
+    const int p = (int)threadIdx.x & ((1 << lgP) - 1);
+    const TCols c(a, x0, p);
+    if (!c.has1) return;
+    const int es = (int)a.es, b0 = base + c.x;
+    const bool plain = a.reg.kind == 0;
+    for (int e0 = (int)threadIdx.x >> lgP; e0 < n; e0 += U * de) {
+        float2 pp[U], bb[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int e = e0 + u * de, i = b0 + e * es;
+            if (e >= n) continue;
+            pp[u] = c.ld(a.pin, i, w);
+            bb[u] = a.bout ? c.ld(a.bout, i, w) : make_float2(1.f, 1.f);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int e = e0 + u * de, i = b0 + e * es;
+            if (e >= n) continue;
+            float2 v = buf[(e << lgP) + p];
+            if (a.bout) {
+                v.x *= bb[u].x;
+                v.y *= bb[u].y;
+            }
+            if (plain) {
+                v.x += a.reg.lambda * pp[u].x;
+                v.y += a.reg.lambda * pp[u].y;
+            } else {
+                const int y = a.axis == 1 ? e : (int)blockIdx.y, z = a.axis == 1 ? (int)blockIdx.y : e;
+                v.x += reg_term(a.reg, a.pin, i, c.x, y, z);
+                if (c.has2) v.y += reg_term(a.reg, a.pin, i + c.second, c.x + c.second, y, z);
+            }
+            c.st(a.qvec, i, w, v);
+            acc->add(pp[u].x, v.x);
+            if (acc2) acc2->add(pp[u].x, pp[u].x);
+            if (c.has2) {
+                acc->add(pp[u].y, v.y);
+                if (acc2) acc2->add(pp[u].y, pp[u].y);
+            }
+        }
+    }
+}
 
 // ---------------------------------------------------------------------------
 // X pass: loaders and storers
@@ -282,6 +383,20 @@ struct RowPairLd {
         if (r + 1 < rows) o.y = v[(long long)(r + 1) * nx + e];
         return o;
     }
+    struct At {
+        const float* v;
+        int nx;
+        bool h1, h2;
+        __device__ __forceinline__ float2 operator()(int e) const
+        {
+            return make_float2(h1 ? v[e] : 0.f, h2 ? v[nx + e] : 0.f);
+        }
+    };
+    __device__ __forceinline__ At at(int p) const
+    {
+        const int r = row0 + 2 * p;
+        return At{v + (long long)r * nx, nx, r < rows, r + 1 < rows};
+    }
 };
 struct RowPairSt {
     float* v;
@@ -292,45 +407,154 @@ struct RowPairSt {
         if (r < rows) v[(long long)r * nx + e] = val.x;
         if (r + 1 < rows) v[(long long)(r + 1) * nx + e] = val.y;
     }
+    struct At {
+        float* v;
+        int nx;
+        bool h1, h2;
+        __device__ __forceinline__ void operator()(int e, float2 val) const
+        {
+            if (h1) v[e] = val.x;
+            if (h2) v[nx + e] = val.y;
+        }
+    };
+    __device__ __forceinline__ At at(int p) const
+    {
+        const int r = row0 + 2 * p;
+        return At{v + (long long)r * nx, nx, r < rows, r + 1 < rows};
+    }
 };
 
-// Forward: portrait spectrum of harmonic k0 + q / P at bin m =
+// Forward: one harmonic's portrait spectrum at bin m =
 // sum_{j < s} A[m + j mx] Xhat_k[m + j mx]   (the fold that realises P).
 struct FoldLd {
     const float2* A;
     int ldA;
-    const float2* __restrict__ Xh;   // Xhat + k0 * nx
-    int nx, mx, s, P;
-    __device__ __forceinline__ float2 operator()(int m, int q) const
-    {
-        const int kk = q / P, p = q - kk * P;
-        const float2* xk = Xh + (long long)kk * nx;
-        float2 acc = c_mul(A[m * ldA + p], __ldg(xk + m));
-        for (int j = 1; j < s; ++j) {
-            const int w = m + j * mx;
-            acc = c_add(acc, c_mul(A[w * ldA + p], __ldg(xk + w)));
+    const float2* __restrict__ xk;   // Xhat + k nx
+    int mx, s;
+    struct At {
+        const float2* A;
+        int ldA;
+        const float2* __restrict__ xk;
+        int mx, s;
+        __device__ __forceinline__ float2 operator()(int m) const
+        {
+            float2 acc = c_mul(A[m * ldA], __ldg(xk + m));
+            for (int j = 1; j < s; ++j) {
+                const int w = m + j * mx;
+                acc = c_add(acc, c_mul(A[w * ldA], __ldg(xk + w)));
+            }
+            return acc;
         }
-        return acc;
+    };
+    __device__ __forceinline__ At at(int p) const { return At{A + p, ldA, xk, mx, s}; }
+};
+
+// One harmonic's portrait rows (row0 + 2p, row0 + 2p + 1) of a pencil.
+// Windowed (padded plans): the portraits in memory are the field of view's,
+// fmx samples a row; row r = z ny + y of the extended mesh is row
+// (z - pz) fny + y - py, sample m is m - pm, and what lies outside the field
+// of view is not stored and reads as zero.
+struct PortraitRows {
+    int row0, rows, mx;
+    PortraitWin w;
+    // the row's offset in memory, or -1
+    __device__ __forceinline__ long long row(int r) const
+    {
+        if (r >= rows) return -1;
+        if (!w.on) return (long long)r * mx;
+        const int z = (int)w.dny.div((uint32_t)r), y = r - z * (int)w.dny.d;
+        const int fz = z - w.pz, fy = y - w.py;
+        if ((unsigned)fz >= (unsigned)w.fnz || (unsigned)fy >= (unsigned)w.fny) return -1;
+        return ((long long)fz * w.fny + fy) * w.fmx;
     }
+    __device__ __forceinline__ int m0() const { return w.on ? w.pm : 0; }
+    __device__ __forceinline__ int len() const { return w.on ? w.fmx : mx; }
 };
 
 struct PortraitSt {
-    float2* d;
-    const float2* __restrict__ phase;   // phase + k0
-    long long M;
-    int mx, row0, rows, P;
-    __device__ __forceinline__ void operator()(int m, int q, float2 val) const
+    float2* d;       // the harmonic's portraits
+    float2 ph;       // e^{i theta_k}
+    const PortraitRows& g;
+    struct At {
+        float2 *d0, *d1;   // the two rows, or null
+        float2 ph;
+        int m0, len;
+        __device__ __forceinline__ void operator()(int m, float2 val) const
+        {
+            m -= m0;
+            if ((unsigned)m >= (unsigned)len) return;
+            if (d0) d0[m] = make_float2(ph.x * val.x, ph.y * val.x);
+            if (d1) d1[m] = make_float2(ph.x * val.y, ph.y * val.y);
+        }
+    };
+    __device__ __forceinline__ At at(int p) const
     {
-        const int kk = q / P, p = q - kk * P;
-        const float2 ph = __ldg(phase + kk);
-        const int r = row0 + 2 * p;
-        float2* dk = d + (long long)kk * M;
-        if (r < rows) dk[(long long)r * mx + m] = make_float2(ph.x * val.x, ph.y * val.x);
-        if (r + 1 < rows) dk[(long long)(r + 1) * mx + m] = make_float2(ph.x * val.y, ph.y * val.y);
+        const long long i0 = g.row(g.row0 + 2 * p), i1 = g.row(g.row0 + 2 * p + 1);
+        return At{i0 >= 0 ? d + i0 : nullptr, i1 >= 0 ? d + i1 : nullptr, ph, g.m0(), g.len()};
     }
 };
 
 // Adjoint: (Re(e^{-i theta} y[row]), Re(e^{-i theta} y[row+1])) at sample m.
+struct PortraitKLd {
+    const float2* __restrict__ d;
+    float2 ph;
+    const PortraitRows& g;
+    struct At {
+        const float2 *d0, *d1;
+        float2 ph;
+        int m0, len;
+        __device__ __forceinline__ float2 operator()(int m) const
+        {
+            m -= m0;
+            const bool in = (unsigned)m < (unsigned)len;
+            const float2 z = make_float2(0.f, 0.f);
+            const float2 y0 = in && d0 ? __ldg(d0 + m) : z, y1 = in && d1 ? __ldg(d1 + m) : z;
+            return make_float2(fmaf(ph.x, y0.x, ph.y * y0.y), fmaf(ph.x, y1.x, ph.y * y1.y));
+        }
+    };
+    __device__ __forceinline__ At at(int p) const
+    {
+        const long long i0 = g.row(g.row0 + 2 * p), i1 = g.row(g.row0 + 2 * p + 1);
+        return At{i0 >= 0 ? d + i0 : nullptr, i1 >= 0 ? d + i1 : nullptr, ph, g.m0(), g.len()};
+    }
+};
+
+// One harmonic's 2 P portrait rows, copied to shared memory [2 P][pitch] by
+// 8-byte asynchronous copies, a warp per row.  What lies outside the field
+// of view or past the last row is not written: the caller zeroes the buffer
+// once.
+__device__ __forceinline__ void stage_portraits(float2* raw, int pitch, const float2* __restrict__ d,
+                                                const PortraitRows& g, int P)
+{
+    const int lane = (int)threadIdx.x & 31, nw = (int)blockDim.x >> 5, len = g.len();
+    for (int rr = (int)threadIdx.x >> 5; rr < 2 * P; rr += nw) {
+        const long long o = g.row(g.row0 + rr);
+        if (o < 0) continue;
+        const float2* src = d + o;
+        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(raw + rr * pitch + g.m0());
+        for (int m = lane; m < len; m += 32)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst + 8 * m), "l"(src + m) : "memory");
+    }
+}
+// Those rows as the adjoint's pencils.
+struct RawRowsLd {
+    const float2* raw;
+    float2 ph;
+    int pitch;
+    struct At {
+        const float2* d;
+        float2 ph;
+        int pitch;
+        __device__ __forceinline__ float2 operator()(int m) const
+        {
+            const float2 y0 = d[m], y1 = d[pitch + m];
+            return make_float2(fmaf(ph.x, y0.x, ph.y * y0.y), fmaf(ph.x, y1.x, ph.y * y1.y));
+        }
+    };
+    __device__ __forceinline__ At at(int p) const { return At{raw + 2 * p * pitch, ph, pitch}; }
+};
+
+// The same for the specialised adjoint (ops_ct.cuh), harmonic k0 + q / P.
 struct PortraitLd {
     const float2* __restrict__ d;
     const float2* __restrict__ phase;
@@ -361,40 +585,62 @@ struct QLd {
     int ldA;
     const float2* __restrict__ Q;
     int mx, s;
-    __device__ __forceinline__ float2 operator()(int w, int p) const
-    {
-        const int a = w / mx, m = w - a * mx;
-        const float2* qm = Q + ((long long)m * s + a) * s;
-        float2 acc = make_float2(0.f, 0.f);
-        for (int b = 0; b < s; ++b) acc = c_add(acc, c_mul(__ldg(qm + b), A[(m + b * mx) * ldA + p]));
-        return acc;
-    }
+    FastDiv dmx;
+    struct At {
+        const float2* A;
+        int ldA;
+        const float2* __restrict__ Q;
+        int mx, s;
+        FastDiv dmx;
+        __device__ __forceinline__ float2 operator()(int w) const
+        {
+            const int a = (int)dmx.div((uint32_t)w), m = w - a * mx;
+            const float2* qm = Q + (m * s + a) * s;
+            float2 acc = make_float2(0.f, 0.f);
+            for (int b = 0; b < s; ++b) acc = c_add(acc, c_mul(__ldg(qm + b), A[(m + b * mx) * ldA]));
+            return acc;
+        }
+    };
+    __device__ __forceinline__ At at(int p) const { return At{A + p, ldA, Q, mx, s, dmx}; }
 };
 
-// Normal epilogue: q = b w + lambda R p, accumulating p^T q.
-struct NrmEpiSt {
-    const XArgs* a;
-    int row0;
-    DotAcc* acc;
-    DotAcc* acc2 = nullptr;   // input . input (single-reduction CG)
-    __device__ __forceinline__ void one(int r, int x, float w) const
-    {
-        const long long i = (long long)r * a->nx + x;
-        float q = a->b ? a->b[i] * w : w;
-        const RegArgs& g = a->reg;
-        const int z = r / g.ny, y = r - z * g.ny;
-        q += reg_term(g, a->pin, i, x, y, z);
-        a->qout[i] = q;
-        const float pv = a->pin[i];
-        acc->add(pv, q);
-        if (acc2) acc2->add(pv, pv);
+// Normal epilogue q = b w + lambda R p over a tile of 2 P rows of w (pencil
+// layout, row 2p the real and row 2p + 1 the imaginary part), accumulating
+// p^T q (and p^T p for acc2), lanes along x.
+__device__ __forceinline__ void nrm_epilogue_rt(const XArgs& a, int row0, int P, const float2* w, int ld, DotAcc* acc,
+                                                DotAcc* acc2)
+{
+    const float* wf = reinterpret_cast<const float*>(w);
+    const bool plain = a.reg.kind == 0;
+    const int nx = a.nx, lane = (int)threadIdx.x & 31, nw = (int)blockDim.x >> 5;
+    constexpr int U = 4;   // elements a step, their loads first
+    for (int rr = (int)threadIdx.x >> 5; rr < 2 * P && row0 + rr < a.rows; rr += nw) {   // a warp per row
+        const int r = row0 + rr, i0 = r * nx;
+        const int z = (int)a.dny.div((uint32_t)r), y = r - z * a.reg.ny;
+        const float* wr = wf + 2 * (rr >> 1) + (rr & 1);
+        for (int x0 = lane; x0 < nx; x0 += 32 * U) {
+            float pv[U], bv[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int x = x0 + 32 * u;
+                if (x >= nx) continue;
+                pv[u] = a.pin[i0 + x];
+                bv[u] = a.b ? a.b[i0 + x] : 1.f;
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int x = x0 + 32 * u;
+                if (x >= nx) continue;
+                const float v = wr[2 * x * ld];
+                float q = a.b ? bv[u] * v : v;
+                if (plain) q += a.reg.lambda * pv[u];
+                else q += reg_term(a.reg, a.pin, i0 + x, x, y, z);
+                a.qout[i0 + x] = q;
+                acc->add(pv[u], q);
+                if (acc2) acc2->add(pv[u], pv[u]);
+            }
+        }
     }
-    __device__ __forceinline__ void operator()(int x, int p, float2 val) const
-    {
-        const int r = row0 + 2 * p;
-        if (r < a->rows) one(r, x, val.x);
-        if (r + 1 < a->rows) one(r + 1, x, val.y);
-    }
-};
+}
 
 }  // namespace mh3d

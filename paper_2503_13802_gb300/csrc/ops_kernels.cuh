@@ -59,6 +59,16 @@ struct TMaps {
     CUtensorMap m[kTmCount];
 };
 
+// The field of view inside the extended portrait mesh of a padded plan: the
+// drive-axis kernels that take it read and write field-of-view portraits
+// (see PortraitRows).
+struct PortraitWin {
+    int on = 0;
+    int pz = 0, py = 0, pm = 0;      // offsets of the field of view
+    int fnz = 0, fny = 0, fmx = 0;   // its portrait mesh
+    FastDiv dny;                     // by the extended ny
+};
+
 // T pass: 1D circular convolution along y or z of tiles of `cols` columns.
 struct TArgs {
     TMaps tm;                        // filled by the bulk-copy launcher
@@ -137,6 +147,12 @@ struct XArgs {
     int cg_active = 0;
     int* status = nullptr;           // device status word for bounded-wait timeouts
     int ks = 0;                      // warp-centric passes: warps per row group (0: default)
+    FastDiv dny;                     // by ny (rows are z ny + y)
+    FastDiv dmx;                     // by mx (run-time normal pass)
+    int lgP = 0;                     // run-time kernels: log2 of the row pairs per CTA
+    int lgK = 0;                     // run-time passes: log2 of the harmonics per round
+    int pitch = 0;                   // run-time adjoint: float2 between staged portrait rows
+    PortraitWin win;                 // padded plans (run-time kernels only)
 };
 
 // The y-slab cluster passes (ops_ct.cuh: k_zxnrm_ct, k_zxfwd_ct,
@@ -150,7 +166,8 @@ struct ZXArgs {
     int C = 0;                       // CTAs per y-slab (2 or 4; 0: default)
 };
 
-// Shared-memory sizes in bytes.
+// Shared-memory sizes in bytes (the plan's acceptance rule; the run-time
+// kernels choose their own launch shapes within it).
 __host__ __forceinline__ size_t tpass_smem_bytes(int n, int cols)
 {
     const int P = cols / 2;
@@ -169,6 +186,11 @@ __host__ __forceinline__ size_t xnrm_smem_bytes(int nx, int pairs)
 {
     return sizeof(float2) * (size_t)(nx + 2 * nx * (pairs + 1));
 }
+
+// Row pairs per CTA of the run-time normal pass.
+int xnrm_rt_pairs(const RadixPlan& rpx);
+// Whether the run-time drive-axis passes take a windowed (padded) mesh.
+bool xpass_windowed(int nx, int mx, int s, int pairs);
 
 // Launchers (ops.cu).
 cudaError_t run_tpass(const TArgs& a, int nouter, cudaStream_t st);

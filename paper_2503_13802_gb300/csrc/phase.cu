@@ -220,7 +220,7 @@ mh3d_status mh3d_estimate_phase(mh3d_plan P, const void* d_dev, double frac, dou
         PH_CK(S.get(&x, sizeof(float) * (size_t)P->N));
         PH_CK(S.get(&f, sizeof(float2) * K));
         PH_CK(S.get(&dpart, sizeof(double) * kPhBlocks));
-        if (P->padded && ensure_portrait(*P) != MH3D_OK) return MH3D_ERR_OOM;
+        if (P->padded && !P->windowed && ensure_portrait(*P) != MH3D_OK) return MH3D_ERR_OOM;
         const int nb = (int)std::min<long long>(((long long)K * Mf + 255) / 256, 4096);
         // y = the de-phased portraits of the harmonics with weight w_j != 0,
         // times w_j, expressed for the plan's own phase (the adjoint and the
@@ -237,7 +237,7 @@ mh3d_status mh3d_estimate_phase(mh3d_plan P, const void* d_dev, double frac, dou
             return cudaGetLastError();
         };
         auto backproject = [&](float* out) -> cudaError_t {
-            if (P->padded) {
+            if (P->padded && !P->windowed) {
                 cudaError_t e = pad_portraits(*P, y, P->w.portrait, st);
                 if (e != cudaSuccess) return e;
                 return launch_adjoint(*P, P->w.portrait, out, P->w.t1, P->w.t2, st);

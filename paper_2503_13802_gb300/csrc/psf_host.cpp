@@ -228,38 +228,51 @@ std::vector<cplx> twiddles(int n)
     return w;
 }
 
-// Radix schedule for a length: factors 8, 4, 2, 3 only.  The default puts
-// large radices first; the autotuner may pick another permutation.
-bool radix_plan(int n, RadixPlan& pl, int variant)
+// The radix schedule of length n = 2^a 3^b: the fewest stages with the
+// radices below, then the smallest sum of radices (the fewest operations and
+// registers), the largest radix first.  Every stage is a round trip of the
+// pencils through shared memory and a barrier: two stages cover every length
+// up to 144 and most up to 256, three every length up to 1024.
+bool radix_plan(int n, RadixPlan& pl, int max_last)
 {
+    static const int kRadix[] = {16, 12, 9, 8, 6, 4, 3, 2};
+    pl = RadixPlan();
     pl.n = n;
-    pl.nst = 0;
-    int m = n, p2 = 0, p3 = 0;
-    while (m % 2 == 0) { m /= 2; ++p2; }
-    while (m % 3 == 0) { m /= 3; ++p3; }
-    if (m != 1 || n < 1 || n > kMaxLen) return false;
-    int rs[kMaxStages];
-    int ns = 0;
-    // variant 0: 8s first; variant 1: 4s (then a trailing 8/2); variant 2: 8s last.
-    int e = p2;
-    if (variant == 1) {
-        while (e >= 2 && ns < kMaxStages) { rs[ns++] = 4; e -= 2; }
-        if (e == 1) rs[ns++] = 2;
-    } else {
-        while (e >= 3 && ns < kMaxStages) { rs[ns++] = 8; e -= 3; }
-        if (e == 2) rs[ns++] = 4;
-        if (e == 1) rs[ns++] = 2;
-        if (variant == 2) {   // reverse the power-of-two part
-            for (int i = 0; i < ns / 2; ++i) { int t = rs[i]; rs[i] = rs[ns - 1 - i]; rs[ns - 1 - i] = t; }
+    if (n < 1 || n > kMaxLen) return false;
+    int best[kMaxStages], cur[kMaxStages], bn = kMaxStages + 1, bs = 1 << 30;
+    // depth-first over non-increasing radices (a schedule of few stages is short)
+    struct Search {
+        int max_last, *best, *cur, &bn, &bs;
+        void go(int left, int depth, int from, int sum)
+        {
+            if (left == 1) {
+                if (depth > 0 && max_last > 0 && cur[depth - 1] > max_last) return;
+                if (depth < bn || (depth == bn && sum < bs)) {
+                    bn = depth;
+                    bs = sum;
+                    for (int i = 0; i < depth; ++i) best[i] = cur[i];
+                }
+                return;
+            }
+            if (depth == kMaxStages) return;
+            for (int i = from; i < (int)(sizeof kRadix / sizeof kRadix[0]); ++i)
+                if (left % kRadix[i] == 0) {
+                    cur[depth] = kRadix[i];
+                    go(left / kRadix[i], depth + 1, i, sum + kRadix[i]);
+                }
         }
+    } search{max_last, best, cur, bn, bs};
+    search.go(n, 0, 0, 0);
+    if (bn > kMaxStages) return false;
+    pl.nst = bn;
+    for (int s = 0; s < bn; ++s) pl.radix[s] = best[s];
+    for (int s = 0; s < bn; ++s) {
+        for (int q = 0; q < s; ++q) pl.ns[s] *= best[q];
+        for (int q = s + 1; q < bn; ++q) pl.nsr[s] *= best[q];
+        pl.dnb[s] = FastDiv(n / best[s]);
+        pl.dns[s] = FastDiv(pl.ns[s]);
+        pl.dnsr[s] = FastDiv(pl.nsr[s]);
     }
-    for (int i = 0; i < p3; ++i) {
-        if (ns >= kMaxStages) return false;
-        rs[ns++] = 3;
-    }
-    pl.nst = ns;
-    for (int i = 0; i < ns; ++i) pl.radix[i] = rs[i];
-    for (int i = ns; i < kMaxStages; ++i) pl.radix[i] = 1;
     return true;
 }
 

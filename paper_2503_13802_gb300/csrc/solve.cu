@@ -248,7 +248,8 @@ mh3d_status solve_alloc(Plan& P)
     // partial-sum slots for the widest grid any tile choice (8-column T pass) can launch
     const size_t cap = (size_t)std::max({update_blocks(P.N), normal_part_count(P, 0), normal_part_count(P, 1),
                                          tpass_blocks(P.nx, 8, tpass_outer(P, 1)),
-                                         xpass_blocks(P.ny * P.nz, 8), 1});
+                                         xpass_blocks(P.ny * P.nz, 8),
+                                         xpass_blocks(P.ny * P.nz, xnrm_rt_pairs(P.ax.rp)), 1});
     w.red_cap = cap;
     const size_t bytes = sizeof(float) * vec * 8 + red_bytes(cap) + 64;
     if (dev_malloc(&w.base, bytes) != cudaSuccess) {
@@ -1453,16 +1454,20 @@ mh3d_status mh3d_solve(mh3d_plan P, const void* d, const mh3d_solve_opts* o, flo
     if (v != MH3D_OK) return v;
     P->err.clear();
     if (P->padded) {
-        // the field of view's portraits zero-padded into the portrait buffer
-        // (read once, by A^T d, before the explicit normal operator reuses
+        // the field of view's portraits, zero-padded into the portrait buffer
+        // unless the passes take them as they are (read once, by A^T d, before the explicit normal operator reuses
         // it); the masked explicit normal operator throughout
         mh3d_status s = ensure_portrait(*P);
         if (s != MH3D_OK) return s;
-        MH3D_CK(*P, pad_portraits(*P, (const float2*)d, P->w.portrait, (cudaStream_t)stream));
+        const float2* src = (const float2*)d;
+        if (!P->windowed) {
+            MH3D_CK(*P, pad_portraits(*P, src, P->w.portrait, (cudaStream_t)stream));
+            src = P->w.portrait;
+        }
         mh3d_solve_opts op = *o;
         op.normal_mode = 1;
-        if (o->solver == 1) return apg_solve(*P, P->w.portrait, op, rho, info, (cudaStream_t)stream);
-        return cg_solve(*P, P->w.portrait, op, rho, info, (cudaStream_t)stream);
+        if (o->solver == 1) return apg_solve(*P, src, op, rho, info, (cudaStream_t)stream);
+        return cg_solve(*P, src, op, rho, info, (cudaStream_t)stream);
     }
     if (o->solver == 1) return apg_solve(*P, (const float2*)d, *o, rho, info, (cudaStream_t)stream);
     return cg_solve(*P, (const float2*)d, *o, rho, info, (cudaStream_t)stream);
