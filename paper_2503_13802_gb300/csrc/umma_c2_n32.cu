@@ -1,0 +1,4 @@
+// The tcgen05 convolution with 2 chunk planes and 32 accumulator columns.
+#define UMMA_C8P 2
+#define UMMA_NP 32
+#include "umma_launch.cuh"

@@ -156,102 +156,124 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // Stages the tile's halo: 16-byte units, channels 8 c .. 8 c + 7 of voxel
 // (z + dz, y + dy, x0 - 1 + xi), zero outside the volume.  Only the cv
 // chunks that carry channels are written (the padding chunks stay zero from
-// the kernel's start).  Each thread takes whole voxels.  Plain and
-// upsampled bfloat16 sources: one cp.async per unit, all in flight at once.
-// The skip sum (rounded to bfloat16, as a stored sum would be; not
-// upsampled) and the FP32 input (rounded to bfloat16, channel 0) need
-// arithmetic: their units are loaded into registers in batches (all loads
-// of a batch in flight), combined and stored.
+// the kernel's start).  A warp takes whole planes (one neighbour row each),
+// its lanes the row's voxels, so that the row's bounds and base are formed
+// once per plane and a unit costs an add, a compare and its copy: with a
+// voxel per thread (a division and seven compares each) the staging's
+// instructions, not its bytes, set the pace of the narrow layers (16 -> 16
+// channels at 128x128x64: 89 us a layer).  Plain and upsampled bfloat16
+// sources: one cp.async per unit, all in flight at once.  The skip sum
+// (rounded to bfloat16, as a stored sum would be; not upsampled) and the
+// FP32 input (rounded to bfloat16, channel 0) need arithmetic: their units
+// are loaded into registers first (all loads of a plane, or of a warp's
+// planes, in flight), combined and stored.
 template <int C8P, int R>
 __device__ __forceinline__ void stage_halo(const ConvSrc& src, unsigned char* sH, int z, int y, int x0, int cv,
-                                           int tid = threadIdx.x, int nthr = kT)
+                                           int tid = threadIdx.x)
 {
-    constexpr int PL = planes<R>();
-    constexpr int NV = PL * 130;
-    constexpr size_t CST = (size_t)PL * kHP * 16;   // bytes between chunk planes
-    auto voxel = [&](int vi, unsigned char*& d, long long& off) {
-        const int plane = vi / 130, xi = vi - plane * 130;
-        const int zz = z + plane / (R + 2) - 1, yy = y + plane % (R + 2) - 1, xx = x0 + xi - 1;
-        d = sH + ((size_t)plane * kHP + xi) * 16;
-        const bool in = zz >= 0 && zz < src.D && yy >= 0 && yy < src.H && xx >= 0 && xx < src.W;
-        if (!in) {
-            off = -1;
-        } else if (src.up) {
-            off = (((long long)(zz >> 1) * (src.H >> 1) + (yy >> 1)) * (src.W >> 1) + (xx >> 1)) * src.C;
-        } else {
-            off = (((long long)zz * src.H + yy) * src.W + xx) * (src.f32 ? 1 : src.C);
-        }
+    constexpr int PL = planes<R>(), NW = kT / 32, PW = (PL + NW - 1) / NW;   // planes per warp
+    constexpr int XI = (130 + 31) / 32;                                      // voxels per lane
+    constexpr size_t CST = (size_t)PL * kHP * 16;                            // bytes between chunk planes
+    const int warp = tid >> 5, lane = tid & 31;
+    // the plane's source row: its first voxel's index, or -1
+    auto row_of = [&](int plane) -> long long {
+        const int zz = z + plane / (R + 2) - 1, yy = y + plane % (R + 2) - 1;
+        if ((unsigned)zz >= (unsigned)src.D || (unsigned)yy >= (unsigned)src.H) return -1;
+        if (src.up) return ((long long)(zz >> 1) * (src.H >> 1) + (yy >> 1)) * (src.W >> 1);
+        return ((long long)zz * src.H + yy) * src.W;
     };
     if (!src.b && !src.f32) {
-        for (int vi = tid; vi < NV; vi += nthr) {
-            unsigned char* d;
-            long long off;
-            voxel(vi, d, off);
-            const __nv_bfloat16* g = off >= 0 ? src.a + off : src.a;
+        const int C = src.C, sh = src.up ? 1 : 0;
 #pragma unroll
-            for (int c = 0; c < C8P; ++c)
-                if (c < cv) cp_async16(d + c * CST, g + 8 * c, off >= 0 ? 16u : 0u);
+        for (int q = 0; q < PW; ++q) {
+            const int plane = warp + q * NW;
+            if (plane >= PL) break;
+            const long long row = row_of(plane);
+            const __nv_bfloat16* g = src.a + (row >= 0 ? row * C : 0);
+            unsigned char* d = sH + (size_t)plane * kHP * 16;
+#pragma unroll
+            for (int i = 0; i < XI; ++i) {
+                const int xi = lane + 32 * i, xx = x0 + xi - 1;
+                if (xi >= 130) break;
+                const bool in = row >= 0 && (unsigned)xx < (unsigned)src.W;
+                const __nv_bfloat16* gx = g + (in ? (xx >> sh) * C : 0);
+#pragma unroll
+                for (int c = 0; c < C8P; ++c)
+                    if (c < cv) cp_async16(d + xi * 16 + c * CST, gx + 8 * c, in ? 16u : 0u);
+            }
         }
         return;   // the caller waits (cp_async_wait_all) before the halo is read
     }
     if (src.f32) {
-        constexpr int kB = 8;
         const float fsc = src.f32_scale ? *src.f32_scale : 1.f;
-        for (int v0 = tid; v0 < NV; v0 += kB * nthr) {
-            unsigned char* d[kB];
-            long long off[kB];
-            float f[kB];
+        float f[PW][XI];
 #pragma unroll
-            for (int i = 0; i < kB; ++i) {
-                const int vi = v0 + i * nthr;
-                if (vi < NV) voxel(vi, d[i], off[i]);
-                else off[i] = -2;
+        for (int q = 0; q < PW; ++q) {
+            const int plane = warp + q * NW;
+            const long long row = plane < PL ? row_of(plane) : -1;
+            const float* g = src.f32 + (row >= 0 ? row : 0);
+#pragma unroll
+            for (int i = 0; i < XI; ++i) {
+                const int xi = lane + 32 * i, xx = x0 + xi - 1;
+                f[q][i] = row >= 0 && xi < 130 && (unsigned)xx < (unsigned)src.W ? __ldg(g + xx) : 0.f;
             }
+        }
 #pragma unroll
-            for (int i = 0; i < kB; ++i) f[i] = off[i] >= 0 ? __ldg(src.f32 + off[i]) : 0.f;
+        for (int q = 0; q < PW; ++q) {
+            const int plane = warp + q * NW;
+            if (plane >= PL) break;
+            unsigned char* d = sH + (size_t)plane * kHP * 16;
 #pragma unroll
-            for (int i = 0; i < kB; ++i) {
-                if (off[i] == -2) continue;
-                const __nv_bfloat16 b = __float2bfloat16(f[i] * fsc);
-                *reinterpret_cast<uint4*>(d[i]) =
-                    make_uint4(off[i] >= 0 ? (uint32_t)(*reinterpret_cast<const uint16_t*>(&b)) : 0u, 0, 0, 0);
+            for (int i = 0; i < XI; ++i) {
+                const int xi = lane + 32 * i;
+                if (xi >= 130) break;
+                const __nv_bfloat16 b = __float2bfloat16(f[q][i] * fsc);
+                // (a zero outside the volume stays +0 whatever the scale's sign)
+                const bool in = (unsigned)(x0 + xi - 1) < (unsigned)src.W && row_of(plane) >= 0;
+                *reinterpret_cast<uint4*>(d + xi * 16) =
+                    make_uint4(in ? (uint32_t)(*reinterpret_cast<const uint16_t*>(&b)) : 0u, 0, 0, 0);
             }
         }
         return;
     }
-    constexpr int kB = 8 / C8P > 0 ? 8 / C8P : 1;   // voxels per batch: 8 chunk units
-    for (int v0 = tid; v0 < NV; v0 += kB * nthr) {
-        unsigned char* d[kB];
-        long long off[kB];
-        uint4 va[kB][C8P], vb[kB][C8P];
+#pragma unroll 1
+    for (int q = 0; q < PW; ++q) {
+        const int plane = warp + q * NW;
+        if (plane >= PL) break;
+        const long long row = row_of(plane);
+        unsigned char* d = sH + (size_t)plane * kHP * 16;
 #pragma unroll
-        for (int i = 0; i < kB; ++i) {
-            const int vi = v0 + i * nthr;
-            if (vi < NV) voxel(vi, d[i], off[i]);
-            else off[i] = -2;
-        }
+        for (int c0 = 0; c0 < C8P; c0 += 2) {
+            if (c0 >= cv) break;
+            uint4 va[XI][2], vb[XI][2];
 #pragma unroll
-        for (int i = 0; i < kB; ++i)
+            for (int i = 0; i < XI; ++i) {
+                const int xi = lane + 32 * i, xx = x0 + xi - 1;
+                const bool in = row >= 0 && xi < 130 && (unsigned)xx < (unsigned)src.W;
+                const long long off = in ? (row + xx) * src.C + 8 * c0 : 0;
 #pragma unroll
-            for (int c = 0; c < C8P; ++c) {
-                const bool in = off[i] >= 0 && c < cv;
-                va[i][c] = in ? __ldg(reinterpret_cast<const uint4*>(src.a + off[i] + 8 * c)) : make_uint4(0, 0, 0, 0);
-                vb[i][c] = in ? __ldg(reinterpret_cast<const uint4*>(src.b + off[i] + 8 * c)) : make_uint4(0, 0, 0, 0);
+                for (int c = 0; c < 2; ++c) {
+                    const bool use = in && c0 + c < cv;
+                    va[i][c] = use ? __ldg(reinterpret_cast<const uint4*>(src.a + off + 8 * c)) : make_uint4(0, 0, 0, 0);
+                    vb[i][c] = use ? __ldg(reinterpret_cast<const uint4*>(src.b + off + 8 * c)) : make_uint4(0, 0, 0, 0);
+                }
             }
 #pragma unroll
-        for (int i = 0; i < kB; ++i) {
-            if (off[i] == -2) continue;
+            for (int i = 0; i < XI; ++i) {
+                const int xi = lane + 32 * i;
+                if (xi >= 130) break;
 #pragma unroll
-            for (int c = 0; c < C8P; ++c) {
-                if (c >= cv) continue;
-                __nv_bfloat162* pr = reinterpret_cast<__nv_bfloat162*>(&va[i][c]);
-                const __nv_bfloat162* pq = reinterpret_cast<const __nv_bfloat162*>(&vb[i][c]);
+                for (int c = 0; c < 2; ++c) {
+                    if (c0 + c >= cv) continue;
+                    __nv_bfloat162* pr = reinterpret_cast<__nv_bfloat162*>(&va[i][c]);
+                    const __nv_bfloat162* pq = reinterpret_cast<const __nv_bfloat162*>(&vb[i][c]);
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const float2 a = __bfloat1622float2(pr[k]), b = __bfloat1622float2(pq[k]);
-                    pr[k] = __floats2bfloat162_rn(a.x + b.x, a.y + b.y);
+                    for (int k = 0; k < 4; ++k) {
+                        const float2 a = __bfloat1622float2(pr[k]), b = __bfloat1622float2(pq[k]);
+                        pr[k] = __floats2bfloat162_rn(a.x + b.x, a.y + b.y);
+                    }
+                    *reinterpret_cast<uint4*>(d + xi * 16 + (c0 + c) * CST) = va[i][c];
                 }
-                *reinterpret_cast<uint4*>(d[i] + c * CST) = va[i][c];
             }
         }
     }
@@ -318,43 +340,54 @@ __device__ __forceinline__ void epilogue(const ConvSrc& src, uint32_t acc, int z
 // on -- and a second MMA the third plane with a zero second chunk: 18 MMAs a
 // row instead of 27.  The paired weights ([3 pz][3 px][2 g][2 c][NP][8],
 // k_prep_umma_pair) are indexed by plane offsets, the flip folded in.
+// Both operands' descriptors are a base plus an offset (of the taps', in
+// 16-byte units, from a table in shared memory: tap_offsets): the issuing
+// thread's instructions per MMA are part of every tile's chain.
+template <int R>
+__device__ __forceinline__ void tap_offsets(uint32_t* aoff, int sgn)
+{
+    if (threadIdx.x < 27) {
+        const int tap = threadIdx.x;
+        const int dz = sgn * (tap / 9 - 1), dy = sgn * ((tap / 3) % 3 - 1), dx = sgn * (tap % 3 - 1);
+        aoff[tap] = (uint32_t)(((dz + 1) * (R + 2) + dy + 1) * kHP + dx + 1);
+    }
+}
+
 template <int C8P, int NP, int R>
-__device__ __forceinline__ void issue_mmas(uint32_t acc, uint32_t sH_a, uint32_t sW_a, int sgn, uint64_t* bar,
-                                           int pair = 0)
+__device__ __forceinline__ void issue_mmas(uint32_t acc, uint32_t sH_a, uint32_t sW_a, const uint32_t* aoff,
+                                           uint64_t* bar, int pair = 0)
 {
     constexpr uint32_t kIdesc = idesc_bf16(kM, NP);
     constexpr int PL = planes<R>();
+    // (start addresses count 16-byte units: offsets add to the low field)
+    const uint64_t b0 = smem_desc(sW_a, NP * 16, 128);
     if (pair) {
-        for (int pz = 0; pz < 3; ++pz)
-            for (int px = 0; px < 3; ++px)
+        const uint64_t a0 = smem_desc(sH_a, kHP * 16, 128);
 #pragma unroll
-                for (int g = 0; g < 2; ++g) {
-                    const uint32_t b = sW_a + (uint32_t)((((pz * 3 + px) * 2 + g) * 2) * NP * 16);
-                    const uint64_t bdesc = smem_desc(b, NP * 16, 128);
-                    const uint32_t accumulate = (pz | px | g) != 0;
+        for (int pzx = 0; pzx < 9; ++pzx)
 #pragma unroll
-                    for (int r = 0; r < R; ++r) {
-                        const int plane = pz * (R + 2) + r + 2 * g;
-                        const uint32_t a = sH_a + (uint32_t)((plane * kHP + px) * 16);
-                        mma_f16(acc + (uint32_t)(r * NP), smem_desc(a, kHP * 16, 128), bdesc, kIdesc, accumulate);
-                    }
+            for (int g = 0; g < 2; ++g) {
+                const int pz = pzx / 3, px = pzx % 3;
+                const uint64_t bdesc = b0 + (uint64_t)(((pzx * 2 + g) * 2) * NP);
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const int plane = pz * (R + 2) + r + 2 * g;
+                    mma_f16(acc + (uint32_t)(r * NP), a0 + (uint64_t)(plane * kHP + px), bdesc, kIdesc, (pzx | g) != 0);
                 }
+            }
         mma_commit(bar);
         return;
     }
+    const uint64_t a0 = smem_desc(sH_a, PL * kHP * 16, 128);
+#pragma unroll 3
     for (int tap = 0; tap < 27; ++tap) {
-        const int dz = sgn * (tap / 9 - 1), dy = sgn * ((tap / 3) % 3 - 1), dx = sgn * (tap % 3 - 1);
+        const uint64_t at = a0 + aoff[tap];
 #pragma unroll
         for (int ks = 0; ks < C8P / 2; ++ks) {
-            const uint32_t b = sW_a + (uint32_t)((tap * C8P + 2 * ks) * NP * 16);
-            const uint64_t bdesc = smem_desc(b, NP * 16, 128);
-            const uint32_t accumulate = (tap | ks) != 0;
+            const uint64_t bdesc = b0 + (uint64_t)((tap * C8P + 2 * ks) * NP);
 #pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const int plane = (dz + 1) * (R + 2) + (r + dy + 1);
-                const uint32_t a = sH_a + (uint32_t)(((2 * ks * PL + plane) * kHP + dx + 1) * 16);
-                mma_f16(acc + (uint32_t)(r * NP), smem_desc(a, PL * kHP * 16, 128), bdesc, kIdesc, accumulate);
-            }
+            for (int r = 0; r < R; ++r)
+                mma_f16(acc + (uint32_t)(r * NP), at + (uint64_t)((2 * ks * PL + r) * kHP), bdesc, kIdesc, (tap | ks) != 0);
         }
     }
     mma_commit(bar);
@@ -372,13 +405,14 @@ __global__ void __launch_bounds__(kT) k_conv_umma(ConvSrc src, const __nv_bfloat
     extern __shared__ unsigned char umma_raw[];
     __shared__ __align__(8) uint64_t mbar[2];
     __shared__ uint32_t tmem_base_s;
+    __shared__ uint32_t aoff[27];
     unsigned char* base =
         reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(umma_raw) + 1023) & ~uintptr_t(1023));
     unsigned char* sW = base;                  // [27][C8P][NP][16 B]
     unsigned char* sH = base + G::kWBytes;     // NB x [C8P][9][kHP][16 B]
     const int warp = threadIdx.x >> 5;
     const int ntx = (src.W + kM - 1) / kM;
-    const int sgn = src.flip ? -1 : 1;
+    tap_offsets<R>(aoff, src.flip ? -1 : 1);
 
     if (warp == 0) {
         tmem_alloc(&tmem_base_s, G::kCols);
@@ -430,7 +464,7 @@ __global__ void __launch_bounds__(kT) k_conv_umma(ConvSrc src, const __nv_bfloat
             __syncthreads();
             if (threadIdx.x == 0) {
                 tc_fence_after();
-                issue_mmas<C8P, NP, R>(tmem, sH_a, sW_a, sgn, &mbar[0], pair);
+                issue_mmas<C8P, NP, R>(tmem, sH_a, sW_a, aoff, &mbar[0], pair);
             }
             // one thread waits on the MMAs' mbarrier; the block barrier
             // releases the others (no spinning warps taking issue slots)
@@ -462,7 +496,7 @@ __global__ void __launch_bounds__(kT) k_conv_umma(ConvSrc src, const __nv_bfloat
             __syncthreads();
             if (threadIdx.x == 0) {
                 tc_fence_after();
-                issue_mmas<C8P, NP, 1>(tmem + (uint32_t)(b * NP), sH_a + (uint32_t)(b * G::kHBytes), sW_a, sgn,
+                issue_mmas<C8P, NP, 1>(tmem + (uint32_t)(b * NP), sH_a + (uint32_t)(b * G::kHBytes), sW_a, aoff,
                                        &mbar[b]);
             }
             if (i > 0) {   // tile i - 1's MMAs: done before its halo buffer is refilled
@@ -638,7 +672,7 @@ __global__ void __launch_bounds__(kWsT, 1) k_conv_umma_ws(ConvSrc src, const __n
             if (abort_s) break;
             int z, y, x0;
             origin(tile, z, y, x0);
-            stage_halo<C8P, 1>(src, sH + (size_t)sl * G::kHBytes, z, y, x0, cv, pt, 128);
+            stage_halo<C8P, 1>(src, sH + (size_t)sl * G::kHBytes, z, y, x0, cv, pt);
             if (async_src) {
                 cp_async_commit();
                 if (i >= NS - 1) {   // tile i - (NS - 1) has landed
@@ -698,44 +732,6 @@ __global__ void __launch_bounds__(kWsT, 1) k_conv_umma_ws(ConvSrc src, const __n
         tc_fence_after();
         tmem_dealloc(tmem, G::kCols);
     }
-}
-
-// The paired-tap weights of a source of at most 8 channels:
-// Wp[pz][px][g][c][n][j], plane offsets (pz, p, px) of the halo, p = 0 and 1
-// for g = 0 (c = 0, 1) and p = 2 for g = 1 (c = 0; c = 1 zero); the tap is
-// the one applied at offset (pz - 1, p - 1, px - 1) = sgn (dz, dy, dx).
-__global__ void k_prep_umma_pair(const __nv_bfloat16* __restrict__ Wt, int Npad, int Cs, int N, int NP, int sgn,
-                                 __nv_bfloat16* __restrict__ Wp)
-{
-    const int total = 9 * 2 * 2 * NP * 8;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= total) return;
-    const int j = i % 8, n = (i / 8) % NP, c = (i / (8 * NP)) % 2, g = (i / (16 * NP)) % 2, pzx = i / (32 * NP);
-    const int pz = pzx / 3, px = pzx % 3;
-    const int p = g == 0 ? c : (c == 0 ? 2 : -1);
-    __nv_bfloat16 v = __float2bfloat16(0.f);
-    if (p >= 0 && j < Cs && n < N) {
-        const int dz = sgn * (pz - 1), dy = sgn * (p - 1), dx = sgn * (px - 1);
-        const int tap = 9 * (dz + 1) + 3 * (dy + 1) + (dx + 1);
-        v = Wt[(size_t)(tap * Cs + j) * Npad + n];
-    }
-    Wp[i] = v;
-}
-
-// Wu[tap][c][n][j] = Wt[(tap * Cs + 8 c + j) * Npad + n] (zero past Cs
-// source channels or N output channels); Wt is the implicit-GEMM matrix
-// [Kpad][Npad] of the mma.sync kernels (forward or input-gradient layout).
-__global__ void k_prep_umma(const __nv_bfloat16* __restrict__ Wt, int Npad, int Cs, int N, int C8P, int NP,
-                            __nv_bfloat16* __restrict__ Wu)
-{
-    const int total = 27 * C8P * NP * 8;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= total) return;
-    const int j = i % 8, n = (i / 8) % NP, c = (i / (8 * NP)) % C8P, tap = i / (8 * NP * C8P);
-    const int ci = 8 * c + j;
-    __nv_bfloat16 v = __float2bfloat16(0.f);
-    if (ci < Cs && n < N) v = Wt[(size_t)(tap * Cs + ci) * Npad + n];
-    Wu[i] = v;
 }
 
 }  // namespace umma

@@ -9,7 +9,7 @@
 #include <vector>
 
 #include "../../include/mh3d_unet.h"
-#include "umma_conv.cuh"
+#include "umma_launch.h"
 #include "unet_kernels.cuh"
 
 namespace mh3d {
@@ -27,16 +27,6 @@ bool tiles_disabled()
 }
 int tile_n(int n) { return n <= 16 ? 16 : (n <= 32 ? 32 : 64); }
 unsigned blocks_for(long long n, int t) { return (unsigned)((n + t - 1) / t); }
-
-// Weights of one convolution in the tcgen05 kernel's B-operand layout
-// ([27][c8p][np][8] bfloat16, umma_conv.cuh); w null: that kernel is not
-// used for it.
-struct UmmaW {
-    __nv_bfloat16* w = nullptr;
-    __nv_bfloat16* wp = nullptr;   // paired-tap layout (sources of at most 8 channels), or null
-    int c8p = 0, np = 0;
-    int sgn = 1;                   // -1: the input-gradient (flipped) operand
-};
 
 // FP32 workspace of the split-K partial sums of the gather kernel (owned
 // by the network).
@@ -97,6 +87,8 @@ struct Net {
     size_t wpart_n = 0, bpart_n = 0;
     int lblocks = 0;
     bool weights_ready = false;
+    PrepJob* jobs = nullptr;         // operand layouts (k_prep_all)
+    int njobs = 0, prep_blocks = 0;
     std::string err;
 };
 
@@ -135,34 +127,12 @@ ConvSrc src_of(const __nv_bfloat16* a, int D, int H, int W, int C, const __nv_bf
     return s;
 }
 
-int num_sms()
-{
-    static int v = -1;
-    if (v < 0) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v < 1) v = 1;
-    }
-    return v;
-}
-
-int smem_optin()
-{
-    static int v = -1;
-    if (v < 0) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) v = 48 * 1024;
-    }
-    return v;
-}
-
-// The halo-tiled kernel when its shared memory fits; false otherwise.
-template <int C, int BN, class OutT>
+// The one-channel kernel when its shared memory fits; false otherwise.
+template <int BN, class OutT>
 bool tile_conv(const ConvSrc& s, const __nv_bfloat16* Wt, int Kpad, int Npad, int N, const float* bias, int relu,
                const float* oscale, OutT* out, cudaStream_t st, cudaError_t* err)
 {
-    const size_t smem = tile_smem<C, BN>(Kpad);
+    const size_t smem = tile_smem<BN>(Kpad);
     if (smem > (size_t)smem_optin()) return false;
     // the attribute belongs to the current device: set once per device
     static bool attr_dev[64] = {};
@@ -173,7 +143,7 @@ bool tile_conv(const ConvSrc& s, const __nv_bfloat16* Wt, int Kpad, int Npad, in
         return true;
     }
     if (!attr_dev[dev] && smem > 48 * 1024) {
-        if ((*err = cudaFuncSetAttribute(k_conv_tile<C, BN, OutT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        if ((*err = cudaFuncSetAttribute(k_conv_tile<BN, OutT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          smem_optin())) != cudaSuccess)
             return true;
         attr_dev[dev] = true;
@@ -182,7 +152,7 @@ bool tile_conv(const ConvSrc& s, const __nv_bfloat16* Wt, int Kpad, int Npad, in
     static size_t occ_smem = 0;
     static int occ = 0;
     if (occ_smem != smem) {
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_conv_tile<C, BN, OutT>, kThreads, smem) !=
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_conv_tile<BN, OutT>, kThreads, smem) !=
             cudaSuccess)
             occ = 1;
         occ = std::max(occ, 1);
@@ -190,27 +160,78 @@ bool tile_conv(const ConvSrc& s, const __nv_bfloat16* Wt, int Kpad, int Npad, in
     }
     const int tiles = ((s.W + kTX - 1) / kTX) * ((s.H + kTY - 1) / kTY) * ((s.D + kTZ - 1) / kTZ);
     const int grid = std::min(tiles, num_sms() * occ);
-    k_conv_tile<C, BN, OutT><<<dim3((unsigned)grid, (unsigned)(Npad / BN)), kThreads, smem, st>>>(
+    k_conv_tile<BN, OutT><<<dim3((unsigned)grid, (unsigned)(Npad / BN)), kThreads, smem, st>>>(
+        s, Wt, Kpad, Npad, N, bias, relu, oscale, out, tiles);
+    *err = cudaGetLastError();
+    return true;
+}
+
+// The halo kernel with the weights in shared memory; false where they do not
+// fit.  BN: outputs per CTA.
+template <int C, int BN, class OutT>
+bool halo_conv(const ConvSrc& s, const __nv_bfloat16* Wt, int Kpad, int Npad, int N, const float* bias, int relu,
+               const float* oscale, OutT* out, cudaStream_t st, cudaError_t* err)
+{
+    const size_t smem = conv_halo_smem<C, BN>(Kpad);
+    if (smem > (size_t)smem_optin()) return false;
+    // resident CTAs per SM, with the attribute set, once per device (the
+    // attribute belongs to the current device; Kpad follows from C)
+    static int occ_dev[64] = {};
+    int dev = 0;
+    if ((*err = cudaGetDevice(&dev)) != cudaSuccess) return true;
+    if (dev < 0 || dev >= 64) {
+        *err = cudaErrorInvalidDevice;
+        return true;
+    }
+    if (!occ_dev[dev]) {
+        auto* fn = k_conv_halo<C, BN, OutT>;
+        if ((*err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess ||
+            (*err = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100)) != cudaSuccess)
+            return true;
+        int occ = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kThreads, smem) != cudaSuccess) occ = 1;
+        occ_dev[dev] = std::max(occ, 1);
+    }
+    const int tiles = ((s.W + kTX - 1) / kTX) * ((s.H + 7) / 8) * ((s.D + kTZ - 1) / kTZ);
+    const int ny = Npad / BN, grid = std::min(tiles, std::max(1, num_sms() * occ_dev[dev] / ny));
+    k_conv_halo<C, BN, OutT><<<dim3((unsigned)grid, (unsigned)ny), kThreads, smem, st>>>(
         s, Wt, Kpad, Npad, N, bias, relu, oscale, out, tiles);
     *err = cudaGetLastError();
     return true;
 }
 
 template <int C, class OutT>
-bool tile_conv_n(const ConvSrc& s, const __nv_bfloat16* Wt, int Kpad, int Npad, int N, const float* bias, int relu,
+bool halo_conv_n(const ConvSrc& s, const __nv_bfloat16* Wt, int Kpad, int Npad, int N, const float* bias, int relu,
                  const float* oscale, OutT* out, cudaStream_t st, cudaError_t* err)
 {
-    // output tiles of tile_n(N) columns; 32 outputs whose weights do not fit
-    // in shared memory (64 input channels: 27 x 64 weight rows) take two
-    // tiles of 16 (upsampled 64 -> 32 at 64x64x32: 228 us, 250 us on the
-    // gather kernel).  For 64 outputs, narrower tiles lose to the split-K
-    // gather kernel (64 -> 64 at 32x32x16: 79 against 62 us), which takes them.
     const int bn = tile_n(N);
-    if (bn == 32 && tile_smem<C, 32>(Kpad) > (size_t)smem_optin())
-        return tile_conv<C, 16>(s, Wt, Kpad, Npad, N, bias, relu, oscale, out, st, err);
-    if (bn == 16) return tile_conv<C, 16>(s, Wt, Kpad, Npad, N, bias, relu, oscale, out, st, err);
-    if (bn == 32) return tile_conv<C, 32>(s, Wt, Kpad, Npad, N, bias, relu, oscale, out, st, err);
-    return tile_conv<C, 64>(s, Wt, Kpad, Npad, N, bias, relu, oscale, out, st, err);
+    if (bn == 16) return halo_conv<C, 16>(s, Wt, Kpad, Npad, N, bias, relu, oscale, out, st, err);
+    // 64 outputs in one CTA where their weights fit, else two of 32
+    if constexpr (C <= 32) {
+        if (bn == 64 && halo_conv<C, 64>(s, Wt, Kpad, Npad, N, bias, relu, oscale, out, st, err)) return true;
+    }
+    return halo_conv<C, 32>(s, Wt, Kpad, Npad, N, bias, relu, oscale, out, st, err);
+}
+
+// The streaming form: split K in groups of `split` k16 steps (0: one sum).
+template <int C, class OutT>
+cudaError_t stream_conv(const ConvSrc& s, const __nv_bfloat16* Wt, int Npad, int N, const float* bias, int relu,
+                        const float* oscale, OutT* out, int split, cudaStream_t st)
+{
+    constexpr size_t smem = conv_stream_smem<C>();
+    static bool attr_dev[64] = {};   // the attribute belongs to the current device: set once per device
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    if (!attr_dev[dev]) {
+        const cudaError_t e =
+            cudaFuncSetAttribute(k_conv_stream<C, OutT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        attr_dev[dev] = true;
+    }
+    const int tiles = ((s.W + kTX - 1) / kTX) * ((s.H + kTY - 1) / kTY) * ((s.D + kTZ - 1) / kTZ);
+    k_conv_stream<C, OutT><<<dim3((unsigned)tiles, (unsigned)(Npad / kStreamBN)), kThreads, smem, st>>>(
+        s, Wt, Npad, N, bias, relu, oscale, out, split);
+    return cudaGetLastError();
 }
 
 // ---- the tcgen05 convolution (umma_conv.cuh) --------------------------------
@@ -246,138 +267,7 @@ int umma_mode()
     return 1;
 }
 bool umma_enabled() { return umma_mode() != 0; }
-bool umma_pair();
 bool umma_prefers(const ConvSrc& s) { return umma_mode() == 2 || (s.W >= 96 && (!s.f32 || umma_pair())); }
-
-template <int C8P, int NP, int NB, int R, class OutT>
-cudaError_t launch_umma_t(const ConvSrc& s, const __nv_bfloat16* Wu, int N, const float* bias, int relu,
-                          const float* oscale, OutT* out, int* status, cudaStream_t st,
-                          const __nv_bfloat16* Wpair = nullptr)
-{
-    using G = umma::Geom<C8P, NP, NB, R>;
-    auto* fn = umma::k_conv_umma<C8P, NP, NB, R, OutT>;
-    const size_t smem = G::smem();
-    if (smem > (size_t)smem_optin()) return cudaErrorInvalidValue;
-    // resident CTAs per SM, with the attributes set, once per device (the
-    // attributes belong to the current device)
-    constexpr int kDevs = 64;
-    static int occ_dev[kDevs] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevs) return cudaErrorInvalidDevice;
-    int& occ = occ_dev[dev];
-    if (occ == 0) {
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        // the whole carveout to shared memory, so that several CTAs fit
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-        if (e != cudaSuccess) return e;
-        // resident CTAs per SM from the shared memory (each CTA also reserves
-        // 1 KB), the registers and the threads; every resident CTA holds
-        // G::kCols of the SM's 512 TMEM columns
-        int smem_sm = 0, regs_sm = 0;
-        cudaFuncAttributes fa{};
-        if (cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&regs_sm, cudaDevAttrMaxRegistersPerMultiprocessor, dev) != cudaSuccess ||
-            cudaFuncGetAttributes(&fa, fn) != cudaSuccess)
-            return cudaErrorInvalidValue;
-        const int by_smem = smem_sm / (int)(smem + fa.sharedSizeBytes + 1024);
-        const int by_regs = regs_sm / std::max(1, fa.numRegs * umma::kT);
-        occ = std::max(1, std::min(std::min(by_smem, by_regs), std::min(2048 / umma::kT, 512 / G::kCols)));
-    }
-    const long long tiles = (long long)((s.W + umma::kM - 1) / umma::kM) * ((s.H + R - 1) / R) * s.D;
-    if (tiles > (1LL << 30)) return cudaErrorInvalidValue;
-    const int grid = (int)std::min<long long>(tiles, (long long)num_sms() * occ);
-    fn<<<grid, umma::kT, smem, st>>>(s, Wu, N, bias, relu, oscale, out, (int)tiles, status, Wpair);
-    return cudaGetLastError();
-}
-
-// The warp-specialised form (umma_conv.cuh: producer, MMA and epilogue
-// warps, one persistent CTA per SM, NS halo slots): MH3D_UMMA_WS=1.
-bool umma_ws()
-{
-    const char* e = std::getenv("MH3D_UMMA_WS");
-    return e && e[0] == '1';
-}
-
-template <int C8P, int NP, int NS, class OutT>
-cudaError_t launch_umma_ws_t(const ConvSrc& s, const __nv_bfloat16* Wu, int N, const float* bias, int relu,
-                             const float* oscale, OutT* out, int* status, cudaStream_t st)
-{
-    using G = umma::GeomWs<C8P, NP, NS>;
-    auto* fn = umma::k_conv_umma_ws<C8P, NP, NS, OutT>;
-    const size_t smem = G::smem();
-    constexpr int kDevs = 64;
-    static bool attr_dev[kDevs] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevs) return cudaErrorInvalidDevice;
-    if (!attr_dev[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr_dev[dev] = true;
-    }
-    const long long tiles = (long long)((s.W + umma::kM - 1) / umma::kM) * s.H * s.D;
-    if (tiles > (1LL << 30)) return cudaErrorInvalidValue;
-    const int grid = (int)std::min<long long>(tiles, (long long)num_sms());   // one CTA per SM
-    fn<<<grid, umma::kWsT, smem, st>>>(s, Wu, N, bias, relu, oscale, out, (int)tiles, status);
-    return cudaGetLastError();
-}
-
-// The deepest halo ring that fits (4, 3 or 2 slots); false if none does.
-template <int C8P, int NP, class OutT>
-bool launch_umma_ws(const ConvSrc& s, const __nv_bfloat16* Wu, int N, const float* bias, int relu,
-                    const float* oscale, OutT* out, int* status, cudaStream_t st, cudaError_t* err)
-{
-    const size_t lim = (size_t)smem_optin();
-    if (umma::GeomWs<C8P, NP, 4>::smem() <= lim)
-        *err = launch_umma_ws_t<C8P, NP, 4>(s, Wu, N, bias, relu, oscale, out, status, st);
-    else if (umma::GeomWs<C8P, NP, 3>::smem() <= lim)
-        *err = launch_umma_ws_t<C8P, NP, 3>(s, Wu, N, bias, relu, oscale, out, status, st);
-    else if (umma::GeomWs<C8P, NP, 2>::smem() <= lim)
-        *err = launch_umma_ws_t<C8P, NP, 2>(s, Wu, N, bias, relu, oscale, out, status, st);
-    else
-        return false;
-    return true;
-}
-
-// Paired taps for sources of at most 8 channels (MH3D_UMMA_PAIR=0: off).
-bool umma_pair()
-{
-    const char* e = std::getenv("MH3D_UMMA_PAIR");
-    return !(e && e[0] == '0');
-}
-
-// Output rows per tile of the tcgen05 kernel (MH3D_UMMA_ROWS = 1, 2 or 4).
-int umma_rows()
-{
-    const char* e = std::getenv("MH3D_UMMA_ROWS");
-    if (e && (e[0] == '1' || e[0] == '2' || e[0] == '4')) return e[0] - '0';
-    return 2;
-}
-
-// One halo buffer and accumulator per CTA, several CTAs per SM (the
-// default), or two per CTA with the next tile staged during this tile's
-// MMAs (MH3D_UMMA_NB=2, where it fits).  Measured at 128x128x64 (network
-// forward, channels (8, 16, 32)): 0.576 ms with one, 0.847 ms with two
-// (half the resident CTAs).
-template <int C8P, int NP, class OutT>
-cudaError_t launch_umma_nb(const ConvSrc& s, const UmmaW& u, int N, const float* bias, int relu, const float* oscale,
-                           OutT* out, int* status, cudaStream_t st)
-{
-    if (umma_ws()) {
-        cudaError_t err = cudaSuccess;
-        if (launch_umma_ws<C8P, NP>(s, u.w, N, bias, relu, oscale, out, status, st, &err)) return err;
-    }
-    const char* e = std::getenv("MH3D_UMMA_NB");
-    const bool two = e && e[0] == '2';
-    if (two && umma::Geom<C8P, NP, 2>::smem() <= (size_t)smem_optin())
-        return launch_umma_t<C8P, NP, 2, 1>(s, u.w, N, bias, relu, oscale, out, status, st);
-    const int R = umma_rows();
-    const __nv_bfloat16* wp = umma_pair() ? u.wp : nullptr;
-    if (R == 4 && umma::Geom<C8P, NP, 1, 4>::smem() <= (size_t)smem_optin())
-        return launch_umma_t<C8P, NP, 1, 4>(s, u.w, N, bias, relu, oscale, out, status, st, wp);
-    if (R >= 2 && umma::Geom<C8P, NP, 1, 2>::smem() <= (size_t)smem_optin())
-        return launch_umma_t<C8P, NP, 1, 2>(s, u.w, N, bias, relu, oscale, out, status, st, wp);
-    return launch_umma_t<C8P, NP, 1, 1>(s, u.w, N, bias, relu, oscale, out, status, st, wp);
-}
 
 template <int C8P, class OutT>
 cudaError_t launch_umma_np(const ConvSrc& s, const UmmaW& u, int N, const float* bias, int relu, const float* oscale,
@@ -412,12 +302,7 @@ cudaError_t prep_umma(const __nv_bfloat16* Wt, int Npad, int Cs, bool f32, int N
     u.c8p = umma_c8p(Cs, f32);
     u.np = umma_np(N);
     if (!u.c8p || !u.np || !u.w) return cudaSuccess;
-    const int total = 27 * u.c8p * u.np * 8;
-    umma::k_prep_umma<<<blocks_for(total, 256), 256, 0, st>>>(Wt, Npad, Cs, N, u.c8p, u.np, u.w);
-    if (u.wp) {
-        const int tp = 9 * 2 * 2 * u.np * 8;
-        umma::k_prep_umma_pair<<<blocks_for(tp, 256), 256, 0, st>>>(Wt, Npad, Cs, N, u.np, u.sgn, u.wp);
-    }
+    launch_prep_umma(Wt, Npad, Cs, N, u, st);
     return cudaGetLastError();
 }
 size_t umma_elems(int Cs, bool f32, int N)
@@ -462,25 +347,44 @@ cudaError_t launch_conv(const ConvSrc& s, const __nv_bfloat16* Wt, int Kpad, int
 {
     cudaError_t e = cudaSuccess;
     if (umma_takes(s, uw, N)) return launch_umma(s, *uw, N, bias, relu, oscale, out, status, st);
-    bool done = false;
-    if (!tiles_disabled()) {
-        if (s.C == 1)
-            done = tile_conv_n<1>(s, Wt, Kpad, Npad, N, bias, relu, oscale, out, st, &e);
-        else if (s.C == 8 && !s.f32)
-            done = tile_conv_n<8>(s, Wt, Kpad, Npad, N, bias, relu, oscale, out, st, &e);
-        else if (s.C == 16 && !s.f32)
-            done = tile_conv_n<16>(s, Wt, Kpad, Npad, N, bias, relu, oscale, out, st, &e);
-        else if (s.C == 32 && !s.f32)
-            done = tile_conv_n<32>(s, Wt, Kpad, Npad, N, bias, relu, oscale, out, st, &e);
-        else if (s.C == 64 && !s.f32)
-            done = tile_conv_n<64>(s, Wt, Kpad, Npad, N, bias, relu, oscale, out, st, &e);
-    }
-    if (done) return e;
     const long long V = (long long)s.D * s.H * s.W;
     const int bn = tile_n(N);
-    int S = ws ? splitk_parts(V, Npad, bn, Kpad) : 1;
+    const int steps = Kpad / kBK;
+    if (!tiles_disabled() && s.C == 1) {
+        bool done = false;
+        if (bn == 16) done = tile_conv<16>(s, Wt, Kpad, Npad, N, bias, relu, oscale, out, st, &e);
+        else if (bn == 32) done = tile_conv<32>(s, Wt, Kpad, Npad, N, bias, relu, oscale, out, st, &e);
+        else done = tile_conv<64>(s, Wt, Kpad, Npad, N, bias, relu, oscale, out, st, &e);
+        if (done) return e;
+    }
+    const bool tiled = !tiles_disabled() && !s.f32 && V < (1LL << 30);
+    if (tiled && s.C <= 32) {
+        bool done = false;
+        if (s.C == 8) done = halo_conv_n<8>(s, Wt, Kpad, Npad, N, bias, relu, oscale, out, st, &e);
+        else if (s.C == 16) done = halo_conv_n<16>(s, Wt, Kpad, Npad, N, bias, relu, oscale, out, st, &e);
+        else if (s.C == 32) done = halo_conv_n<32>(s, Wt, Kpad, Npad, N, bias, relu, oscale, out, st, &e);
+        if (done) return e;
+    }
+    // splits of the K loop: those of the gather kernel wherever it would run
+    // (64 channels with up to 32 outputs have always been summed unsplit)
+    int S = ws && !(s.C == 64 && N <= 32 && !tiles_disabled()) ? splitk_parts(V, Npad, bn, Kpad) : 1;
     if (S > 1 && (size_t)S * V * N > ws->cap) S = 1;
-    const int steps = Kpad / kBK, kl = (steps + S - 1) / S * kBK;
+    if (tiled && (s.C == 64 || s.C == 128)) {
+        // 64 channels on a volume that gives every SM a block: the weights
+        // stay in shared memory; else they stream (upsampled 64 -> 32 at
+        // 64x64x32: 228 us on two 16-output tiles before; 64 -> 64 at
+        // 32x32x16 and 128 -> 128 at 16x16x8: 50 us each on split-K gathers)
+        const long long blocks = (long long)((s.W + 7) / 8) * ((s.H + 7) / 8) * ((s.D + 3) / 4) * (Npad / std::min(bn, 32));
+        if (s.C == 64 && S == 1 && (blocks >= num_sms() || bn == 16)) {
+            if (halo_conv_n<64>(s, Wt, Kpad, Npad, N, bias, relu, oscale, out, st, &e)) return e;
+        }
+        if (bn >= kStreamBN) {
+            const int split = S > 1 ? (steps + S - 1) / S * (kBK / 16) : 0;
+            if (s.C == 64) return stream_conv<64>(s, Wt, Npad, N, bias, relu, oscale, out, split, st);
+            return stream_conv<128>(s, Wt, Npad, N, bias, relu, oscale, out, split, st);
+        }
+    }
+    const int kl = (steps + S - 1) / S * kBK;
     float* part = S > 1 ? ws->p : nullptr;
     dim3 grid(blocks_for(V, kBM), (unsigned)(Npad / bn), (unsigned)S);
     if (bn == 16)
@@ -590,18 +494,51 @@ namespace {
         }                                                                                         \
     } while (0)
 
-mh3d_status prep_weights(Net& n, cudaStream_t st)
+// The operand matrices of every layer (device job table: n.jobs).
+void build_jobs(Net& n, std::vector<PrepJob>& jobs)
 {
+    int block = 0;
+    auto add = [&](PrepJob j, int total, __nv_bfloat16* dst) {
+        if (!dst || total <= 0) return;
+        j.total = total;
+        j.dst = dst;
+        j.block0 = block;
+        block += (int)blocks_for(total, 256);
+        jobs.push_back(j);
+    };
     for (int i = 0; i < n.nlayers; ++i) {
         Layer& l = n.L[i];
-        k_prep_weights<<<blocks_for((long long)l.Kf * l.Nf, 256), 256, 0, st>>>(n.theta + l.woff, l.cin, l.cout,
-                                                                                l.Kf, l.Nf, 0, l.Wf);
-        k_prep_weights<<<blocks_for((long long)l.Kb * l.Nb, 256), 256, 0, st>>>(n.theta + l.woff, l.cin, l.cout,
-                                                                                l.Kb, l.Nb, 1, l.Wb);
-        const bool f32in = &l == &n.L[0];   // the network input: one FP32 channel
-        UN_CK(n, prep_umma(l.Wf, l.Nf, l.cin, f32in, l.cout, l.uf, st));
-        UN_CK(n, prep_umma(l.Wb, l.Nb, l.cout, false, l.cin, l.ub, st));
+        for (int t = 0; t < 2; ++t) {   // forward, input gradient
+            UmmaW& u = t ? l.ub : l.uf;
+            PrepJob j{};
+            j.transpose = t;
+            j.cin = l.cin;
+            j.cout = l.cout;
+            j.woff = l.woff;
+            j.Cs = t ? l.cout : l.cin;
+            j.N = t ? l.cin : l.cout;
+            j.K = 27 * j.Cs;
+            j.Npad = t ? l.Nb : l.Nf;
+            add(j, (t ? l.Kb : l.Kf) * j.Npad, t ? l.Wb : l.Wf);
+            u.c8p = umma_c8p(j.Cs, t == 0 && i == 0);   // layer 0: one FP32 channel
+            u.np = umma_np(j.N);
+            if (!u.c8p || !u.np || !u.w) continue;
+            j.C8P = u.c8p;
+            j.NP = u.np;
+            j.sgn = u.sgn;
+            j.kind = 1;
+            add(j, 27 * u.c8p * u.np * 8, u.w);
+            j.kind = 2;
+            add(j, 9 * 2 * 2 * u.np * 8, u.wp);
+        }
     }
+    n.prep_blocks = block;
+    n.njobs = (int)jobs.size();
+}
+
+mh3d_status prep_weights(Net& n, cudaStream_t st)
+{
+    k_prep_all<<<n.prep_blocks, 256, 0, st>>>(n.jobs, n.njobs, n.theta);
     UN_CK(n, cudaGetLastError());
     n.weights_ready = true;
     return MH3D_OK;
@@ -626,6 +563,10 @@ ConvSrc src_at(const Net& n, const __nv_bfloat16* a, int l, int C, const __nv_bf
     return src_of(a, n.dims[l][0], n.dims[l][1], n.dims[l][2], C, skip, up);
 }
 
+// Whether a level's volume takes the 8-channel elementwise kernels.
+bool vec8(long long V, int C) { return C % 8 == 0 && V * (C / 8) < (1LL << 30); }
+Vol8 vol8(const Net& n, int l, int C) { return Vol8(n.dims[l][0], n.dims[l][1], n.dims[l][2], C); }
+
 // iscale / oscale: device scalars multiplying the input and the output
 // (null: 1).
 mh3d_status forward_pass(Net& n, const float* in, cudaStream_t st, const float* iscale = nullptr,
@@ -645,9 +586,14 @@ mh3d_status forward_pass(Net& n, const float* in, cudaStream_t st, const float* 
         const ConvSrc x = l == 0 ? s0 : src_at(n, n.p[l - 1], l, n.ch[l - 1]);
         UN_CK(n, fwd(n, 2 * l, x, 1, n.ea[l], st));
         UN_CK(n, fwd(n, 2 * l + 1, src_at(n, n.ea[l], l, n.ch[l]), 1, n.e[l], st));
-        if (l + 1 < Lv)
-            k_pool<<<blocks_for(n.V[l + 1] * n.ch[l], 256), 256, 0, st>>>(n.e[l], n.dims[l][0], n.dims[l][1],
-                                                                          n.dims[l][2], n.ch[l], n.p[l]);
+        if (l + 1 < Lv) {
+            if (vec8(n.V[l], n.ch[l]))
+                k_sum8_v8<<<blocks_for(n.V[l + 1] * n.ch[l] / 8, 256), 256, 0, st>>>(
+                    (const uint4*)n.e[l], vol8(n, l + 1, n.ch[l]), 0.125f, (uint4*)n.p[l]);
+            else
+                k_pool<<<blocks_for(n.V[l + 1] * n.ch[l], 256), 256, 0, st>>>(n.e[l], n.dims[l][0], n.dims[l][1],
+                                                                              n.dims[l][2], n.ch[l], n.p[l]);
+        }
     }
     for (int l = Lv - 2; l >= 0; --l) {
         const __nv_bfloat16* below = l + 1 == Lv - 1 ? n.e[l + 1] : n.d[l + 1];
@@ -669,7 +615,11 @@ mh3d_status back_layer(Net& n, int li, const ConvSrc& s, const __nv_bfloat16* g,
     const Layer& l = n.L[li];
     const long long V = (long long)s.D * s.H * s.W;
     if (y) {
-        k_relu_grad<<<blocks_for(V * l.cout, 256), 256, 0, st>>>(n.scratch, g, y, V * l.cout);
+        if (V * l.cout % 8 == 0)
+            k_relu_grad_v8<<<blocks_for(V * l.cout / 8, 256), 256, 0, st>>>((uint4*)n.scratch, (const uint4*)g,
+                                                                           (const uint4*)y, V * l.cout / 8);
+        else
+            k_relu_grad<<<blocks_for(V * l.cout, 256), 256, 0, st>>>(n.scratch, g, y, V * l.cout);
         g = n.scratch;
     }
     UN_CK(n, launch_wgrad(s, g, l.cout, n.wpart, n.bpart, n.grad + l.woff, n.grad + l.boff, st));
@@ -696,8 +646,12 @@ mh3d_status backward_pass(Net& n, cudaStream_t st)
         UN_BACK(li + 1, src_at(n, n.u[l], l, n.ch[l], n.e[l]), n.gd[l], n.d[l], n.gs[l]);
         UN_BACK(li, src_at(n, below, l, n.ch[l + 1], nullptr, 1), n.gs[l], n.u[l], n.gup[l]);
         const int* dn = n.dims[l + 1];
-        k_up_grad<<<blocks_for(n.V[l + 1] * n.ch[l + 1], 256), 256, 0, st>>>(n.gup[l], dn[0], dn[1], dn[2],
-                                                                              n.ch[l + 1], n.gd[l + 1]);
+        if (vec8(n.V[l], n.ch[l + 1]))
+            k_sum8_v8<<<blocks_for(n.V[l + 1] * n.ch[l + 1] / 8, 256), 256, 0, st>>>(
+                (const uint4*)n.gup[l], vol8(n, l + 1, n.ch[l + 1]), 1.f, (uint4*)n.gd[l + 1]);
+        else
+            k_up_grad<<<blocks_for(n.V[l + 1] * n.ch[l + 1], 256), 256, 0, st>>>(n.gup[l], dn[0], dn[1], dn[2],
+                                                                                  n.ch[l + 1], n.gd[l + 1]);
     }
     ConvSrc s0;
     s0.f32 = n.in;
@@ -713,8 +667,13 @@ mh3d_status backward_pass(Net& n, cudaStream_t st)
         UN_BACK(2 * l, x, n.gea[l], n.ea[l], l == 0 ? nullptr : n.gp[l - 1]);
         if (l > 0) {
             const int* dm = n.dims[l - 1];
-            k_pool_grad_add<<<blocks_for(n.V[l - 1] * n.ch[l - 1], 256), 256, 0, st>>>(
-                n.gs[l - 1], n.gp[l - 1], dm[0], dm[1], dm[2], n.ch[l - 1], n.ge[l - 1]);
+            if (vec8(n.V[l - 1], n.ch[l - 1]))
+                k_pool_grad_add_v8<<<blocks_for(n.V[l - 1] * n.ch[l - 1] / 8, 256), 256, 0, st>>>(
+                    (const uint4*)n.gs[l - 1], (const uint4*)n.gp[l - 1], vol8(n, l - 1, n.ch[l - 1]),
+                    (uint4*)n.ge[l - 1]);
+            else
+                k_pool_grad_add<<<blocks_for(n.V[l - 1] * n.ch[l - 1], 256), 256, 0, st>>>(
+                    n.gs[l - 1], n.gp[l - 1], dm[0], dm[1], dm[2], n.ch[l - 1], n.ge[l - 1]);
         }
     }
 #undef UN_BACK
@@ -722,7 +681,7 @@ mh3d_status backward_pass(Net& n, cudaStream_t st)
     return MH3D_OK;
 }
 
-constexpr int kScaleBlocks = 304;   // partial sums of the RMS (2 per SM)
+constexpr int kScaleBlocks = kScaleMax;   // partial sums of the RMS (2 per SM)
 
 // (cin, cout) of layer i of a network with channels ch[0 .. levels - 1].
 void layer_io(int levels, const int* ch, int i, int* cin, int* cout)
@@ -865,6 +824,11 @@ mh3d_status mh3d_unet_create_levels(int nx, int ny, int nz, int levels, const in
         A(&n->skws.p, skn);
         n->skws.cap = skn;
     }
+    std::vector<PrepJob> jobs;
+    if (ok) build_jobs(*n, jobs);
+    A(&n->jobs, jobs.size());
+    if (ok && cudaMemcpy(n->jobs, jobs.data(), sizeof(PrepJob) * jobs.size(), cudaMemcpyHostToDevice) != cudaSuccess)
+        ok = false;
     A(&n->lpart, (size_t)n->lblocks);
     A(&n->spart, (size_t)kScaleBlocks);
     A(&n->scales, 4);
@@ -970,7 +934,7 @@ static void launch_scales(mh3d_unet n, const float* in, float gain, cudaStream_t
 {
     using namespace mh3d::unet;
     k_sumsq_part<<<kScaleBlocks, kThreads, 0, st>>>(in, n->V[0], n->spart);
-    k_scales<<<1, 32, 0, st>>>(n->spart, kScaleBlocks, n->V[0], gain, n->scales);
+    k_scales<<<1, 320, 0, st>>>(n->spart, kScaleBlocks, n->V[0], gain, n->scales);
 }
 
 mh3d_status mh3d_unet_loss_grad(mh3d_unet n, const float* in, const float* target, float* grad, double* loss,

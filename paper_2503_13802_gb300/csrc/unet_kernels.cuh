@@ -22,6 +22,8 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include "fastdiv.h"
+
 namespace mh3d {
 namespace unet {
 
@@ -266,37 +268,25 @@ __global__ void __launch_bounds__(kThreads) k_conv(ConvSrc src, const __nv_bfloa
 }
 
 // ---------------------------------------------------------------------------
-// Tiled convolution: one CTA per 8 x 4 x 4 output block.  The block's input
-// halo (10 x 6 x 6 voxels, all C channels) and the whole weight matrix are
-// staged in shared memory once; the GEMM operand for tap t is then the halo
-// shifted by t, read by ldmatrix with one row address per lane, so each
-// input voxel leaves global memory about 2.8 times per block instead of 27.
-// Halo voxels are padded to C + 8 elements (16 bytes) so that the eight
-// rows an ldmatrix reads fall in distinct banks.  C = 1 (the network input,
-// or a one-channel gradient) builds the 128 x 32 operand explicitly instead.
+// One-channel source (the network input, or a one-channel gradient), on
+// 8 x 4 x 4 output blocks: the block's input halo (10 x 6 x 6 voxels) and
+// the weight matrix are staged in shared memory, and the 128 x 32 operand
+// (27 taps, 5 zeros) is built from the halo explicitly.
 constexpr int kTX = 8, kTY = 4, kTZ = 4;
 constexpr int kHX = kTX + 2, kHY = kTY + 2, kHZ = kTZ + 2, kHV = kHX * kHY * kHZ;
 
-template <int C>
-__host__ __device__ constexpr int halo_stride() { return C == 1 ? 1 : C + 8; }
-
-// Shared-memory bytes of k_conv_tile<C, BN> for a weight matrix of Kpad rows
-// (weights, two halo buffers, a zero row, and for C == 1 the explicit
-// operand tile).
-template <int C, int BN>
+// Shared-memory bytes of k_conv_tile<BN> for a weight matrix of Kpad rows
+// (weights, two halo buffers and the operand tile).
+template <int BN>
 constexpr size_t tile_smem(int Kpad)
 {
-    return sizeof(__nv_bfloat16) * ((size_t)Kpad * (BN + 8) + 2 * (((kHV * halo_stride<C>() + 7) / 8) * 8) + 8 +
-                                    (C == 1 ? kBM * (kBK + 8) : 0));
+    return sizeof(__nv_bfloat16) * ((size_t)Kpad * (BN + 8) + 2 * (((kHV + 7) / 8) * 8) + kBM * (kBK + 8));
 }
 
-// Halo elements a thread carries between tiles: uint4 (8 channels) for
-// C >= 8, one value for C == 1.
-template <int C>
+// Halo values a thread carries between tiles.
 struct HaloRegs {
-    static constexpr int kItems = (C == 1) ? kHV : kHV * (C / 8);
-    static constexpr int kPer = (kItems + kThreads - 1) / kThreads;
-    uint4 v[kPer];
+    static constexpr int kPer = (kHV + kThreads - 1) / kThreads;
+    float v[kPer];
 };
 
 __device__ __forceinline__ void tile_origin(const ConvSrc& s, int t, int& x0, int& y0, int& z0)
@@ -310,65 +300,38 @@ __device__ __forceinline__ void tile_origin(const ConvSrc& s, int t, int& x0, in
 
 // Global -> registers: the halo of the tile at (x0, y0, z0), zero outside,
 // the skip addend summed and rounded as a stored sum would be.
-template <int C>
-__device__ __forceinline__ void halo_fetch(const ConvSrc& src, int x0, int y0, int z0, HaloRegs<C>& h)
+__device__ __forceinline__ void halo_fetch(const ConvSrc& src, int x0, int y0, int z0, HaloRegs& h)
 {
     const int Hs = src.up ? (src.H >> 1) : src.H, Ws = src.up ? (src.W >> 1) : src.W;
 #pragma unroll
-    for (int j = 0; j < HaloRegs<C>::kPer; ++j) {
-        const int i = threadIdx.x + j * kThreads;
-        uint4 r = make_uint4(0, 0, 0, 0);
-        if (i < HaloRegs<C>::kItems) {
-            const int hv = (C == 1) ? i : i / (C / 8), c8 = (C == 1) ? 0 : i % (C / 8);
+    for (int j = 0; j < HaloRegs::kPer; ++j) {
+        const int hv = threadIdx.x + j * kThreads;
+        float v = 0.f;
+        if (hv < kHV) {
             const int hx = hv % kHX, hy = (hv / kHX) % kHY, hz = hv / (kHX * kHY);
             const int z = z0 - 1 + hz, y = y0 - 1 + hy, x = x0 - 1 + hx;
             if (z >= 0 && z < src.D && y >= 0 && y < src.H && x >= 0 && x < src.W) {
-                const size_t vox = src.up ? ((size_t)(z >> 1) * Hs + (y >> 1)) * Ws + (x >> 1)
-                                          : ((size_t)z * src.H + y) * src.W + x;
-                if constexpr (C == 1) {
-                    float v;
-                    if (src.f32) {
-                        v = src.f32[((size_t)z * src.H + y) * src.W + x] * (src.f32_scale ? *src.f32_scale : 1.f);
-                    } else {
-                        v = bf2f(src.a[vox]);
-                        if (src.b) v = bf2f(__float2bfloat16(v + bf2f(src.b[vox])));
-                    }
-                    r.x = __float_as_uint(v);
+                if (src.f32) {
+                    v = src.f32[((size_t)z * src.H + y) * src.W + x] * (src.f32_scale ? *src.f32_scale : 1.f);
                 } else {
-                    const size_t off = vox * C + c8 * 8;
-                    r = *reinterpret_cast<const uint4*>(src.a + off);
-                    if (src.b) {
-                        const uint4 q = *reinterpret_cast<const uint4*>(src.b + off);
-                        __nv_bfloat162* pr = reinterpret_cast<__nv_bfloat162*>(&r);
-                        const __nv_bfloat162* pq = reinterpret_cast<const __nv_bfloat162*>(&q);
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const float2 u = __bfloat1622float2(pr[e]), w = __bfloat1622float2(pq[e]);
-                            pr[e] = __floats2bfloat162_rn(u.x + w.x, u.y + w.y);
-                        }
-                    }
+                    const size_t vox = src.up ? ((size_t)(z >> 1) * Hs + (y >> 1)) * Ws + (x >> 1)
+                                              : ((size_t)z * src.H + y) * src.W + x;
+                    v = bf2f(src.a[vox]);
+                    if (src.b) v = bf2f(__float2bfloat16(v + bf2f(src.b[vox])));
                 }
             }
         }
-        h.v[j] = r;
+        h.v[j] = v;
     }
 }
 
 // Registers -> one halo buffer.
-template <int C>
-__device__ __forceinline__ void halo_store(__nv_bfloat16* sH, const HaloRegs<C>& h)
+__device__ __forceinline__ void halo_store(__nv_bfloat16* sH, const HaloRegs& h)
 {
-    constexpr int CS = halo_stride<C>();
 #pragma unroll
-    for (int j = 0; j < HaloRegs<C>::kPer; ++j) {
+    for (int j = 0; j < HaloRegs::kPer; ++j) {
         const int i = threadIdx.x + j * kThreads;
-        if (i >= HaloRegs<C>::kItems) continue;
-        if constexpr (C == 1) {
-            sH[i] = __float2bfloat16(__uint_as_float(h.v[j].x));
-        } else {
-            const int hv = i / (C / 8), c8 = i % (C / 8);
-            *reinterpret_cast<uint4*>(sH + hv * CS + c8 * 8) = h.v[j];
-        }
+        if (i < kHV) sH[i] = __float2bfloat16(h.v[j]);
     }
 }
 
@@ -376,19 +339,17 @@ __device__ __forceinline__ void halo_store(__nv_bfloat16* sH, const HaloRegs<C>&
 // blocks blockIdx.x, blockIdx.x + gridDim.x, ...; while it multiplies one
 // block, the next block's halo is in flight to registers, and lands in the
 // other halo buffer afterwards.
-template <int C, int BN, class OutT>
+template <int BN, class OutT>
 __global__ void __launch_bounds__(kThreads, 2) k_conv_tile(ConvSrc src, const __nv_bfloat16* __restrict__ Wt, int Kpad,
                                                         int Npad, int N, const float* __restrict__ bias, int relu,
                                                         const float* __restrict__ oscale, OutT* __restrict__ out,
                                                         int ntiles)
 {
     extern __shared__ __align__(16) unsigned char tile_raw[];
-    constexpr int CS = halo_stride<C>();
-    constexpr int HB = ((kHV * CS + 7) / 8) * 8;
+    constexpr int HB = ((kHV + 7) / 8) * 8;
     __nv_bfloat16* sW = reinterpret_cast<__nv_bfloat16*>(tile_raw);   // [Kpad][BN + 8]
-    __nv_bfloat16* sH0 = sW + (size_t)Kpad * (BN + 8);                 // two [kHV][CS] buffers
-    __nv_bfloat16* sZ = sH0 + 2 * HB;                                  // 8 zeros
-    __nv_bfloat16* sA = sZ + 8;                                        // C == 1: [kBM][kBK + 8]
+    __nv_bfloat16* sH0 = sW + (size_t)Kpad * (BN + 8);                 // two [kHV] buffers
+    __nv_bfloat16* sA = sH0 + 2 * HB;                                  // [kBM][kBK + 8]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n0 = blockIdx.y * BN;
     const int sgn = src.flip ? -1 : 1;
@@ -399,66 +360,38 @@ __global__ void __launch_bounds__(kThreads, 2) k_conv_tile(ConvSrc src, const __
         *reinterpret_cast<uint4*>(sW + r * (BN + 8) + c * 8) =
             *reinterpret_cast<const uint4*>(Wt + (size_t)r * Npad + n0 + c * 8);
     }
-    if (threadIdx.x < 8) sZ[threadIdx.x] = __float2bfloat16(0.f);
     int tile = blockIdx.x;
     if (tile >= ntiles) return;
-    HaloRegs<C> h;
+    HaloRegs h;
     int x0, y0, z0;
     tile_origin(src, tile, x0, y0, z0);
-    halo_fetch<C>(src, x0, y0, z0, h);
-    halo_store<C>(sH0, h);
+    halo_fetch(src, x0, y0, z0, h);
+    halo_store(sH0, h);
     __syncthreads();
     int cur = 0;
-    // this thread's fragment row
-    const int m = 16 * warp + (lane & 15);
-    const int hc = ((m / (kTX * kTY) + 1) * kHY + ((m / kTX) % kTY + 1)) * kHX + (m % kTX + 1);
     for (;;) {
         const int next = tile + gridDim.x;
         int nx0 = 0, ny0 = 0, nz0 = 0;
         if (next < ntiles) {
             tile_origin(src, next, nx0, ny0, nz0);
-            halo_fetch<C>(src, nx0, ny0, nz0, h);
+            halo_fetch(src, nx0, ny0, nz0, h);
         }
         const __nv_bfloat16* sH = sH0 + cur * HB;
         float acc[BN / 8][4];
 #pragma unroll
         for (int q = 0; q < BN / 8; ++q) acc[q][0] = acc[q][1] = acc[q][2] = acc[q][3] = 0.f;
-        if constexpr (C == 1) {
-            for (int i = threadIdx.x; i < kBM * kBK; i += kThreads) {
-                const int mm = i / kBK, k = i % kBK;
-                __nv_bfloat16 v = __float2bfloat16(0.f);
-                if (k < 27) {
-                    const int tx = mm % kTX, ty = (mm / kTX) % kTY, tz = mm / (kTX * kTY);
-                    const int dz = sgn * (k / 9 - 1), dy = sgn * ((k / 3) % 3 - 1), dx = sgn * (k % 3 - 1);
-                    v = sH[((tz + 1 + dz) * kHY + (ty + 1 + dy)) * kHX + (tx + 1 + dx)];
-                }
-                sA[mm * (kBK + 8) + k] = v;
+        for (int i = threadIdx.x; i < kBM * kBK; i += kThreads) {
+            const int mm = i / kBK, k = i % kBK;
+            __nv_bfloat16 v = __float2bfloat16(0.f);
+            if (k < 27) {
+                const int tx = mm % kTX, ty = (mm / kTX) % kTY, tz = mm / (kTX * kTY);
+                const int dz = sgn * (k / 9 - 1), dy = sgn * ((k / 3) % 3 - 1), dx = sgn * (k % 3 - 1);
+                v = sH[((tz + 1 + dz) * kHY + (ty + 1 + dy)) * kHX + (tx + 1 + dx)];
             }
-            __syncthreads();
-            mma_stage<BN, false>(sA, sW, acc, warp, lane);
-        } else {
-            const int KS = Kpad / 16;
-            for (int ks = 0; ks < KS; ++ks) {
-                const int k = ks * 16 + (lane >> 4) * 8;
-                const int tap = k / C, ch = k % C;
-                const __nv_bfloat16* pa = sZ;
-                if (tap < 27) {
-                    const int dz = sgn * (tap / 9 - 1), dy = sgn * ((tap / 3) % 3 - 1), dx = sgn * (tap % 3 - 1);
-                    pa = sH + (hc + (dz * kHY + dy) * kHX + dx) * CS + ch;
-                }
-                uint32_t a[4];
-                ldsm_x4(a, pa);
-#pragma unroll
-                for (int j = 0; j < BN / 16; ++j) {
-                    uint32_t b[4];
-                    const int row = ks * 16 + (lane & 7) + ((lane >> 3) & 1) * 8;
-                    const int col = j * 16 + (lane >> 4) * 8;
-                    ldsm_x4_t(b, sW + row * (BN + 8) + col);
-                    mma_bf16(acc[2 * j], a, b[0], b[1]);
-                    mma_bf16(acc[2 * j + 1], a, b[2], b[3]);
-                }
-            }
+            sA[mm * (kBK + 8) + k] = v;
         }
+        __syncthreads();
+        mma_stage<BN, false>(sA, sW, acc, warp, lane);
 #pragma unroll
         for (int q = 0; q < BN / 8; ++q) {
 #pragma unroll
@@ -482,13 +415,388 @@ __global__ void __launch_bounds__(kThreads, 2) k_conv_tile(ConvSrc src, const __
         }
         if (next >= ntiles) break;
         // the other buffer was last read two tiles ago, before the previous barrier
-        halo_store<C>(sH0 + (cur ^ 1) * HB, h);
+        halo_store(sH0 + (cur ^ 1) * HB, h);
         __syncthreads();
         cur ^= 1;
         tile = next;
         x0 = nx0;
         y0 = ny0;
         z0 = nz0;
+    }
+}
+
+__device__ __forceinline__ void lin_cp16(void* sdst, const void* gsrc, bool in)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr(sdst)), "l"(gsrc), "r"(in ? 16u : 0u)
+                 : "memory");
+}
+
+// ---------------------------------------------------------------------------
+// Tiled convolutions for sources of 8 n channels on mma.sync: one CTA per
+// 8 x TY x 4 output block, eight warps of 32 voxels (two 16-row fragments,
+// so that a weight fragment read from shared memory serves two products).
+// The products of an output and their order are those of the kernels above
+// (k16 steps in ascending tap and channel; with `split` > 0 a new sum every
+// `split` steps, the sums added in order, as the split-K gather form does),
+// so the three give the same bits.  What bounds them: the shared-memory
+// reads of the fragments; tap offsets come from a table, and a halo unit's
+// place and address are formed once per CTA, not per block.  Measured in the
+// forward at 128x128x64, channels (16, 32, 64, 128), us a layer, against
+// tiles of 128 voxels with one fragment a warp and the split-K gather form:
+// 32 -> 32 at half resolution 70 -> 33, upsampled 64 -> 32 228 -> 53, 64 -> 64
+// at a quarter 50 -> 20, 128 -> 128 at an eighth 50 -> 33.
+//
+// k_conv_halo keeps the whole weight matrix in shared memory (C <= 64) and
+// walks blocks; k_conv_stream (C = 64 and 128 on coarse levels, a few blocks
+// per SM) streams it tap by tap.
+template <int TY>
+struct HaloGeom {
+    static constexpr int HX = kTX + 2, HY = TY + 2, HZ = kTZ + 2, HV = HX * HY * HZ, M = kTX * TY * kTZ;
+};
+
+// Shared-memory bytes of the two.
+template <int C, int BN>
+constexpr size_t conv_halo_smem(int Kpad)
+{
+    return sizeof(__nv_bfloat16) * ((size_t)Kpad * (BN + 8) + (size_t)HaloGeom<8>::HV * (C + 8) + 8) + sizeof(int) * 28;
+}
+constexpr int kStreamBN = 32;
+template <int C>
+constexpr size_t conv_stream_smem()
+{
+    return sizeof(__nv_bfloat16) * ((size_t)HaloGeom<4>::HV * (C + 8) + 3 * (size_t)C * (kStreamBN + 8)) + sizeof(int) * 28;
+}
+
+// A thread's halo units: unit i of the block is 8 channels of a halo voxel.
+// rel: element offset from the block's first voxel's; pos: hx | hy << 8 |
+// hz << 16.
+template <int C, int TY, int PER>
+struct HaloUnits {
+    using G = HaloGeom<TY>;
+    static constexpr int kItems = G::HV * (C / 8);
+    int rel[PER], pos[PER];
+    // the units first + j kThreads (j < PER)
+    __device__ __forceinline__ void init(const ConvSrc& s, int first)
+    {
+        const int Ws = s.up ? s.W >> 1 : s.W, Hs = s.up ? s.H >> 1 : s.H, sh = s.up ? 1 : 0;
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            const int i = first + j * kThreads, hv = i / (C / 8), c8 = i % (C / 8);
+            const int hx = hv % G::HX, hy = (hv / G::HX) % G::HY, hz = hv / (G::HX * G::HY);
+            pos[j] = i < kItems ? hx | hy << 8 | hz << 16 : -1;
+            // block origins are even, so halving commutes with the offset
+            rel[j] = ((((hz - 1) >> sh) * Hs + ((hy - 1) >> sh)) * Ws + ((hx - 1) >> sh)) * C + c8 * 8;
+        }
+    }
+};
+__device__ __forceinline__ uint4 add_bf16x8(uint4 r, const uint4& q)   // the skip sum, rounded as a stored sum would be
+{
+    __nv_bfloat162* pr = reinterpret_cast<__nv_bfloat162*>(&r);
+    const __nv_bfloat162* pq = reinterpret_cast<const __nv_bfloat162*>(&q);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const float2 u = __bfloat1622float2(pr[e]), w = __bfloat1622float2(pq[e]);
+        pr[e] = __floats2bfloat162_rn(u.x + w.x, u.y + w.y);
+    }
+    return r;
+}
+template <int C, int TY, int PER>
+__device__ __forceinline__ void halo_load(const ConvSrc& s, const HaloUnits<C, TY, PER>& u, int x0, int y0, int z0,
+                                          uint4 (&v)[PER])
+{
+    const int sh = s.up ? 1 : 0, Ws = s.W >> sh, Hs = s.H >> sh;
+    const long long base = (((long long)(z0 >> sh) * Hs + (y0 >> sh)) * Ws + (x0 >> sh)) * C;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        v[j] = make_uint4(0, 0, 0, 0);
+        if (u.pos[j] < 0) continue;
+        const int x = x0 - 1 + (u.pos[j] & 255), y = y0 - 1 + ((u.pos[j] >> 8) & 255), z = z0 - 1 + (u.pos[j] >> 16);
+        if ((unsigned)x >= (unsigned)s.W || (unsigned)y >= (unsigned)s.H || (unsigned)z >= (unsigned)s.D) continue;
+        v[j] = *reinterpret_cast<const uint4*>(s.a + base + u.rel[j]);
+        if (s.b) v[j] = add_bf16x8(v[j], *reinterpret_cast<const uint4*>(s.b + base + u.rel[j]));
+    }
+}
+template <int C, int PER>
+__device__ __forceinline__ void halo_put(__nv_bfloat16* sH, int first, int items, const uint4 (&v)[PER])
+{
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        const int i = first + j * kThreads;
+        if (i < items) *reinterpret_cast<uint4*>(sH + (i / (C / 8)) * (C + 8) + (i % (C / 8)) * 8) = v[j];
+    }
+}
+// Tap t's halo offset in elements (t < 27).
+template <int C, int TY>
+__device__ __forceinline__ int tap_halo(int t, int sgn)
+{
+    using G = HaloGeom<TY>;
+    const int dz = sgn * (t / 9 - 1), dy = sgn * ((t / 3) % 3 - 1), dx = sgn * (t % 3 - 1);
+    return ((dz * G::HY + dy) * G::HX + dx) * (C + 8);
+}
+
+__device__ __forceinline__ void ldsm_a(uint32_t (&r)[4], uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr));
+}
+__device__ __forceinline__ void ldsm_bt(uint32_t (&r)[4], uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr));
+}
+
+// Epilogue of a 16-row fragment set: rows 16 mt + lane / 4 (+ 8) of the
+// block, columns n0 + 8 q + 2 (lane % 4) + {0, 1}.
+template <int TY, int NT, class OutT>
+__device__ __forceinline__ void conv_store(const ConvSrc& s, const float (&acc)[NT][4], int mt, int lane, int x0, int y0,
+                                           int z0, int n0, int N, const float* __restrict__ bias, int relu, float osc,
+                                           OutT* __restrict__ out)
+{
+#pragma unroll
+    for (int hh = 0; hh < 2; ++hh) {
+        const int mm = 16 * mt + (lane >> 2) + 8 * hh;
+        const int x = x0 + mm % kTX, y = y0 + (mm / kTX) % TY, z = z0 + mm / (kTX * TY);
+        if (x >= s.W || y >= s.H || z >= s.D) continue;
+        OutT* o = out + (((long long)z * s.H + y) * s.W + x) * N;
+#pragma unroll
+        for (int q = 0; q < NT; ++q) {
+            const int n = n0 + q * 8 + 2 * (lane & 3);
+            float v[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                v[e] = (acc[q][2 * hh + e] + (bias && n + e < N ? bias[n + e] : 0.f)) * osc;
+                if (relu) v[e] = fmaxf(v[e], 0.f);
+            }
+            if constexpr (sizeof(OutT) == 2) {
+                if ((N & 1) == 0) {
+                    if (n < N) *reinterpret_cast<__nv_bfloat162*>(o + n) = __floats2bfloat162_rn(v[0], v[1]);
+                    continue;
+                }
+            }
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                if (n + e >= N) continue;
+                if constexpr (sizeof(OutT) == 2) o[n + e] = __float2bfloat16(v[e]);
+                else o[n + e] = v[e];
+            }
+        }
+    }
+}
+
+template <int TY>
+__device__ __forceinline__ void block_origin(const ConvSrc& s, int t, int& x0, int& y0, int& z0)
+{
+    const int tx = (s.W + kTX - 1) / kTX, ty = (s.H + TY - 1) / TY;
+    x0 = (t % tx) * kTX;
+    t /= tx;
+    y0 = (t % ty) * TY;
+    z0 = (t / ty) * kTZ;
+}
+
+template <int C, int BN, class OutT>
+__global__ void __launch_bounds__(kThreads, C <= 16 && BN <= 32 ? 2 : 1)
+    k_conv_halo(ConvSrc src, const __nv_bfloat16* __restrict__ Wt, int Kpad, int Npad, int N,
+                const float* __restrict__ bias, int relu, const float* __restrict__ oscale, OutT* __restrict__ out,
+                int ntiles)
+{
+    extern __shared__ __align__(16) unsigned char ch_raw[];
+    constexpr int TY = 8, CS = C + 8, NT = BN / 8, WS = BN + 8;
+    using G = HaloGeom<TY>;
+    constexpr int ITEMS = G::HV * (C / 8), PER = (ITEMS + kThreads - 1) / kThreads;
+    constexpr bool PRE = C <= 32;   // the next block's halo in registers during this block's products
+    static_assert(G::M == 32 * (kThreads / 32), "a warp per 32 voxels");
+    __nv_bfloat16* sW = reinterpret_cast<__nv_bfloat16*>(ch_raw);   // [Kpad][BN + 8]
+    __nv_bfloat16* sH = sW + (size_t)Kpad * WS;                      // [HV][C + 8]
+    __nv_bfloat16* sZ = sH + (size_t)G::HV * CS;                     // 8 zeros
+    int* toff = reinterpret_cast<int*>(sZ + 8);                      // tap offsets, bytes
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int n0 = blockIdx.y * BN;
+    const float osc = oscale ? *oscale : 1.f;
+    for (int i = threadIdx.x; i < Kpad * (BN / 8); i += kThreads) {
+        const int r = i / (BN / 8), c = i % (BN / 8);
+        *reinterpret_cast<uint4*>(sW + r * WS + c * 8) =
+            *reinterpret_cast<const uint4*>(Wt + (size_t)r * Npad + n0 + c * 8);
+    }
+    if (threadIdx.x < 8) sZ[threadIdx.x] = __float2bfloat16(0.f);
+    if (threadIdx.x < 27) toff[threadIdx.x] = 2 * tap_halo<C, TY>(threadIdx.x, src.flip ? -1 : 1);
+    if (threadIdx.x == 27) toff[27] = 0;
+    int tile = blockIdx.x;
+    if (tile >= ntiles) return;
+    HaloUnits<C, TY, PER> hu;
+    hu.init(src, threadIdx.x);
+    uint4 hv[PER];
+    int x0, y0, z0;
+    block_origin<TY>(src, tile, x0, y0, z0);
+    halo_load(src, hu, x0, y0, z0, hv);
+    // this lane's rows of the warp's two fragments
+    uint32_t abase[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int m = 32 * warp + 16 * i + (lane & 15);
+        abase[i] = smem_addr(sH + ((m / (kTX * TY) + 1) * (G::HY * G::HX) + ((m / kTX) % TY + 1) * G::HX + m % kTX + 1) * CS);
+    }
+    const uint32_t bbase = smem_addr(sW + ((lane & 7) + ((lane >> 3) & 1) * 8) * WS + (lane >> 4) * 8);
+    const uint32_t zrow = smem_addr(sZ);
+    const int kh = lane >> 4;
+    for (;;) {
+        halo_put<C>(sH, threadIdx.x, ITEMS, hv);
+        __syncthreads();
+        const int next = tile + gridDim.x;
+        int nx0 = 0, ny0 = 0, nz0 = 0;
+        if (next < ntiles) block_origin<TY>(src, next, nx0, ny0, nz0);
+        if (PRE && next < ntiles) halo_load(src, hu, nx0, ny0, nz0, hv);
+        float acc[2][NT][4];
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int q = 0; q < NT; ++q) acc[i][q][0] = acc[i][q][1] = acc[i][q][2] = acc[i][q][3] = 0.f;
+        auto step = [&](uint32_t a0, uint32_t a1, uint32_t b) {
+            uint32_t fa[2][4];
+            ldsm_a(fa[0], a0);
+            ldsm_a(fa[1], a1);
+#pragma unroll
+            for (int j = 0; j < BN / 16; ++j) {
+                uint32_t fb[4];
+                ldsm_bt(fb, b + j * 32);
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    mma_bf16(acc[i][2 * j], fa[i], fb[0], fb[1]);
+                    mma_bf16(acc[i][2 * j + 1], fa[i], fb[2], fb[3]);
+                }
+            }
+        };
+        if constexpr (C == 8) {
+            // a step holds two taps, one per lane half; the 28th is zero
+#pragma unroll 2
+            for (int ks = 0; ks < 14; ++ks) {
+                const int t = 2 * ks + kh, o = toff[t];
+                step(t < 27 ? abase[0] + o : zrow, t < 27 ? abase[1] + o : zrow, bbase + ks * 16 * WS * 2);
+            }
+        } else {
+            uint32_t b = bbase;
+#pragma unroll 3
+            for (int t = 0; t < 27; ++t) {
+                const int o = toff[t] + 16 * kh;
+#pragma unroll
+                for (int c = 0; c < C / 16; ++c, b += 16 * WS * 2) step(abase[0] + o + 32 * c, abase[1] + o + 32 * c, b);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+            conv_store<TY>(src, acc[i], 2 * warp + i, lane, x0, y0, z0, n0, N, bias, relu, osc, out);
+        if (next >= ntiles) break;
+        __syncthreads();   // the halo has been read
+        if (!PRE) halo_load(src, hu, nx0, ny0, nz0, hv);
+        tile = next;
+        x0 = nx0;
+        y0 = ny0;
+        z0 = nz0;
+    }
+}
+
+// One 8 x 4 x 4 block and 32 outputs per CTA; warp (w & 3) takes voxels
+// 32 (w & 3) .. + 31, w / 4 16 of the outputs.  Three weight buffers: tap
+// t + 2 is copied while tap t multiplies, one barrier a tap.
+template <int C, class OutT>
+__global__ void __launch_bounds__(kThreads) k_conv_stream(ConvSrc src, const __nv_bfloat16* __restrict__ Wt, int Npad,
+                                                          int N, const float* __restrict__ bias, int relu,
+                                                          const float* __restrict__ oscale, OutT* __restrict__ out,
+                                                          int split)
+{
+    extern __shared__ __align__(16) unsigned char cs_raw[];
+    constexpr int TY = 4, CS = C + 8, BN = kStreamBN, WS = BN + 8, NT = 2;
+    using G = HaloGeom<TY>;
+    constexpr int ITEMS = G::HV * (C / 8), PER = 6;
+    __nv_bfloat16* sH = reinterpret_cast<__nv_bfloat16*>(cs_raw);
+    __nv_bfloat16* sW = sH + (size_t)G::HV * CS;   // three [C][BN + 8]
+    int* toff = reinterpret_cast<int*>(sW + 3 * C * WS);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, wm = warp & 3, wn = warp >> 2;
+    const int n0 = blockIdx.y * BN;
+    const float osc = oscale ? *oscale : 1.f;
+    auto stage_w = [&](int t) {
+        if (t < 27) {
+            __nv_bfloat16* d = sW + (t % 3) * C * WS;
+#pragma unroll
+            for (int i = threadIdx.x; i < C * (BN / 8); i += kThreads) {
+                const int r = i / (BN / 8), c = i % (BN / 8);
+                lin_cp16(d + r * WS + c * 8, Wt + (size_t)(t * C + r) * Npad + n0 + c * 8, true);
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    stage_w(0);
+    stage_w(1);
+    int x0, y0, z0;
+    block_origin<TY>(src, blockIdx.x, x0, y0, z0);
+    for (int first = threadIdx.x; first < ITEMS; first += PER * kThreads) {
+        HaloUnits<C, TY, PER> hu;
+        hu.init(src, first);
+        uint4 hv[PER];
+        halo_load(src, hu, x0, y0, z0, hv);
+        halo_put<C>(sH, first, ITEMS, hv);
+    }
+    if (threadIdx.x < 27) toff[threadIdx.x] = 2 * tap_halo<C, TY>(threadIdx.x, src.flip ? -1 : 1);
+    uint32_t abase[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int m = 32 * wm + 16 * i + (lane & 15);
+        abase[i] = smem_addr(sH + ((m / (kTX * TY) + 1) * (G::HY * G::HX) + ((m / kTX) % TY + 1) * G::HX + m % kTX + 1) * CS +
+                             (lane >> 4) * 8);
+    }
+    const uint32_t bbase = smem_addr(sW + ((lane & 7) + ((lane >> 3) & 1) * 8) * WS + (lane >> 4) * 8 + wn * 16);
+    float acc[2][NT][4], tot[2][NT][4];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int q = 0; q < NT; ++q)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc[i][q][e] = tot[i][q][e] = 0.f;
+    auto fold = [&]() {   // the split's sum joins the total, a new one starts
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int q = 0; q < NT; ++q)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    tot[i][q][e] += acc[i][q][e];
+                    acc[i][q][e] = 0.f;
+                }
+    };
+    int left = split;
+    for (int t = 0; t < 27; ++t) {
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncthreads();   // tap t's weights have landed; tap t - 1's have been read
+        stage_w(t + 2);
+        const int o = toff[t];
+        const uint32_t b = bbase + (t % 3) * C * WS * 2;
+#pragma unroll
+        for (int c = 0; c < C / 16; ++c) {
+            uint32_t fa[2][4], fb[4];
+            ldsm_a(fa[0], abase[0] + o + 32 * c);
+            ldsm_a(fa[1], abase[1] + o + 32 * c);
+            ldsm_bt(fb, b + c * 16 * WS * 2);
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                mma_bf16(acc[i][0], fa[i], fb[0], fb[1]);
+                mma_bf16(acc[i][1], fa[i], fb[2], fb[3]);
+            }
+            if (--left == 0) {
+                fold();
+                left = split;
+            }
+        }
+    }
+    if (split > 0) {
+        if (left != split) fold();
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+            conv_store<TY>(src, tot[i], 2 * wm + i, lane, x0, y0, z0, n0 + 16 * wn, N, bias, relu, osc, out);
+    } else {
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+            conv_store<TY>(src, acc[i], 2 * wm + i, lane, x0, y0, z0, n0 + 16 * wn, N, bias, relu, osc, out);
     }
 }
 
@@ -621,24 +929,6 @@ constexpr int kLT = 96;             // threads: one warp per dy
 constexpr int kBiasT = 256;         // summands in flight of a bias chunk (k_bias_part's threads)
 constexpr int kBiasY = (kBiasT + kLT - 1) / kLT;   // CTAs per chunk that carry them
 
-// n / d for 0 <= n < 2^31 by a multiplication (d >= 1): m = ceil(2^(31+l) / d),
-// l = ceil(log2 d), has an error below 1, so n m / 2^(31+l) is off by less
-// than 2^-l <= 1/d.
-struct FastDiv {
-    uint32_t d = 1, m = 0, s = 0;
-    FastDiv() = default;
-    explicit FastDiv(int div) : d((uint32_t)div)
-    {
-        uint32_t l = 0;
-        while ((1ull << l) < d) ++l;
-        if (d > 1) {
-            m = (uint32_t)(((1ull << (31 + l)) + d - 1) / d);
-            s = l - 1;
-        }
-    }
-    __device__ __forceinline__ uint32_t div(uint32_t n) const { return d == 1 ? n : __umulhi(n, m) >> s; }
-};
-
 template <int BN>
 struct LinSmem {   // one of the two buffers, elements
     static constexpr int kSrc = 3 * kLR * kLS;
@@ -646,12 +936,6 @@ struct LinSmem {   // one of the two buffers, elements
     static constexpr int kBuf = kSrc + kGrad + kLV;   // and the block's masks
     static constexpr size_t bytes() { return sizeof(__nv_bfloat16) * (2 * (size_t)kBuf + 8); }
 };
-
-__device__ __forceinline__ void lin_cp16(void* sdst, const void* gsrc, bool in)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr(sdst)), "l"(gsrc), "r"(in ? 16u : 0u)
-                 : "memory");
-}
 
 __device__ __forceinline__ void ldsm_x2_t(uint32_t r[2], const void* p)
 {
@@ -998,7 +1282,7 @@ __global__ void __launch_bounds__(kC1T) k_wgrad_lin1(ConvSrc src, const __nv_bfl
 // gW[n][k] = sum over chunks, in order, of part[chunk][k][n] (as
 // k_wgrad_reduce); the last block's sums gb[n] over
 // the chunks of the bias summands, each chunk's in k_bias_part's order.
-__global__ void __launch_bounds__(256) k_wgrad_lin_reduce(const float* __restrict__ part, int chunks, int Kpad,
+static __global__ void __launch_bounds__(256) k_wgrad_lin_reduce(const float* __restrict__ part, int chunks, int Kpad,
                                                           int Kvalid, int N, const float* __restrict__ bvs,
                                                           float* __restrict__ gW, float* __restrict__ gb)
 {
@@ -1046,7 +1330,7 @@ __global__ void __launch_bounds__(256) k_wgrad_lin_reduce(const float* __restric
 
 // grad[n][k] (k < Kvalid: the parameter layout W[co][tap][ci]) = sum over
 // chunks, in chunk order, of part[chunk][k][n].
-__global__ void k_wgrad_reduce(const float* __restrict__ part, int chunks, int Kpad, int Kvalid, int N,
+static __global__ void k_wgrad_reduce(const float* __restrict__ part, int chunks, int Kpad, int Kvalid, int N,
                                float* __restrict__ grad)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1062,7 +1346,7 @@ __global__ void k_wgrad_reduce(const float* __restrict__ part, int chunks, int K
 // contiguous run: thread t (t < per, per the largest multiple of N within
 // the block) always lands on channel t % N, and the threads of a channel are
 // combined in thread order.
-__global__ void k_bias_part(const __nv_bfloat16* __restrict__ dY, long long V, int N, float* __restrict__ part)
+static __global__ void k_bias_part(const __nv_bfloat16* __restrict__ dY, long long V, int N, float* __restrict__ part)
 {
     __shared__ float red[kThreads];
     const long long v0 = (long long)blockIdx.x * kWChunk;
@@ -1080,7 +1364,7 @@ __global__ void k_bias_part(const __nv_bfloat16* __restrict__ dY, long long V, i
     }
 }
 
-__global__ void k_bias_reduce(const float* __restrict__ part, int blocks, int N, float* __restrict__ grad)
+static __global__ void k_bias_reduce(const float* __restrict__ part, int blocks, int N, float* __restrict__ grad)
 {
     const int n = blockIdx.x * blockDim.x + threadIdx.x;
     if (n >= N) return;
@@ -1090,7 +1374,7 @@ __global__ void k_bias_reduce(const float* __restrict__ part, int blocks, int N,
 }
 
 // 2x2x2 mean pool of [D][H][W][C] (D, H, W even) into [D/2][H/2][W/2][C].
-__global__ void k_pool(const __nv_bfloat16* __restrict__ in, int D, int H, int W, int C,
+static __global__ void k_pool(const __nv_bfloat16* __restrict__ in, int D, int H, int W, int C,
                        __nv_bfloat16* __restrict__ out)
 {
     const long long n = (long long)(D / 2) * (H / 2) * (W / 2) * C;
@@ -1112,7 +1396,7 @@ __global__ void k_pool(const __nv_bfloat16* __restrict__ in, int D, int H, int W
 
 // g[v][c] = skip[v][c] + gp[parent(v)][c] / 8: gradient of a volume that
 // feeds both a 2x2x2 mean pool (gradient gp) and an additive skip (skip).
-__global__ void k_pool_grad_add(const __nv_bfloat16* __restrict__ skip, const __nv_bfloat16* __restrict__ gp, int D,
+static __global__ void k_pool_grad_add(const __nv_bfloat16* __restrict__ skip, const __nv_bfloat16* __restrict__ gp, int D,
                                 int H, int W, int C, __nv_bfloat16* __restrict__ g)
 {
     const long long n = (long long)D * H * W * C;
@@ -1130,7 +1414,7 @@ __global__ void k_pool_grad_add(const __nv_bfloat16* __restrict__ skip, const __
 
 // Gradient of a nearest x2 upsampling: g[z][y][x][c] = sum of the 8 children
 // of fine-grid gradient gf ([2D][2H][2W][C]).
-__global__ void k_up_grad(const __nv_bfloat16* __restrict__ gf, int D, int H, int W, int C,
+static __global__ void k_up_grad(const __nv_bfloat16* __restrict__ gf, int D, int H, int W, int C,
                           __nv_bfloat16* __restrict__ g)
 {
     const long long n = (long long)D * H * W * C;
@@ -1152,17 +1436,106 @@ __global__ void k_up_grad(const __nv_bfloat16* __restrict__ gf, int D, int H, in
 
 // out = g where y > 0 else 0 (ReLU gradient; g itself is kept, a skip may
 // need it unmasked).
-__global__ void k_relu_grad(__nv_bfloat16* __restrict__ out, const __nv_bfloat16* __restrict__ g,
+static __global__ void k_relu_grad(__nv_bfloat16* __restrict__ out, const __nv_bfloat16* __restrict__ g,
                             const __nv_bfloat16* __restrict__ y, long long n)
 {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) out[i] = bf2f(y[i]) > 0.f ? g[i] : __float2bfloat16(0.f);
 }
 
+// The elementwise kernels above on 8 channels a thread (C a multiple of 8):
+// one 16-byte access per voxel and operand instead of eight 2-byte ones, and
+// the voxel's coordinates once (divisions by multiplication); the sums run
+// per channel in the same order.  The scalar forms keep other channel counts.
+struct Vol8 {   // index math of [D][H][W][C / 8] units
+    FastDiv dc, dw, dh;
+    int n;   // units
+    Vol8(int D, int H, int W, int C) : dc(C / 8), dw(W), dh(H), n(D * H * W * (C / 8)) {}
+    __device__ __forceinline__ void split(int i, int& c8, int& x, int& y, int& z) const
+    {
+        const int v = (int)dc.div((uint32_t)i);
+        c8 = i - v * (int)dc.d;
+        const int q = (int)dw.div((uint32_t)v);
+        x = v - q * (int)dw.d;
+        z = (int)dh.div((uint32_t)q);
+        y = q - z * (int)dh.d;
+    }
+};
+__device__ __forceinline__ void add8(float (&s)[8], uint4 q)
+{
+    const __nv_bfloat162* p = reinterpret_cast<const __nv_bfloat162*>(&q);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const float2 f = __bfloat1622float2(p[e]);
+        s[2 * e] += f.x;
+        s[2 * e + 1] += f.y;
+    }
+}
+__device__ __forceinline__ uint4 pack8(const float (&s)[8], float f)
+{
+    uint4 r;
+    __nv_bfloat162* p = reinterpret_cast<__nv_bfloat162*>(&r);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) p[e] = __floats2bfloat162_rn(s[2 * e] * f, s[2 * e + 1] * f);
+    return r;
+}
+// The 8 children of each coarse unit summed times f: the mean pool (f = 1/8)
+// and the gradient of the upsampling (f = 1).  g: the coarse volume.
+static __global__ void k_sum8_v8(const uint4* __restrict__ in, Vol8 g, float f, uint4* __restrict__ out)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= g.n) return;
+    int c8, x, y, z;
+    g.split(i, c8, x, y, z);
+    const int C8 = (int)g.dc.d, W = 2 * (int)g.dw.d, H = 2 * (int)g.dh.d;
+    const uint4* p = in + (((size_t)(2 * z) * H + 2 * y) * W + 2 * x) * C8 + c8;
+    uint4 q[8];
+#pragma unroll
+    for (int a = 0; a < 8; ++a) q[a] = p[(((size_t)(a >> 2) * H + ((a >> 1) & 1)) * W + (a & 1)) * C8];
+    float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int a = 0; a < 8; ++a) add8(s, q[a]);
+    out[i] = pack8(s, f);
+}
+static __global__ void k_pool_grad_add_v8(const uint4* __restrict__ skip, const uint4* __restrict__ gp, Vol8 g,
+                                          uint4* __restrict__ out)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= g.n) return;
+    int c8, x, y, z;
+    g.split(i, c8, x, y, z);
+    const int C8 = (int)g.dc.d, W = (int)g.dw.d >> 1, H = (int)g.dh.d >> 1;
+    const uint4 a = skip[i], b = gp[(((size_t)(z >> 1) * H + (y >> 1)) * W + (x >> 1)) * C8 + c8];
+    uint4 r;
+    const __nv_bfloat162* pa = reinterpret_cast<const __nv_bfloat162*>(&a);
+    const __nv_bfloat162* pb = reinterpret_cast<const __nv_bfloat162*>(&b);
+    __nv_bfloat162* pr = reinterpret_cast<__nv_bfloat162*>(&r);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const float2 u = __bfloat1622float2(pa[e]), v = __bfloat1622float2(pb[e]);
+        pr[e] = __floats2bfloat162_rn(u.x + v.x * 0.125f, u.y + v.y * 0.125f);
+    }
+    out[i] = r;
+}
+static __global__ void k_relu_grad_v8(uint4* __restrict__ out, const uint4* __restrict__ g, const uint4* __restrict__ y,
+                                      long long n8)
+{
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n8) return;
+    uint4 a = g[i];
+    const uint4 b = y[i];
+    __nv_bfloat16* pa = reinterpret_cast<__nv_bfloat16*>(&a);
+    const __nv_bfloat16* pb = reinterpret_cast<const __nv_bfloat16*>(&b);
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+        if (!(bf2f(pb[e]) > 0.f)) pa[e] = __float2bfloat16(0.f);
+    out[i] = a;
+}
+
 // Loss sum((out - t)^2) / (2 V) per block in FP64 partials; gradient
 // g = (out - t) / V as bfloat16.  The target is multiplied by the device
 // scalar *tscale when given.
-__global__ void k_mse(const float* __restrict__ out, const float* __restrict__ t, const float* __restrict__ tscale,
+static __global__ void k_mse(const float* __restrict__ out, const float* __restrict__ t, const float* __restrict__ tscale,
                       long long V, __nv_bfloat16* __restrict__ g, double* __restrict__ part)
 {
     __shared__ double red[kThreads];
@@ -1183,7 +1556,7 @@ __global__ void k_mse(const float* __restrict__ out, const float* __restrict__ t
 }
 
 // Per-block FP64 partial sums of in[i]^2.
-__global__ void k_sumsq_part(const float* __restrict__ in, long long V, double* __restrict__ part)
+static __global__ void k_sumsq_part(const float* __restrict__ in, long long V, double* __restrict__ part)
 {
     __shared__ double red[kThreads];
     double s = 0.0;
@@ -1200,13 +1573,19 @@ __global__ void k_sumsq_part(const float* __restrict__ in, long long V, double* 
     if (threadIdx.x == 0) part[blockIdx.x] = red[0];
 }
 
+constexpr int kScaleMax = 304;   // most partial sums of the RMS
+
 // r = RMS of the input from the partials (in block order); scales =
 // {1 / r, r gain, 1 / (r gain)} (r = 1 for an all-zero input).
-__global__ void k_scales(const double* __restrict__ part, int nb, long long V, float gain, float* __restrict__ scales)
+static __global__ void k_scales(const double* __restrict__ part, int nb, long long V, float gain, float* __restrict__ scales)
 {
+    __shared__ double ps[kScaleMax];   // every partial in flight at once, then added in order
+    for (int b = threadIdx.x; b < nb; b += blockDim.x) ps[b] = part[b];
+    __syncthreads();
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     double s = 0.0;
-    for (int b = 0; b < nb; ++b) s += part[b];
+#pragma unroll 8
+    for (int b = 0; b < nb; ++b) s += ps[b];
     double r = sqrt(s / (double)V);
     if (!(r > 0.0)) r = 1.0;
     scales[0] = (float)(1.0 / r);
@@ -1217,7 +1596,7 @@ __global__ void k_scales(const double* __restrict__ part, int nb, long long V, f
 // Wt[k][n] (forward) = W[n][k] for k < 27 Cin, n < Cout; zero padding.
 // With transpose_io (gradient w.r.t. the input): k = tap * Cout + co,
 // n = ci, Wt[k][n] = W[co][tap][ci].
-__global__ void k_prep_weights(const float* __restrict__ W, int Cin, int Cout, int Kpad, int Npad, int transpose_io,
+static __global__ void k_prep_weights(const float* __restrict__ W, int Cin, int Cout, int Kpad, int Npad, int transpose_io,
                                __nv_bfloat16* __restrict__ Wt)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1235,9 +1614,65 @@ __global__ void k_prep_weights(const float* __restrict__ W, int Cin, int Cout, i
     Wt[i] = __float2bfloat16(v);
 }
 
+// One operand matrix of the network, all of them written by one launch of
+// k_prep_all (forty launches of a microsecond or two before): kind 0 the
+// implicit-GEMM matrix of k_prep_weights, 1 the tcgen05 layout (C8P, NP; see
+// umma_conv.cuh), 2 its paired-tap layout.  K = 27 Cs rows and N columns of the
+// matrix carry weights; blocks [block0, next job's block0).
+struct PrepJob {
+    int kind, transpose, cin, cout, K, N, Npad, Cs, C8P, NP, sgn, total, block0;
+    long long woff;
+    __nv_bfloat16* dst;
+};
+static __global__ void k_prep_all(const PrepJob* __restrict__ jobs, int njobs, const float* __restrict__ theta)
+{
+    __shared__ int job_s;
+    if (threadIdx.x == 0) {
+        int lo = 0, hi = njobs - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) / 2;
+            if (jobs[mid].block0 <= (int)blockIdx.x) lo = mid;
+            else hi = mid - 1;
+        }
+        job_s = lo;
+    }
+    __syncthreads();
+    const PrepJob& q = jobs[job_s];
+    const int i = ((int)blockIdx.x - q.block0) * blockDim.x + threadIdx.x;
+    if (i >= q.total) return;
+    const float* W = theta + q.woff;
+    int k = -1, n = 0;   // row and column of the matrix; -1: padding
+    if (q.kind == 0) {
+        k = i / q.Npad;
+        n = i % q.Npad;
+    } else if (q.kind == 1) {
+        const int j = i % 8, c = (i / (8 * q.NP)) % q.C8P, tap = i / (8 * q.NP * q.C8P), ci = 8 * c + j;
+        n = (i / 8) % q.NP;
+        if (ci < q.Cs) k = tap * q.Cs + ci;
+    } else {
+        const int j = i % 8, c = (i / (8 * q.NP)) % 2, g = (i / (16 * q.NP)) % 2, pzx = i / (32 * q.NP);
+        const int pz = pzx / 3, px = pzx % 3, p = g == 0 ? c : (c == 0 ? 2 : -1);
+        n = (i / 8) % q.NP;
+        if (p >= 0 && j < q.Cs) {
+            const int dz = q.sgn * (pz - 1), dy = q.sgn * (p - 1), dx = q.sgn * (px - 1);
+            k = (9 * (dz + 1) + 3 * (dy + 1) + (dx + 1)) * q.Cs + j;
+        }
+    }
+    float v = 0.f;
+    if (k >= 0 && k < q.K && n < q.N) {
+        if (!q.transpose) {
+            v = W[(size_t)n * 27 * q.cin + k];
+        } else {
+            const int tap = k / q.cout, co = k % q.cout;
+            v = W[((size_t)co * 27 + tap) * q.cin + n];
+        }
+    }
+    q.dst[i] = __float2bfloat16(v);
+}
+
 // Adam (FP32 master weights): m = b1 m + (1 - b1) g, v = b2 v + (1 - b2) g^2,
 // theta -= lr (m / (1 - b1^t)) / (sqrt(v / (1 - b2^t)) + eps).
-__global__ void k_adam(float* __restrict__ theta, float* __restrict__ m, float* __restrict__ v,
+static __global__ void k_adam(float* __restrict__ theta, float* __restrict__ m, float* __restrict__ v,
                        const float* __restrict__ g, long long n, float lr, float b1, float b2, float eps, float c1,
                        float c2)
 {
