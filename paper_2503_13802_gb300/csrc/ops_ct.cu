@@ -392,11 +392,16 @@ static cudaError_t run_x_ct(const XArgs& a, int which, cudaStream_t st)
     return cudaGetLastError();
 }
 
-// MH3D_XFWD_PAIRS=8: 16 rows per CTA for the forward pass (A/B).
-static bool xfwd_small()
+// Rows per CTA of the forward pass: 32, or 16 where the buffers of 32 rows
+// leave an SM one CTA of four warps (n_x = 256, s = 1: 135 KB; the drive pass
+// of 256x256x128, K = 16 took 308 us so, 43 % of the copy bandwidth, and takes
+// 222 with three CTAs of 16 rows).
+// MH3D_XFWD_PAIRS=8 or 16 chooses (A/B).
+static bool xfwd_small(const XArgs& a)
 {
     const char* e = std::getenv("MH3D_XFWD_PAIRS");
-    return e && e[0] == '8';
+    if (e && e[0]) return e[0] == '8';
+    return xpass_desc(a.nx, a.s, 0).smem > 110 * 1024;
 }
 
 // Harmonics per CTA of the forward pass: all of them by default (13.5 us
@@ -413,7 +418,7 @@ cudaError_t run_xfwd_ct(const XArgs& a0, cudaStream_t st)
 {
     XArgs a = a0;
     a.kpc = xfwd_kpc(a.K);
-    const XDesc d = xpass_desc(a.nx, a.s, xfwd_small() ? 6 : 0);
+    const XDesc d = xpass_desc(a.nx, a.s, xfwd_small(a) ? 6 : 0);
     const dim3 grid(xpass_blocks(a.rows, d.pairs), (a.K + a.kpc - 1) / a.kpc);
     d.fn<<<grid, d.threads, d.smem, st>>>(a);
     return cudaGetLastError();
