@@ -705,6 +705,27 @@ __device__ __forceinline__ void nrm_epilogue(const XArgs& a, int row0, const flo
     const float* __restrict__ bp = a.b;
     const float* __restrict__ pp = a.pin;
     float* __restrict__ qp = a.qout;
+    if (a.reg.kind != 0 && a.vec4 && (((uintptr_t)pp | (uintptr_t)qp) & 15u) == 0) {
+        // the stencil prior, four voxels a thread (a pass at 96 x 96 x 64: 20 us
+        // with a voxel a thread, 15 loads and 12 integer modulos each; 7.3 so)
+#pragma unroll 1
+        for (int idx = threadIdx.x; idx < TOTAL; idx += T) {
+            const int rr = idx / V, x = 4 * (idx - rr * V);
+            const int r = row0 + rr;
+            if (r >= a.rows) continue;
+            const long long i = (long long)r * NX + x;
+            const int z = r / a.reg.ny, y = r - z * a.reg.ny;
+            const float4 rt = reg_term4(a.reg, pp, i, x, y, z);
+            const float4 w = *reinterpret_cast<const float4*>(stg + rr * NXS + x);
+            const float4 b = bp ? __ldg(reinterpret_cast<const float4*>(bp + i)) : make_float4(1.f, 1.f, 1.f, 1.f);
+            const float4 pv = __ldg(reinterpret_cast<const float4*>(pp + i));
+            const float4 q = make_float4(fmaf(b.x, w.x, rt.x), fmaf(b.y, w.y, rt.y), fmaf(b.z, w.z, rt.z),
+                                         fmaf(b.w, w.w, rt.w));
+            *reinterpret_cast<float4*>(qp + i) = q;
+            nrm_dots(pv, q, acc, acc2);
+        }
+        return;
+    }
     if (!a.vec4 || a.reg.kind != 0) {
         for (int idx = threadIdx.x; idx < ROWS * NX; idx += T) {
             const int rr = idx / NX, x = idx - rr * NX;
@@ -748,16 +769,7 @@ __device__ __forceinline__ void nrm_epilogue(const XArgs& a, int row0, const flo
         q.z = fmaf(B[it].z, W[it].z, lam * Pv[it].z);
         q.w = fmaf(B[it].w, W[it].w, lam * Pv[it].w);
         *reinterpret_cast<float4*>(qp + i) = q;
-        acc->add(Pv[it].x, q.x);
-        acc->add(Pv[it].y, q.y);
-        acc->add(Pv[it].z, q.z);
-        acc->add(Pv[it].w, q.w);
-        if (acc2) {
-            acc2->add(Pv[it].x, Pv[it].x);
-            acc2->add(Pv[it].y, Pv[it].y);
-            acc2->add(Pv[it].z, Pv[it].z);
-            acc2->add(Pv[it].w, Pv[it].w);
-        }
+        nrm_dots(Pv[it], q, acc, acc2);
     }
 }
 

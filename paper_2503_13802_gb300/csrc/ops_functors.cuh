@@ -24,7 +24,15 @@ __device__ __forceinline__ void st2(float* __restrict__ p, long long i, bool has
     }
 }
 
-__device__ __forceinline__ int wrap(int a, int n) { a %= n; return a < 0 ? a + n : a; }
+// a mod n for a in [-2, n + 1] (n >= 1): two steps either way cover n = 1.
+__device__ __forceinline__ int wrap(int a, int n)
+{
+    if (a < 0) a += n;
+    if (a < 0) a += n;
+    if (a >= n) a -= n;
+    if (a >= n) a -= n;
+    return a;
+}
 
 // lambda * (R p)[i] at voxel (x, y, z).
 __device__ __forceinline__ float reg_term(const RegArgs& g, const float* __restrict__ p, long long i, int x, int y,
@@ -56,6 +64,35 @@ __device__ __forceinline__ float reg_term(const RegArgs& g, const float* __restr
                        z >= g.nz - g.shell;
     if (shell) acc += g.alpha * pc;
     return g.lambda * acc;
+}
+
+// The same at voxels x .. x + 3 of a row (x and nx multiples of 4, p 16-byte
+// aligned): eleven float4 loads where reg_term takes 52 scalar ones.
+__device__ __forceinline__ float4 reg_term4(const RegArgs& g, const float* __restrict__ p, long long i, int x, int y,
+                                            int z)
+{
+    const int sy = g.nx, sz = g.nx * g.ny;
+    const float* c0 = p + i;
+    auto ld = [&](long long off) { return __ldg(reinterpret_cast<const float4*>(c0 + off)); };
+    auto dy = [&](int d) { return ld((long long)(wrap(y + d, g.ny) - y) * sy); };
+    auto dz = [&](int d) { return ld((long long)(wrap(z + d, g.nz) - z) * sz); };
+    const float4 c = ld(0), l = ld(x == 0 ? g.nx - 4 : -4), r = ld(x + 4 == g.nx ? 4 - g.nx : 4);
+    const float4 y0 = dy(-2), y1 = dy(-1), y3 = dy(1), y4 = dy(2), z0 = dz(-2), z1 = dz(-1), z3 = dz(1), z4 = dz(2);
+    auto one = [&](float x0, float x1, float pc, float x3, float x4, float ya, float yb, float yc, float yd, float za,
+                   float zb, float zc, float zd, int xx) {
+        float acc = 0.f;
+        acc += x0 - 4.f * x1 + 6.f * pc - 4.f * x3 + x4;
+        acc += ya - 4.f * yb + 6.f * pc - 4.f * yc + yd;
+        acc += za - 4.f * zb + 6.f * pc - 4.f * zc + zd;
+        const bool shell = xx < g.shell || y < g.shell || z < g.shell || xx >= g.nx - g.shell ||
+                           y >= g.ny - g.shell || z >= g.nz - g.shell;
+        if (shell) acc += g.alpha * pc;
+        return g.lambda * acc;
+    };
+    return make_float4(one(l.z, l.w, c.x, c.y, c.z, y0.x, y1.x, y3.x, y4.x, z0.x, z1.x, z3.x, z4.x, x),
+                       one(l.w, c.x, c.y, c.z, c.w, y0.y, y1.y, y3.y, y4.y, z0.y, z1.y, z3.y, z4.y, x + 1),
+                       one(c.x, c.y, c.z, c.w, r.x, y0.z, y1.z, y3.z, y4.z, z0.z, z1.z, z3.z, z4.z, x + 2),
+                       one(c.y, c.z, c.w, r.x, r.y, y0.w, y1.w, y3.w, y4.w, z0.w, z1.w, z3.w, z4.w, x + 3));
 }
 
 // CG loop control at the start of an iteration's kernels.  Returns false
@@ -604,6 +641,21 @@ struct QLd {
     __device__ __forceinline__ At at(int p) const { return At{A + p, ldA, Q, mx, s, dmx}; }
 };
 
+// p^T q (and p^T p for acc2) of four voxels.
+__device__ __forceinline__ void nrm_dots(const float4& p, const float4& q, DotAcc* acc, DotAcc* acc2)
+{
+    acc->add(p.x, q.x);
+    acc->add(p.y, q.y);
+    acc->add(p.z, q.z);
+    acc->add(p.w, q.w);
+    if (acc2) {
+        acc2->add(p.x, p.x);
+        acc2->add(p.y, p.y);
+        acc2->add(p.z, p.z);
+        acc2->add(p.w, p.w);
+    }
+}
+
 // Normal epilogue q = b w + lambda R p over a tile of 2 P rows of w (pencil
 // layout, row 2p the real and row 2p + 1 the imaginary part), accumulating
 // p^T q (and p^T p for acc2), lanes along x.
@@ -614,10 +666,27 @@ __device__ __forceinline__ void nrm_epilogue_rt(const XArgs& a, int row0, int P,
     const bool plain = a.reg.kind == 0;
     const int nx = a.nx, lane = (int)threadIdx.x & 31, nw = (int)blockDim.x >> 5;
     constexpr int U = 4;   // elements a step, their loads first
+    // the stencil prior in groups of four voxels (reg_term4)
+    const bool v4 = !plain && (nx & 3) == 0 && (((uintptr_t)a.pin | (uintptr_t)a.qout) & 15u) == 0;
     for (int rr = (int)threadIdx.x >> 5; rr < 2 * P && row0 + rr < a.rows; rr += nw) {   // a warp per row
         const int r = row0 + rr, i0 = r * nx;
         const int z = (int)a.dny.div((uint32_t)r), y = r - z * a.reg.ny;
         const float* wr = wf + 2 * (rr >> 1) + (rr & 1);
+        if (v4) {
+            for (int x = 4 * lane; x < nx; x += 128) {
+                const float4 rt = reg_term4(a.reg, a.pin, i0 + x, x, y, z);
+                const float4 pv = __ldg(reinterpret_cast<const float4*>(a.pin + i0 + x));
+                float4 bv = make_float4(1.f, 1.f, 1.f, 1.f), q;
+                if (a.b) bv = make_float4(a.b[i0 + x], a.b[i0 + x + 1], a.b[i0 + x + 2], a.b[i0 + x + 3]);
+                q.x = fmaf(bv.x, wr[2 * x * ld], rt.x);
+                q.y = fmaf(bv.y, wr[2 * (x + 1) * ld], rt.y);
+                q.z = fmaf(bv.z, wr[2 * (x + 2) * ld], rt.z);
+                q.w = fmaf(bv.w, wr[2 * (x + 3) * ld], rt.w);
+                *reinterpret_cast<float4*>(a.qout + i0 + x) = q;
+                nrm_dots(pv, q, acc, acc2);
+            }
+            continue;
+        }
         for (int x0 = lane; x0 < nx; x0 += 32 * U) {
             float pv[U], bv[U];
 #pragma unroll
