@@ -286,6 +286,24 @@ __global__ void k_gen_weight(const float* __restrict__ rho, const float* __restr
     }
 }
 
+// Index arithmetic of the fold and the unfold: coordinates by multiplication
+// (an index is below 1024^3 / 2 < 2^31), negation modulo a length without a
+// division.  With 64-bit divisions, a dozen per thread, the unfold took 37 us
+// and the fold 34 us at 128x128x64, K = 8, s = 2, three components; they take
+// 26 and 30 so, of which the spectra's DRAM reads are 15.
+constexpr int kGF = 128;   // threads per CTA: one frequency each, a short last wave
+struct GenDims {
+    FastDiv dnx, dny, dmx;
+    int nz;
+    GenDims(int nx, int ny, int nz_, int mx) : dnx(nx), dny(ny), dmx(mx), nz(nz_) {}
+    __device__ __forceinline__ int nx() const { return (int)dnx.d; }
+    __device__ __forceinline__ int ny() const { return (int)dny.d; }
+    __device__ __forceinline__ int mx() const { return (int)dmx.d; }
+    // a mod nx
+    __device__ __forceinline__ int phase(int a) const { return a - (int)dnx.div((uint32_t)a) * (int)dnx.d; }
+};
+__device__ __forceinline__ int neg_mod(int a, int n) { return a == 0 ? 0 : n - a; }
+
 // Portrait-grid spectra of every harmonic, D_k(w) = sum_a e^{2 pi i f r / nx}
 // sum_j H_kj(f) W_j(f), f = w + a mx (the row selector x = s i' + r as an
 // alias sum), q over [nz][ny][mx], written in harmonic pairs: Z_c = D_{2c} +
@@ -300,18 +318,19 @@ __global__ void k_gen_weight(const float* __restrict__ rho, const float* __restr
 // z <= nz / 2 and write the mirror of every q off the planes z = 0 and
 // 2 z = nz (which hold their own mirrors and are computed in full): each
 // spectrum sample is read for one of f and -f only.
-template <int SR>
-__global__ void k_gen_fold(const float2* __restrict__ H, const float2* __restrict__ W, float2* __restrict__ Z,
-                           int nx, int ny, int nz, int mx, int s, int r, int nc, int K, long long N, long long Q,
-                           const float2* __restrict__ twx)
+template <int SR, int NC>
+__global__ void __launch_bounds__(kGF) k_gen_fold(const float2* __restrict__ H, const float2* __restrict__ W,
+                                                  float2* __restrict__ Z, GenDims g, int s, int r, int K, long long N,
+                                                  long long Q, const float2* __restrict__ twx)
 {
-    const long long Qh = (long long)(nz / 2 + 1) * ny * mx;
-    for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < Qh; q += (long long)gridDim.x * blockDim.x) {
-        const int w = (int)(q % mx);
-        const long long row = (q - w) / mx * nx;   // (z ny + y) nx
-        const int yz = (int)((q - w) / mx), y = yz % ny, z = yz / ny;
+    const int nx = g.nx(), ny = g.ny(), nz = g.nz, mx = g.mx();
+    const int q = (int)(blockIdx.x * kGF + threadIdx.x);
+    if (q < (nz / 2 + 1) * ny * mx) {
+        const int yz = (int)g.dmx.div((uint32_t)q), w = q - yz * mx;
+        const int z = (int)g.dny.div((uint32_t)yz), y = yz - z * ny;
+        const int row = yz * nx;
         const bool mirror = z != 0 && 2 * z != nz;
-        const long long qm = ((long long)(nz - z) * ny + (ny - y) % ny) * mx + (mx - w) % mx;
+        const int yzm = neg_mod(z, nz) * ny + neg_mod(y, ny), qm = yzm * mx + neg_mod(w, mx);
         auto put = [&](int c, float2 da, float2 db) {
             Z[(long long)c * Q + q] = make_float2(da.x - db.y, da.y + db.x);
             if (mirror) Z[(long long)c * Q + qm] = make_float2(da.x + db.y, db.x - da.y);
@@ -319,14 +338,13 @@ __global__ void k_gen_fold(const float2* __restrict__ H, const float2* __restric
         // W holds the component pairs b_{2c} rho + i b_{2c+1} rho transformed:
         // with A = P_c(f) and B = conj(P_c(-f)), W_{2c} = (A + B) / 2 and
         // W_{2c+1} = (A - B) / 2i; a lone last component is P_c(f) itself
-        const int zm = (nz - z) % nz, ym = (ny - y) % ny;
         auto wcomp = [&](int f, float2* out) {
-            const long long i = row + f, im = ((long long)zm * ny + ym) * nx + (nx - f) % nx;
+            const int i = row + f, im = yzm * nx + neg_mod(f, nx);
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
-                if (2 * c >= nc) break;
+                if (2 * c >= NC) break;
                 const float2 A = W[(long long)c * N + i];
-                if (2 * c + 1 < nc) {
+                if (2 * c + 1 < NC) {
                     const float2 Bm = W[(long long)c * N + im];
                     out[2 * c] = make_float2(0.5f * (A.x + Bm.x), 0.5f * (A.y - Bm.y));
                     out[2 * c + 1] = make_float2(0.5f * (A.y + Bm.y), -0.5f * (A.x - Bm.x));
@@ -343,7 +361,7 @@ __global__ void k_gen_fold(const float2* __restrict__ H, const float2* __restric
                 wv[a][0] = wv[a][1] = wv[a][2] = make_float2(0.f, 0.f);
                 if (a < s) wcomp(f, wv[a]);
                 // e^{+2 pi i f r / nx} = conj(W_nx^{f r mod nx})
-                const float2 tw = a < s ? twx[(int)(((long long)f * r) % nx)] : make_float2(0.f, 0.f);
+                const float2 tw = a < s ? twx[g.phase(f * r)] : make_float2(0.f, 0.f);
                 ph[a] = make_float2(tw.x, -tw.y);
             }
             auto fold_k = [&](int k) {
@@ -354,33 +372,34 @@ __global__ void k_gen_fold(const float2* __restrict__ H, const float2* __restric
                     if (a < s) {
                         float2 t = make_float2(0.f, 0.f);
 #pragma unroll
-                        for (int j = 0; j < 3; ++j)
-                            if (j < nc) t = c_add(t, c_mul(Hk[(long long)j * N + a * mx], wv[a][j]));
+                        for (int j = 0; j < NC; ++j) t = c_add(t, c_mul(Hk[(long long)j * N + a * mx], wv[a][j]));
                         acc = c_add(acc, c_mul(t, ph[a]));
                     }
                 }
                 return acc;
             };
-            for (int c = 0; 2 * c < K; ++c)
-                put(c, fold_k(2 * c), 2 * c + 1 < K ? fold_k(2 * c + 1) : make_float2(0.f, 0.f));
+#pragma unroll 2
+            for (int c = 0; c < K / 2; ++c) put(c, fold_k(2 * c), fold_k(2 * c + 1));
+            if (K & 1) put(K / 2, fold_k(K - 1), make_float2(0.f, 0.f));
         } else {
             auto fold_k = [&](int k) {
                 const float2* __restrict__ Hk = H + (long long)k * 3 * N;
                 float2 acc = make_float2(0.f, 0.f);
                 for (int a = 0; a < s; ++a) {
                     const int f = w + a * mx;
-                    const long long i = row + f;
+                    const int i = row + f;
                     float2 wj[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
                     wcomp(f, wj);
                     float2 t = make_float2(0.f, 0.f);
-                    for (int j = 0; j < nc; ++j) t = c_add(t, c_mul(Hk[(long long)j * N + i], wj[j]));
-                    const float2 tw = twx[(int)(((long long)f * r) % nx)];
+                    for (int j = 0; j < NC; ++j) t = c_add(t, c_mul(Hk[(long long)j * N + i], wj[j]));
+                    const float2 tw = twx[g.phase(f * r)];
                     acc = c_add(acc, c_mul(t, make_float2(tw.x, -tw.y)));
                 }
                 return acc;
             };
-            for (int c = 0; 2 * c < K; ++c)
-                put(c, fold_k(2 * c), 2 * c + 1 < K ? fold_k(2 * c + 1) : make_float2(0.f, 0.f));
+#pragma unroll 2
+            for (int c = 0; c < K / 2; ++c) put(c, fold_k(2 * c), fold_k(2 * c + 1));
+            if (K & 1) put(K / 2, fold_k(K - 1), make_float2(0.f, 0.f));
         }
     }
 }
@@ -430,51 +449,48 @@ __global__ void k_gen_unphase(const float2* __restrict__ d, float2* __restrict__
 // a real image (H, U real images' spectra): V_j(-f) = conj(V_j(f)), so the
 // threads cover the planes z <= nz / 2 and write the mirrors off the planes
 // z = 0 and 2 z = nz, as the fold does.
-__global__ void k_gen_unfold(const float2* __restrict__ H, const float2* __restrict__ U, float2* __restrict__ V,
-                             int nx, int ny, int nz, int mx, int r, int nc, int K, long long N, long long Q,
-                             const float2* __restrict__ twx)
+template <int NC>
+__global__ void __launch_bounds__(kGF) k_gen_unfold(const float2* __restrict__ H, const float2* __restrict__ U,
+                                                    float2* __restrict__ V, GenDims g, int r, int K, long long N,
+                                                    long long Q, const float2* __restrict__ twx)
 {
-    const long long Nh = (long long)(nz / 2 + 1) * ny * nx;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < Nh; i += (long long)gridDim.x * blockDim.x) {
-        const int f = (int)(i % nx);
-        const int yz = (int)((i - f) / nx), y = yz % ny, z = yz / ny;
-        const bool mirror = z != 0 && 2 * z != nz;
-        const long long im = ((long long)(nz - z) * ny + (ny - y) % ny) * nx + (nx - f) % nx;
-        const int w = f % mx;
-        const long long qi = (long long)yz * mx + w;
-        // the portrait-grid mirror -g of g = (w, y, z)
-        const long long qim = ((long long)((nz - z) % nz) * ny + (ny - y) % ny) * mx + (mx - w) % mx;
-        float2 acc[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-        for (int c = 0; 2 * c < K; ++c) {
-            // U holds z_c = u_{2c} + i u_{2c+1} transformed: with A = Z(g) and
-            // B = conj(Z(-g)), U_{2c}(g) = (A + B) / 2, U_{2c+1}(g) = (A - B) / 2i
-            const float2 A = U[(long long)c * Q + qi], Bm = U[(long long)c * Q + qim];
-            const float2 B = make_float2(Bm.x, -Bm.y);
-            const float2 ua = make_float2(0.5f * (A.x + B.x), 0.5f * (A.y + B.y));
-            const float2 ub = make_float2(0.5f * (A.y - B.y), -0.5f * (A.x - B.x));
+    const int nx = g.nx(), ny = g.ny(), nz = g.nz, mx = g.mx();
+    const int i = (int)(blockIdx.x * kGF + threadIdx.x);
+    if (i >= (nz / 2 + 1) * ny * nx) return;
+    const int yz = (int)g.dnx.div((uint32_t)i), f = i - yz * nx;
+    const int z = (int)g.dny.div((uint32_t)yz), y = yz - z * ny;
+    const bool mirror = z != 0 && 2 * z != nz;
+    const int yzm = neg_mod(z, nz) * ny + neg_mod(y, ny), im = yzm * nx + neg_mod(f, nx);
+    const int w = f - (int)g.dmx.div((uint32_t)f) * mx;
+    const float2* __restrict__ Uq = U + yz * mx + w;
+    const float2* __restrict__ Um = U + yzm * mx + neg_mod(w, mx);   // the portrait-grid mirror
+    const float2* __restrict__ Hi = H + i;
+    float2 acc[NC];
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int k = 2 * c + h;
-                if (k >= K) break;
-                const float2 u = h == 0 ? ua : ub;
-                const float2* __restrict__ Hk = H + (long long)k * 3 * N + i;
+    for (int j = 0; j < NC; ++j) acc[j] = make_float2(0.f, 0.f);
+    auto add = [&](const float2* __restrict__ Hk, float2 u) {
 #pragma unroll
-                for (int j = 0; j < 3; ++j) {
-                    if (j < nc) {
-                        const float2 hv = Hk[(long long)j * N];
-                        acc[j] = c_add(acc[j], c_mul(make_float2(hv.x, -hv.y), u));
-                    }
-                }
-            }
+        for (int j = 0; j < NC; ++j) {
+            const float2 hv = Hk[(long long)j * N];
+            acc[j] = c_add(acc[j], c_mul(make_float2(hv.x, -hv.y), u));
         }
-        const float2 tw = twx[(int)(((long long)f * r) % nx)];   // e^{-2 pi i f r / nx}
+    };
+#pragma unroll 2
+    for (int c = 0; c < (K + 1) / 2; ++c) {
+        // U holds z_c = u_{2c} + i u_{2c+1} transformed: with A = Z(g) and
+        // B = conj(Z(-g)), U_{2c}(g) = (A + B) / 2, U_{2c+1}(g) = (A - B) / 2i
+        const float2 A = Uq[c * Q], Bm = Um[c * Q];
+        const float2 B = make_float2(Bm.x, -Bm.y);
+        add(Hi + (long long)(2 * c) * 3 * N, make_float2(0.5f * (A.x + B.x), 0.5f * (A.y + B.y)));
+        if (2 * c + 1 < K)
+            add(Hi + (long long)(2 * c + 1) * 3 * N, make_float2(0.5f * (A.y - B.y), -0.5f * (A.x - B.x)));
+    }
+    const float2 tw = twx[g.phase(f * r)];   // e^{-2 pi i f r / nx}
 #pragma unroll
-        for (int j = 0; j < 3; ++j)
-            if (j < nc) {
-                const float2 v = c_mul(acc[j], tw);
-                V[(long long)j * N + i] = v;
-                if (mirror) V[(long long)j * N + im] = make_float2(v.x, -v.y);
-            }
+    for (int j = 0; j < NC; ++j) {
+        const float2 v = c_mul(acc[j], tw);
+        V[(long long)j * N + i] = v;
+        if (mirror) V[(long long)j * N + im] = make_float2(v.x, -v.y);
     }
 }
 
@@ -711,15 +727,12 @@ mh3d_status mh3d_general_forward(mh3d_plan Pp, const float* rho, const float* bv
         GEN_CK(P, gen_fft3(P, W, nv, P.ax, false, st));
     }
     const long long Qh = (long long)(P.nz / 2 + 1) * P.ny * P.mx;   // the planes the fold's threads cover
-    if (P.s <= 2)
-        k_gen_fold<2><<<gen_blocks(Qh), kGB, 0, st>>>(P.gen_H, W, Z, P.nx, P.ny, P.nz, P.mx, P.s, P.r, nc, P.K, N, Q,
-                                                      P.ax.tw);
-    else if (P.s <= 4)
-        k_gen_fold<4><<<gen_blocks(Qh), kGB, 0, st>>>(P.gen_H, W, Z, P.nx, P.ny, P.nz, P.mx, P.s, P.r, nc, P.K, N, Q,
-                                                      P.ax.tw);
-    else
-        k_gen_fold<0><<<gen_blocks(Qh), kGB, 0, st>>>(P.gen_H, W, Z, P.nx, P.ny, P.nz, P.mx, P.s, P.r, nc, P.K, N, Q,
-                                                      P.ax.tw);
+    const GenDims gd(P.nx, P.ny, P.nz, P.mx);
+    const unsigned gf = (unsigned)((Qh + kGF - 1) / kGF);
+    auto fold = [&](auto* fn) { fn<<<gf, kGF, 0, st>>>(P.gen_H, W, Z, gd, P.s, P.r, P.K, N, Q, P.ax.tw); };
+    if (P.s <= 2) fold(bvec ? k_gen_fold<2, 3> : k_gen_fold<2, 1>);
+    else if (P.s <= 4) fold(bvec ? k_gen_fold<4, 3> : k_gen_fold<4, 1>);
+    else fold(bvec ? k_gen_fold<0, 3> : k_gen_fold<0, 1>);
     GEN_CK(P, cudaGetLastError());
     if (gen_ct_length(P.az.n)) {   // the pairs unpacked and phased in the z pass's store
         GEN_CK(P, gen_fft3(P, Z, Kh, P.am, true, st, 0, 2, io));
@@ -758,7 +771,9 @@ mh3d_status mh3d_general_adjoint(mh3d_plan Pp, const void* d, const float* bvec,
         GEN_CK(P, gen_fft3(P, U, Kh, P.am, false, st));
     }
     const long long Nh = (long long)(P.nz / 2 + 1) * P.ny * P.nx;   // the planes the unfold's threads cover
-    k_gen_unfold<<<gen_blocks(Nh), kGB, 0, st>>>(P.gen_H, U, V, P.nx, P.ny, P.nz, P.mx, P.r, nc, P.K, N, Q, P.ax.tw);
+    const GenDims gd(P.nx, P.ny, P.nz, P.mx);
+    auto* unfold = bvec ? k_gen_unfold<3> : k_gen_unfold<1>;
+    unfold<<<(unsigned)((Nh + kGF - 1) / kGF), kGF, 0, st>>>(P.gen_H, U, V, gd, P.r, P.K, N, Q, P.ax.tw);
     GEN_CK(P, cudaGetLastError());
     GEN_CK(P, gen_fft3(P, V, nc, P.ax, true, st));
     k_gen_out<<<gen_blocks(N), kGB, 0, st>>>(V, bvec, out, N, nc);

@@ -51,6 +51,53 @@ static size_t red_bytes(size_t cap) { return sizeof(double) * (cap * kNPart + 16
 // ---------------------------------------------------------------------------
 // Kernels
 // ---------------------------------------------------------------------------
+// The vector kernels move four elements a thread and access (16-byte aligned
+// vectors, which the workspace's are; one element else, and for the last
+// N mod 4) and take the totals of what they write in the same pass.  Bounded
+// by the launch and the last CTA's sum, not the bytes (1.05 M elements, out of
+// L2): the general CG's q += lambda p with p . q takes 7.3 us (5.3 + 6.8 as
+// two kernels), its two updates with r . r 9.1 (9.7 + 6.8).
+template <int W>
+struct Pack {
+    float v[W];
+};
+template <int W>
+__device__ __forceinline__ Pack<W> ldp(const float* p, long long i)
+{
+    Pack<W> r;
+    if constexpr (W == 4) {
+        const float4 t = reinterpret_cast<const float4*>(p)[i];
+        r.v[0] = t.x; r.v[1] = t.y; r.v[2] = t.z; r.v[3] = t.w;
+    } else {
+        r.v[0] = p[i];
+    }
+    return r;
+}
+template <int W>
+__device__ __forceinline__ void stp(float* p, long long i, const Pack<W>& r)
+{
+    if constexpr (W == 4) reinterpret_cast<float4*>(p)[i] = make_float4(r.v[0], r.v[1], r.v[2], r.v[3]);
+    else p[i] = r.v[0];
+}
+template <int W>
+struct Width {
+    static constexpr int w = W;
+};
+// f(Width<W>, i) for every pack i of the vector's W = 4 packs, then its rest.
+template <class F>
+__device__ __forceinline__ void vec_loop(long long N, bool v4, F f)
+{
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
+    const long long n4 = v4 ? N >> 2 : 0;
+    for (long long i = t; i < n4; i += stride) f(Width<4>{}, i);
+    for (long long i = 4 * n4 + t; i < N; i += stride) f(Width<1>{}, i);
+}
+template <class... Ps>
+__device__ __forceinline__ bool al16v(Ps... ps)
+{
+    return ((... | (uintptr_t)ps) & 15u) == 0;
+}
+
 // r = rhs - q (q may be null: zero start), x = 0 on a zero start; the
 // search direction starts as p = r (classic CG) or p = qd = 0 (single-
 // reduction CG, whose first update forms p = r); totals r^T r, rhs^T rhs.
@@ -58,29 +105,32 @@ __global__ void __launch_bounds__(256) k_cg_init(const float* __restrict__ rhs, 
                                                  float* __restrict__ r, float* __restrict__ p, float* __restrict__ qd,
                                                  float* __restrict__ x, int zero_x, long long N, double* rr_part,
                                                  unsigned int* rr_tk, double* rr_out, double* bn_part,
-                                                 unsigned int* bn_tk, double* bn_out)
+                                                 double* bn_out)
 {
     __shared__ double red[34];
     DotAcc ar, ab;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-        const float b = rhs[i];
-        const float rv = q ? b - q[i] : b;
-        r[i] = rv;
-        if (qd) {
-            p[i] = 0.f;
-            qd[i] = 0.f;
-        } else {
-            p[i] = rv;
+    vec_loop(N, al16v(rhs, q, r, p, qd, x), [&](auto wd, long long i) {
+        constexpr int W = decltype(wd)::w;
+        const Pack<W> b = ldp<W>(rhs, i), zero{};
+        Pack<W> rv = b;
+        if (q) {
+            const Pack<W> qv = ldp<W>(q, i);
+#pragma unroll
+            for (int e = 0; e < W; ++e) rv.v[e] = b.v[e] - qv.v[e];
         }
-        if (zero_x) x[i] = 0.f;
-        ar.add(rv, rv);
-        ab.add(b, b);
-    }
+        stp<W>(r, i, rv);
+        stp<W>(p, i, qd ? zero : rv);
+        if (qd) stp<W>(qd, i, zero);
+        if (zero_x) stp<W>(x, i, zero);
+#pragma unroll
+        for (int e = 0; e < W; ++e) {
+            ar.add(rv.v[e], rv.v[e]);
+            ab.add(b.v[e], b.v[e]);
+        }
+    });
     float2 t, t2;
     block_pair_acc2(ar, &ab, reinterpret_cast<float*>(red), &t, &t2);
-    grid_sum_finalize(t, rr_part, blockIdx.x, gridDim.x, rr_tk, rr_out);
-    __syncthreads();   // every thread has read the first ticket's flag before thread 0 reuses it
-    grid_sum_finalize(t2, bn_part, blockIdx.x, gridDim.x, bn_tk, bn_out);
+    grid_sum_finalize2(t, t2, rr_part, bn_part, blockIdx.x, gridDim.x, rr_tk, rr_out, bn_out);
 }
 
 // Warm-start fallback: if r0^T r0 >= rhs^T rhs the initial iterate is no
@@ -181,10 +231,17 @@ __global__ void __launch_bounds__(256) k_diff_norm2(const float* __restrict__ a,
 {
     __shared__ double red[34];
     DotAcc acc;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-        const float d = a[i] - (b ? b[i] : 0.f);
-        acc.add(d, d);
-    }
+    vec_loop(N, al16v(a, b), [&](auto wd, long long i) {
+        constexpr int W = decltype(wd)::w;
+        const Pack<W> av = ldp<W>(a, i);
+        Pack<W> bv{};
+        if (b) bv = ldp<W>(b, i);
+#pragma unroll
+        for (int e = 0; e < W; ++e) {
+            const float d = av.v[e] - bv.v[e];
+            acc.add(d, d);
+        }
+    });
     grid_sum_finalize(block_pair_acc(acc, red), part, blockIdx.x, gridDim.x, tk, out);
 }
 
@@ -194,8 +251,12 @@ __global__ void __launch_bounds__(256) k_dot(const float* __restrict__ a, const 
 {
     __shared__ double red[34];
     DotAcc acc;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x)
-        acc.add(a[i], b[i]);
+    vec_loop(N, al16v(a, b), [&](auto wd, long long i) {
+        constexpr int W = decltype(wd)::w;
+        const Pack<W> av = ldp<W>(a, i), bv = ldp<W>(b, i);
+#pragma unroll
+        for (int e = 0; e < W; ++e) acc.add(av.v[e], bv.v[e]);
+    });
     grid_sum_finalize(block_pair_acc(acc, red), part, blockIdx.x, gridDim.x, tk, out);
 }
 
@@ -219,20 +280,31 @@ __global__ void __launch_bounds__(256) k_apg_step(float* __restrict__ x, float* 
                                                   float* __restrict__ y, const float* __restrict__ ny,
                                                   const float* __restrict__ rhs, float tau, float mom_next, long long N)
 {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-        const float g = ny[i] - rhs[i];
-        const float xn = fmaxf(fmaf(-tau, g, y[i]), 0.f);
-        const float xo = x[i];
-        xprev[i] = xo;
-        x[i] = xn;
-        y[i] = fmaf(mom_next, xn - xo, xn);
-    }
+    vec_loop(N, al16v(x, xprev, y, ny, rhs), [&](auto wd, long long i) {
+        constexpr int W = decltype(wd)::w;
+        const Pack<W> nv = ldp<W>(ny, i), bv = ldp<W>(rhs, i), yv = ldp<W>(y, i), xo = ldp<W>(x, i);
+        Pack<W> xn, yn;
+#pragma unroll
+        for (int e = 0; e < W; ++e) {
+            const float g = nv.v[e] - bv.v[e];
+            xn.v[e] = fmaxf(fmaf(-tau, g, yv.v[e]), 0.f);
+            yn.v[e] = fmaf(mom_next, xn.v[e] - xo.v[e], xn.v[e]);
+        }
+        stp<W>(xprev, i, xo);
+        stp<W>(x, i, xn);
+        stp<W>(y, i, yn);
+    });
 }
 
 __global__ void __launch_bounds__(256) k_scale(float* __restrict__ v, const float* __restrict__ u, float s, long long N)
 {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x)
-        v[i] = s * u[i];
+    vec_loop(N, al16v(v, u), [&](auto wd, long long i) {
+        constexpr int W = decltype(wd)::w;
+        Pack<W> t = ldp<W>(u, i);
+#pragma unroll
+        for (int e = 0; e < W; ++e) t.v[e] *= s;
+        stp<W>(v, i, t);
+    });
 }
 
 cudaError_t solve_set_attributes() { return cudaSuccess; }
@@ -530,7 +602,7 @@ static mh3d_status cg_prefix(Plan& P, const float2* d, const mh3d_solve_opts& o,
     const bool cgcg = (o.cg_variant == 0);
     k_cg_init<<<nU, 256, 0, st>>>(w.rhs, qinit, w.r, w.p, cgcg ? w.q : nullptr, w.x, o.x0_dev ? 0 : 1, P.N,
                                   part_slot(P, kPartRR), ticket(P, kTkRR), scal(P, kRR1), part_slot(P, kPartBN),
-                                  ticket(P, kTkBN), scal(P, kBN));
+                                  scal(P, kBN));
     MH3D_CK(P, cudaGetLastError());
     if (o.x0_dev && o.x0_fallback) {
         k_cg_fallback<<<nU, 256, 0, st>>>(w.rhs, w.r, w.p, cgcg ? w.q : nullptr, w.x, P.N, scal(P, kRR1), scal(P, kBN),
@@ -1211,24 +1283,33 @@ static mh3d_status apg_solve(Plan& P, const float2* d, const mh3d_solve_opts& o,
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_axpy(float* __restrict__ y, const float* __restrict__ x, float a, long long N)
 {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x)
-        y[i] = fmaf(a, x[i], y[i]);
+    vec_loop(N, al16v(y, x), [&](auto wd, long long i) {
+        constexpr int W = decltype(wd)::w;
+        const Pack<W> xv = ldp<W>(x, i);
+        Pack<W> t = ldp<W>(y, i);
+#pragma unroll
+        for (int e = 0; e < W; ++e) t.v[e] = fmaf(a, xv.v[e], t.v[e]);
+        stp<W>(y, i, t);
+    });
 }
-// x += a p; r -= a q
-__global__ void __launch_bounds__(256) k_cg_xr(float* __restrict__ x, float* __restrict__ r, const float* __restrict__ p,
-                                               const float* __restrict__ q, float a, long long N)
+// q += a p and the total p . q in one pass.
+__global__ void __launch_bounds__(256) k_axpy_dot(float* __restrict__ q, const float* __restrict__ p, float a,
+                                                  long long N, double* part, unsigned int* tk, double* out)
 {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-        x[i] = fmaf(a, p[i], x[i]);
-        r[i] = fmaf(-a, q[i], r[i]);
-    }
-}
-// p = r + beta p
-__global__ void __launch_bounds__(256) k_xpby(float* __restrict__ p, const float* __restrict__ r, float beta,
-                                              long long N)
-{
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x)
-        p[i] = fmaf(beta, p[i], r[i]);
+    __shared__ double red[34];
+    DotAcc acc;
+    vec_loop(N, al16v(q, p), [&](auto wd, long long i) {
+        constexpr int W = decltype(wd)::w;
+        const Pack<W> pv = ldp<W>(p, i);
+        Pack<W> t = ldp<W>(q, i);
+#pragma unroll
+        for (int e = 0; e < W; ++e) {
+            t.v[e] = fmaf(a, pv.v[e], t.v[e]);
+            acc.add(pv.v[e], t.v[e]);
+        }
+        stp<W>(q, i, t);
+    });
+    grid_sum_finalize(block_pair_acc(acc, red), part, blockIdx.x, gridDim.x, tk, out);
 }
 // d = b - a (elementwise), for the residual
 __global__ void __launch_bounds__(256) k_sub(float* __restrict__ d, const float* __restrict__ b,
@@ -1242,23 +1323,40 @@ __global__ void __launch_bounds__(256) k_sub(float* __restrict__ d, const float*
 enum GenCg { kGBn = 0, kGRr = 1, kGPq = 2, kGRn = 3, kGDone = 4, kGIt = 5, kGBad = 6, kGHist = 8 };
 
 // x += alpha p, r -= alpha q with alpha = rr / pq (FP64, once per CTA), unless
-// the loop is done or pq is not positive (recorded by k_gcg_step).
+// the loop is done or pq is not positive (recorded by k_gcg_step); the total
+// r . r in the same pass.
 __global__ void __launch_bounds__(256) k_gcg_xr(float* __restrict__ x, float* __restrict__ r,
                                                 const float* __restrict__ p, const float* __restrict__ q,
-                                                const double* __restrict__ g, long long N)
+                                                const double* __restrict__ g, long long N, double* part,
+                                                unsigned int* tk, double* out)
 {
     __shared__ float a_s;
+    __shared__ double red[34];
     if (threadIdx.x == 0) {
         const double pq = g[kGPq];
         a_s = (g[kGDone] != 0.0 || !(pq > 0.0)) ? 0.f : (float)(g[kGRr] / pq);
     }
     __syncthreads();
     const float a = a_s;
-    if (a == 0.f) return;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-        x[i] = fmaf(a, p[i], x[i]);
-        r[i] = fmaf(-a, q[i], r[i]);
-    }
+    DotAcc acc;
+    vec_loop(N, al16v(x, r, p, q), [&](auto wd, long long i) {
+        constexpr int W = decltype(wd)::w;
+        Pack<W> rv = ldp<W>(r, i);
+        if (a != 0.f) {
+            const Pack<W> pv = ldp<W>(p, i), qv = ldp<W>(q, i);
+            Pack<W> xv = ldp<W>(x, i);
+#pragma unroll
+            for (int e = 0; e < W; ++e) {
+                xv.v[e] = fmaf(a, pv.v[e], xv.v[e]);
+                rv.v[e] = fmaf(-a, qv.v[e], rv.v[e]);
+            }
+            stp<W>(x, i, xv);
+            stp<W>(r, i, rv);
+        }
+#pragma unroll
+        for (int e = 0; e < W; ++e) acc.add(rv.v[e], rv.v[e]);
+    });
+    grid_sum_finalize(block_pair_acc(acc, red), part, blockIdx.x, gridDim.x, tk, out);
 }
 
 // p = r + beta p with beta = rr_new / rr, unless the loop is done.
@@ -1275,8 +1373,14 @@ __global__ void __launch_bounds__(256) k_gcg_p(float* __restrict__ p, const floa
     __syncthreads();
     if (skip) return;
     const float beta = b_s;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x)
-        p[i] = fmaf(beta, p[i], r[i]);
+    vec_loop(N, al16v(p, r), [&](auto wd, long long i) {
+        constexpr int W = decltype(wd)::w;
+        const Pack<W> rv = ldp<W>(r, i);
+        Pack<W> t = ldp<W>(p, i);
+#pragma unroll
+        for (int e = 0; e < W; ++e) t.v[e] = fmaf(beta, t.v[e], rv.v[e]);
+        stp<W>(p, i, t);
+    });
 }
 
 // The step's scalars (one thread): rr = rr_new, the iteration count, the
@@ -1309,19 +1413,19 @@ __global__ void k_gcg_init(double* __restrict__ g, double tol2, int max_iter)
                     ? 1.0 : 0.0;
 }
 
+static int dot_blocks(const Plan& P) { return (int)std::min<long long>(update_blocks(P.N), (long long)P.w.red_cap); }
+
 // a^T b on the device into *out (no host synchronisation).
 static cudaError_t dot_dev(Plan& P, const float* a, const float* b, double* out, cudaStream_t st)
 {
-    const int nb = (int)std::min<long long>(update_blocks(P.N), (long long)P.w.red_cap);
-    k_dot<<<nb, 256, 0, st>>>(a, b, P.N, part_slot(P, kPartRES), ticket(P, kTkRES), out);
+    k_dot<<<dot_blocks(P), 256, 0, st>>>(a, b, P.N, part_slot(P, kPartRES), ticket(P, kTkRES), out);
     return cudaGetLastError();
 }
 
 // a^T b on the device, returned to the host (synchronises `st`).
 static mh3d_status dot_host(Plan& P, const float* a, const float* b, cudaStream_t st, double* out)
 {
-    const int nb = (int)std::min<long long>(update_blocks(P.N), (long long)P.w.red_cap);
-    k_dot<<<nb, 256, 0, st>>>(a, b, P.N, part_slot(P, kPartRES), ticket(P, kTkRES), scal(P, kRES));
+    k_dot<<<dot_blocks(P), 256, 0, st>>>(a, b, P.N, part_slot(P, kPartRES), ticket(P, kTkRES), scal(P, kRES));
     MH3D_CK(P, cudaGetLastError());
     MH3D_CK(P, cudaMemcpyAsync(P.w.red_host, scal(P, kRES), sizeof(double), cudaMemcpyDeviceToHost, st));
     MH3D_CK(P, cudaStreamSynchronize(st));
@@ -1337,14 +1441,19 @@ struct mh3d_plan_s : public Plan {};
 
 namespace mh3d {
 
-// q = (A^T A + lambda I) p for the general model.
-static mh3d_status general_normal(Plan& P, const float* p, const float* bvec, double lam, float* q, cudaStream_t st)
+// q = (A^T A + lambda I) p for the general model; with pq, also p . q there
+// (device).
+static mh3d_status general_normal(Plan& P, const float* p, const float* bvec, double lam, float* q, double* pq,
+                                  cudaStream_t st)
 {
     mh3d_plan h = static_cast<mh3d_plan>(&P);
     mh3d_status s = mh3d_general_forward(h, p, bvec, P.w.portrait, st);
     if (s == MH3D_OK) s = mh3d_general_adjoint(h, P.w.portrait, bvec, q, st);
     if (s != MH3D_OK) return s;
-    k_axpy<<<update_blocks(P.N), 256, 0, st>>>(q, p, (float)lam, P.N);
+    if (pq)
+        k_axpy_dot<<<dot_blocks(P), 256, 0, st>>>(q, p, (float)lam, P.N, part_slot(P, kPartRES), ticket(P, kTkRES), pq);
+    else
+        k_axpy<<<update_blocks(P.N), 256, 0, st>>>(q, p, (float)lam, P.N);
     MH3D_CK(P, cudaGetLastError());
     return MH3D_OK;
 }
@@ -1362,7 +1471,7 @@ static mh3d_status general_cg(Plan& P, const void* d, const float* bvec, const m
     if ((s = mh3d_general_adjoint(h, d, bvec, w.rhs, st)) != MH3D_OK) return s;
     if (o.x0_dev) {
         MH3D_CK(P, cudaMemcpyAsync(w.x, o.x0_dev, vb, cudaMemcpyDeviceToDevice, st));
-        if ((s = general_normal(P, w.x, bvec, o.lambda, w.q, st)) != MH3D_OK) return s;
+        if ((s = general_normal(P, w.x, bvec, o.lambda, w.q, nullptr, st)) != MH3D_OK) return s;
         k_sub<<<nU, 256, 0, st>>>(w.r, w.rhs, w.q, P.N);
         MH3D_CK(P, cudaGetLastError());
     } else {
@@ -1394,11 +1503,10 @@ static mh3d_status general_cg(Plan& P, const void* d, const float* bvec, const m
         MH3D_CK(P, cudaStreamSynchronize(st));
         if (P.w.red_host[0] != 0.0) break;
         for (int c = 0; c < kChunk && launched < o.max_iter; ++c, ++launched) {
-            if ((s = general_normal(P, w.p, bvec, o.lambda, w.q, st)) != MH3D_OK) return s;
-            MH3D_CK(P, dot_dev(P, w.p, w.q, g + kGPq, st));
-            k_gcg_xr<<<nU, 256, 0, st>>>(w.x, w.r, w.p, w.q, g, P.N);
+            if ((s = general_normal(P, w.p, bvec, o.lambda, w.q, g + kGPq, st)) != MH3D_OK) return s;
+            k_gcg_xr<<<dot_blocks(P), 256, 0, st>>>(w.x, w.r, w.p, w.q, g, P.N, part_slot(P, kPartRES),
+                                                    ticket(P, kTkRES), g + kGRn);
             MH3D_CK(P, cudaGetLastError());
-            MH3D_CK(P, dot_dev(P, w.r, w.r, g + kGRn, st));
             k_gcg_p<<<nU, 256, 0, st>>>(w.p, w.r, g, P.N);
             k_gcg_step<<<1, 1, 0, st>>>(g, tol2, o.max_iter);
             MH3D_CK(P, cudaGetLastError());
@@ -1416,7 +1524,7 @@ static mh3d_status general_cg(Plan& P, const void* d, const float* bvec, const m
     else if (tol2 > 0.0 && rr > tol2 * bn && bn > 0.0 && rr > 0.0)
         status = MH3D_ERR_NOT_CONVERGED;
     // true residual ||A^T d - (A^T A + lambda I) x|| / ||A^T d||
-    if ((s = general_normal(P, w.x, bvec, o.lambda, w.q, st)) != MH3D_OK) return s;
+    if ((s = general_normal(P, w.x, bvec, o.lambda, w.q, nullptr, st)) != MH3D_OK) return s;
     k_sub<<<nU, 256, 0, st>>>(w.q, w.rhs, w.q, P.N);
     MH3D_CK(P, cudaGetLastError());
     double res2 = 0.0;
