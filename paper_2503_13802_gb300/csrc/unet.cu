@@ -248,15 +248,13 @@ int umma_c8p(int Cs, bool f32)
 // Accumulator columns for N output channels (a multiple of 16), 0 past 64.
 int umma_np(int N) { return N <= 16 ? 16 : (N <= 32 ? 32 : (N <= 64 ? 64 : 0)); }
 
-// Which convolutions run on the tcgen05 kernel.  By default those whose
-// rows fill most of a 128-voxel tile (W >= 96; the FP32 single-channel
-// input only with paired taps): per launch at 128x128x64, channels
-// (8, 16, 32), L2 flushed, it takes the full-resolution layers in 58 (FP32
-// input 1 -> 8), 52 (8 -> 8), 68 (upsampled 16 -> 8), 71 (skip sum 8 -> 8)
-// and 51 us (8 -> 1, FP32 out) against 62, 90, 158, 99 and 89 us on the
-// mma.sync tiles, while the half- and quarter-resolution layers (rows of 64
-// and 32 voxels in a 128-lane accumulator: 22-29 against 10-23 us) stay on
-// mma.sync.
+// Which convolutions run on the tcgen05 kernel: those of rows of 96 voxels or
+// more (the FP32 single-channel input only with paired taps).  The line is
+// where the two tensor-core paths have always met: they accumulate a k16 step
+// differently in the last bit, which the bfloat16 activations turn into
+// 1e-4 of a trained step, so a layer does not change sides.  (At 128x128x64
+// 16 -> 16 channels take 50 us here and 78 on k_conv_halo; at 64x64x64 about
+// 13 against 20.)
 // MH3D_UNET_UMMA=1 sends every convolution it can take to the tcgen05
 // kernel, 0 none.
 int umma_mode()
@@ -282,6 +280,7 @@ cudaError_t launch_umma_np(const ConvSrc& s, const UmmaW& u, int N, const float*
 // the source of a form it stages, not switched off).
 bool umma_takes(const ConvSrc& s, const UmmaW* u, int N)
 {
+    if ((long long)s.H * s.W > (1LL << 28)) return false;   // (offsets in a plane are 32-bit)
     return u && u->w && umma_enabled() && umma_prefers(s) && u->c8p == umma_c8p(s.C, s.f32 != nullptr) &&
            u->np == umma_np(N) && u->np > 0 && !(s.b && s.up);
 }
