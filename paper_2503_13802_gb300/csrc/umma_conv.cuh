@@ -4,41 +4,46 @@
 // descriptors and accumulating in tensor memory (TMEM); the epilogue reads
 // the accumulators back with tcgen05.ld.
 //
-// The GEMM of one output tile.  A tile is 8 x 16 voxels (x, y) of one z
-// plane; its accumulator D[128][NP] (FP32, NP >= N output channels, a
-// multiple of 16) has TMEM lane m = 8 (y - y0) + x - x0.  For every tap
-// (dz, dy, dx) and 16 input channels
-//     D[m][n] += sum_{c < 16} in[z + dz][y + dy][x + dx][c] W[n][tap][c]
-// is one tcgen05.mma with M = 128, N = NP, K = 16.
+// The GEMM of one tile.  A tile is 8 x 16 voxels (x, y) of one z plane; TMEM
+// lane m = 8 (y - y0) + x - x0.  An input plane p enters three output planes,
+// p + 1, p and p - 1 (taps dz = -1, 0, 1; the walk runs down z for a flipped
+// operand, so that every output still adds its planes in the order dz = -1, 0,
+// 1).  For every (dy, dx) and 16 input channels, with t the tap's dz + 1,
+//     D_{p + 1 - t}[m][n] += sum_{c < 16} in[p][y + dy][x + dx][c] W[n][t, dy, dx][c]
+// for the three t together is one tcgen05.mma with M = 128, N = 3 NP, K = 16
+// (NP >= the output channels, a multiple of 16).
+//
+// Accumulators: output plane o has the NP columns of TMEM slot o mod 3, so a
+// plane's MMA covers all three slots; which t a slot takes turns with p, and
+// the weights hold five groups t = 2, 1, 0, 2, 1 of which the B descriptor
+// starts at group 2 - (p + 1) mod 3.  After plane p's MMAs output p - 1 is
+// complete: the epilogue reads its slot and stores zeros there.
 //
 // Operand layout (no swizzle, K-major canonical layout: 8 rows x 16 bytes
 // per core matrix, rows 16 bytes apart, core matrices along M `SBO` and
 // along K `LBO` bytes apart):
-//   halo: input planes z - 1, z, z + 1 of 18 x 10 voxels, each
-//         [chunk of 8 channels][18 y][10 x][8]: eight x neighbours are a
-//         core matrix, the next y row is SBO = 160 bytes on, so the A operand
-//         of a tap is its plane started at voxel (1 + dy, 1 + dx) -- a
-//         descriptor offset, no data movement -- and the tap's second 8
-//         channels sit LBO = 180 voxels on;
-//   weights: [tap][chunk][NP][8], the B operand of (tap, chunk pair) one
-//         descriptor, its second 8 channels NP rows on.
+//   halo: input planes of 18 x 10 voxels, each [chunk of 8 channels][18 y][10
+//         x][8]: eight x neighbours are a core matrix, the next y row is SBO =
+//         160 bytes on, so the A operand of a tap is its plane started at voxel
+//         (1 + dy, 1 + dx) -- a descriptor offset, no data movement -- and the
+//         tap's second 8 channels sit LBO = 180 voxels on;
+//   weights: [dy, dx][chunk][5 groups][NP][8], the B operand of (dy, dx, chunk
+//         pair) one descriptor, its second 8 channels 5 NP rows on.
 // Chunks are padded to an even count with zeros (8 channels: one zero
 // chunk; the FP32 single-channel network input: channel 0 of chunk 0).
 //
-// A CTA of 128 threads walks z up a column of tiles with a ring of four
-// planes: one new plane a tile (1.4 input voxels staged per output voxel; a
-// tile of 128 x voxels stages its nine neighbour rows, or six a row for two
-// rows together) and two accumulators, so that the MMAs of plane z run while
-// the threads stage plane z + 2 and write plane z - 1 out.  The columns' planes
-// are one sequence, of which every CTA takes an equal run.
+// A CTA of 128 threads walks a column of tiles with two staged planes: one is
+// multiplied while the next is staged (1.4 input voxels staged per output
+// voxel).  The columns' planes are one sequence, of which every CTA takes an
+// equal run; a run of R outputs multiplies R + 2 planes.
 // What bounds it: a K = 16 MMA with M = 128 takes 69 cycles for N = 16 and 76
 // for N = 64, whatever the operands' strides and alignment (two chunks of A
-// read from shared memory), so 27 of them a tile put 16 -> 16 channels at
-// 128x128x64 at 52 us.  Issued from a branch on the thread index they take 133
-// cycles each; from one on elect.sync, 69.
-// Measured, us a layer at 128x128x64 (row tiles before): 16 -> 16 channels 50
-// (76), FP32 input -> 16 50 (84), upsampled 32 -> 16 100 (233), a whole forward
-// of channels (16, 32, 64, 128) 651 (900).
+// read from shared memory): with one MMA a tap, 27 a tile, 16 -> 16 channels at
+// 128x128x64 took 50 us, so the three dz of a plane share the read of A.
+// Issued from a branch on the thread index an MMA takes 133 cycles; from one on
+// elect.sync, 69.
+// Measured, a whole forward of channels (16, 32, 64, 128) at 128x128x64: 650 us
+// with one MMA a tap, 559 with three.  Every output bit stays.
 // The wait on an mbarrier is bounded (%globaltimer): on expiry the CTA
 // records MH3D_ERR_TIMEOUT in *status, frees its TMEM and returns.
 #pragma once
@@ -58,17 +63,18 @@ namespace umma {
 constexpr int kM = 128;                       // voxels per tile (TMEM lanes)
 constexpr int kX = 8, kY = 16;                // the tile's extents
 constexpr int kHX = kX + 2, kHV = kHX * (kY + 2);   // a staged plane: 180 voxels
-constexpr int kSlots = 4;                     // planes in the ring
+constexpr int kSlots = 2;                     // staged planes
+constexpr int kGroups = 5;                    // weight groups t = 2, 1, 0, 2, 1
 constexpr int kT = 128;                       // threads per CTA
 
 template <int C8P, int NP>
 struct Geom {
     static_assert(C8P % 2 == 0 && NP % 16 == 0 && NP >= 16 && NP <= 64, "operand shape");
-    static constexpr int kWBytes = 27 * C8P * NP * 16;
-    static constexpr int kPlane = C8P * kHV;               // 16-byte units of a staged plane
-    static constexpr int kCols = 2 * NP;                   // TMEM columns: two accumulators
-    static constexpr int kPer = (kPlane + kT - 1) / kT;    // units a thread stages
-    static constexpr size_t smem() { return 128 + (size_t)kWBytes + (size_t)kSlots * kPlane * 16; }
+    static constexpr int kWUnits = 9 * C8P * kGroups * NP;   // 16-byte units
+    static constexpr int kPlane = C8P * kHV;                 // 16-byte units of a staged plane
+    static constexpr int kCols = NP == 16 ? 64 : 4 * NP;     // TMEM columns: 3 NP, to a power of two
+    static constexpr int kPer = (kPlane + kT - 1) / kT;      // units a thread stages
+    static constexpr size_t smem() { return 128 + (size_t)kWUnits * 16 + (size_t)kSlots * kPlane * 16; }
 };
 
 // One thread of a converged warp.
@@ -140,6 +146,15 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16])
 #pragma unroll
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
+// Zeros into those columns.
+__device__ __forceinline__ void tmem_zero16(uint32_t taddr)
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1};" ::"r"(
+                     taddr),
+                 "r"(0)
+                 : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // Shared-memory matrix descriptor: start address, leading (K) and stride
@@ -172,7 +187,8 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // ---- the kernel --------------------------------------------------------------
 
 // Epilogue of one tile: warp w holds TMEM lanes 32 w .. 32 w + 31, columns
-// acc .. acc + NP - 1 = output channels; x, y: the lane's voxel.
+// acc .. acc + NP - 1 = output channels; x, y: the lane's voxel.  The columns
+// are zero afterwards.
 template <int NP, class OutT>
 __device__ __forceinline__ void epilogue(const ConvSrc& src, uint32_t acc, int z, int y, int x, int N,
                                          const float* __restrict__ bias, int relu, float osc, OutT* __restrict__ out)
@@ -182,8 +198,10 @@ __device__ __forceinline__ void epilogue(const ConvSrc& src, uint32_t acc, int z
 #pragma unroll
     for (int c0 = 0; c0 < NP; c0 += 16) {
         float a[16];
+        __syncwarp();   // (lanes outside the volume leave an iteration early)
         tmem_ld16(acc + ((uint32_t)(32 * warp) << 16) + (uint32_t)c0, a);
         tmem_ld_wait();
+        tmem_zero16(acc + ((uint32_t)(32 * warp) << 16) + (uint32_t)c0);
         if (x >= src.W || y >= src.H) continue;
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
@@ -217,50 +235,46 @@ __device__ __forceinline__ void epilogue(const ConvSrc& src, uint32_t acc, int z
     }
 }
 
-// The 27 x C8P / 2 MMAs of plane z into the accumulator at column acc,
-// committed to `bar` (one thread).  Descriptor start addresses count 16-byte
-// units, so offsets add to the low field.
+// The 9 x C8P / 2 MMAs of one plane into the three accumulators at column
+// acc, committed to `bar` (one thread).  g0: the first weight group.
+// Descriptor start addresses count 16-byte units, so offsets add to the low
+// field.
 //
 // Paired taps (sources of at most 8 channels, whose second chunk is zero
-// padding): one MMA takes two taps of the same (dz, dx) and neighbouring y --
-// row offsets 0 and 1, the second chunk LBO = one row on -- and a second MMA
-// the third row with a zero second chunk: 18 MMAs a tile instead of 27.  The
-// paired weights ([3 pz][3 px][2 g][2 c][NP][8], k_prep_umma_pair) are
-// indexed by plane offsets, the flip folded in.  (The third row's second
-// chunk is the row below it, one past the halo for the last tile row, where
-// the zeroed second chunk plane begins.)
+// padding): one MMA takes two taps of the same dx and neighbouring y -- row
+// offsets 0 and 1, the second chunk LBO = one row on -- and a second MMA the
+// third row with a zero second chunk: 6 MMAs a plane instead of 9.  The paired
+// weights ([3 px][2 g][2 c][5 groups][NP][8]) are indexed by plane offsets, the
+// flip folded in.  (The third row's second chunk is the row below it, one past
+// the halo for the last tile row, where the zeroed second chunk plane begins.)
 template <int C8P, int NP>
-__device__ __forceinline__ void issue_mmas(uint32_t acc, uint32_t sH_a, uint32_t sW_a, int z, int sgn, int pair,
+__device__ __forceinline__ void issue_mmas(uint32_t acc, uint32_t sP_a, uint32_t sW_a, int g0, int sgn, int pair,
                                            uint64_t* bar)
 {
-    constexpr uint32_t kIdesc = idesc_bf16(kM, NP);
-    using G = Geom<C8P, NP>;
-    const uint64_t b0 = smem_desc(sW_a, NP * 16, 128);
-    auto slot = [&](int plane) { return (uint64_t)(((plane + 1) & (kSlots - 1)) * G::kPlane); };
+    constexpr uint32_t kIdesc = idesc_bf16(kM, 3 * NP);
+    const uint64_t b0 = smem_desc(sW_a, kGroups * NP * 16, 128) + (uint64_t)(g0 * NP);
     if (pair) {
-        const uint64_t a0 = smem_desc(sH_a, kHX * 16, kHX * 16);
+        const uint64_t a0 = smem_desc(sP_a, kHX * 16, kHX * 16);
 #pragma unroll
-        for (int pzx = 0; pzx < 9; ++pzx)
+        for (int px = 0; px < 3; ++px)
 #pragma unroll
             for (int g = 0; g < 2; ++g)
-                mma_f16(acc, a0 + slot(z + pzx / 3 - 1) + (uint64_t)(2 * g * kHX + pzx % 3),
-                        b0 + (uint64_t)((pzx * 2 + g) * 2 * NP), kIdesc, (pzx | g) != 0);
+                mma_f16(acc, a0 + (uint64_t)(2 * g * kHX + px), b0 + (uint64_t)((px * 2 + g) * 2 * kGroups * NP), kIdesc, 1);
     } else {
-        const uint64_t a0 = smem_desc(sH_a, kHV * 16, kHX * 16) + (uint64_t)(kHX + 1);
-        const uint64_t az[3] = {a0 + slot(z - sgn), a0 + slot(z), a0 + slot(z + sgn)};
+        const uint64_t a0 = smem_desc(sP_a, kHV * 16, kHX * 16) + (uint64_t)(kHX + 1);
 #pragma unroll
-        for (int tap = 0; tap < 27; ++tap) {
-            const uint64_t at = az[tap / 9] + (uint64_t)(int64_t)(sgn * (((tap / 3) % 3 - 1) * kHX + tap % 3 - 1));
+        for (int yx = 0; yx < 9; ++yx) {
+            const uint64_t at = a0 + (uint64_t)(int64_t)(sgn * ((yx / 3 - 1) * kHX + yx % 3 - 1));
 #pragma unroll
             for (int ks = 0; ks < C8P / 2; ++ks)
-                mma_f16(acc, at + (uint64_t)(2 * ks * kHV), b0 + (uint64_t)((tap * C8P + 2 * ks) * NP), kIdesc,
-                        (tap | ks) != 0);
+                mma_f16(acc, at + (uint64_t)(2 * ks * kHV), b0 + (uint64_t)((yx * C8P + 2 * ks) * kGroups * NP), kIdesc, 1);
         }
     }
     mma_commit(bar);
 }
 
-// Wu: [27][C8P][NP][8] bfloat16 (k_prep_umma); out: [V][N] channels last.
+// Wu: [27][C8P][NP][8] bfloat16 (k_prep_umma), Wpair: [3 pz][3 px][2 g][2 c][NP][8]
+// (k_prep_umma_pair) or null; out: [V][N] channels last.
 //
 // Staging: 16-byte units, channels 8 c .. 8 c + 7 of a halo voxel, zero
 // outside the volume; only the cv chunks that carry channels (the padding
@@ -269,8 +283,7 @@ __device__ __forceinline__ void issue_mmas(uint32_t acc, uint32_t sH_a, uint32_t
 // upsampled bfloat16 sources: one cp.async a unit.  The skip sum (rounded to
 // bfloat16, as a stored sum would be; not upsampled) and the FP32 input
 // (rounded to bfloat16, channel 0) need arithmetic: their units are loaded
-// into registers before the wait on the previous tile's MMAs, combined and
-// stored after it.
+// into registers, combined and stored.
 template <int C8P, int NP, class OutT>
 __global__ void __launch_bounds__(kT) k_conv_umma(ConvSrc src, const __nv_bfloat16* __restrict__ Wu, int N,
                                                   const float* __restrict__ bias, int relu,
@@ -280,12 +293,12 @@ __global__ void __launch_bounds__(kT) k_conv_umma(ConvSrc src, const __nv_bfloat
     using G = Geom<C8P, NP>;
     constexpr int U = G::kPer;
     extern __shared__ unsigned char umma_raw[];
-    __shared__ __align__(8) uint64_t mbar[2];
+    __shared__ __align__(8) uint64_t mbar;
     __shared__ uint32_t tmem_base_s;
     unsigned char* base =
         reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(umma_raw) + 127) & ~uintptr_t(127));
-    uint4* sW = reinterpret_cast<uint4*>(base);                  // [27][C8P][NP]
-    uint4* sH = reinterpret_cast<uint4*>(base + G::kWBytes);     // [kSlots][C8P][kHV]
+    uint4* sW = reinterpret_cast<uint4*>(base);                  // [9][C8P][kGroups][NP]
+    uint4* sH = sW + G::kWUnits;                                 // [kSlots][C8P][kHV]
     const int tid = threadIdx.x, warp = tid >> 5;
     const int pair = Wpair != nullptr ? 1 : 0;
     const int sgn = src.flip ? -1 : 1;
@@ -295,15 +308,19 @@ __global__ void __launch_bounds__(kT) k_conv_umma(ConvSrc src, const __nv_bfloat
         tmem_relinquish();
     }
     if (tid == 0) {
-        mbar_init(&mbar[0], 1);
-        mbar_init(&mbar[1], 1);
+        mbar_init(&mbar, 1);
         fence_barrier_init();
     }
     const int cv = src.f32 ? 1 : src.C / 8;   // chunks carrying channels
     {
+        // unit (a, g, n) of the layout is row n of tap row t(g) of a; a = (dy, dx,
+        // chunk), or (px, g, c) of the paired taps
         const uint4* w4 = reinterpret_cast<const uint4*>(pair ? Wpair : Wu);
-        const int n16 = pair ? 9 * 2 * 2 * NP : G::kWBytes / 16;   // the paired layout is smaller
-        for (int i = tid; i < n16; i += kT) sW[i] = w4[i];
+        const int na = pair ? 3 * 2 * 2 : 9 * C8P;
+        for (int i = tid; i < na * kGroups * NP; i += kT) {
+            const int n = i % NP, ag = i / NP, a = ag / kGroups, g = ag - a * kGroups;
+            sW[i] = w4[((5 - g) % 3 * na + a) * NP + n];
+        }
         const int pad = (C8P - cv) * kHV;
         for (int q = 0; q < kSlots; ++q)
             for (int i = tid; i < pad; i += kT) sH[q * G::kPlane + cv * kHV + i] = make_uint4(0, 0, 0, 0);
@@ -321,13 +338,15 @@ __global__ void __launch_bounds__(kT) k_conv_umma(ConvSrc src, const __nv_bfloat
     const uint4* ga = reinterpret_cast<const uint4*>(src.a);
     const uint4* gb = reinterpret_cast<const uint4*>(src.b);
 
-    int j = 0;   // tiles so far: accumulator j & 1
+    int j = 0;   // planes so far: staged slot j & 1, phase j & 1 of the barrier
     bool ok = true;
-    auto wait_tile = [&](int t) {   // tile t's MMAs have completed (one thread spins)
-        ok = __syncthreads_and(tid != 0 || mbar_wait(&mbar[t & 1], (t >> 1) & 1, status));
+    auto wait_plane = [&](int t) {   // plane t's MMAs have completed (one thread spins)
+        ok = __syncthreads_and(tid != 0 || mbar_wait(&mbar, t & 1, status));
         tc_fence_after();
         return ok;
     };
+    const bool rev = src.flip && !pair;   // (the paired weights hold the flip)
+    auto real = [&](int p) { return rev ? src.D - 1 - p : p; };   // the walk's plane p
     // this CTA's run of the ntx x nty columns' planes
     const long long total = (long long)ntx * nty * src.D;
     long long pos = total * blockIdx.x / gridDim.x;
@@ -347,7 +366,7 @@ __global__ void __launch_bounds__(kT) k_conv_umma(ConvSrc src, const __nv_bfloat
             goff[k] = in ? ((yy >> sh) * (src.W >> sh) + (xx >> sh)) * cv + c : -1;
         }
         uint4 va[U], vb[U];
-        auto fetch = [&](int z) {   // register-staged sources: the plane's loads
+        auto fetch = [&](int z) {   // register-staged sources: the loads of source plane z
             if (!src.b && !src.f32) return;
             const bool zin = (unsigned)z < (unsigned)src.D;
 #pragma unroll
@@ -362,8 +381,8 @@ __global__ void __launch_bounds__(kT) k_conv_umma(ConvSrc src, const __nv_bfloat
                 }
             }
         };
-        auto put = [&](int z) {   // the plane into its slot
-            uint4* d = sH + ((z + 1) & (kSlots - 1)) * G::kPlane;
+        auto put = [&](int z, int slot) {   // the plane into its slot
+            uint4* d = sH + slot * G::kPlane;
             const bool zin = (unsigned)z < (unsigned)src.D;
 #pragma unroll
             for (int k = 0; k < U; ++k) {
@@ -387,33 +406,38 @@ __global__ void __launch_bounds__(kT) k_conv_umma(ConvSrc src, const __nv_bfloat
                 }
             }
         };
-        for (int z = zb - 1; z <= zb + 1; ++z) {
-            fetch(z);
-            put(z);
-        }
+        fetch(real(zb - 1));
+        put(real(zb - 1), j & 1);
         const int m = 32 * warp + (tid & 31), ex = x0 + m % kX, ey = y0 + m / kX;   // this thread's output voxel
-        for (int z = zb; z < ze; ++z, ++j) {
+        const uint32_t tlane = tmem + ((uint32_t)(32 * warp) << 16);
+#pragma unroll
+        for (int c0 = 0; c0 < 3 * NP; c0 += 16) tmem_zero16(tlane + (uint32_t)c0);
+        for (int p = zb - 1; p <= ze; ++p, ++j) {
+            tmem_st_wait();
             cp_async_wait_all();
             fence_proxy_async_smem();
             tc_fence_before();
             __syncthreads();
             if (warp == 0 && elect_one()) {
                 tc_fence_after();
-                issue_mmas<C8P, NP>(tmem + (uint32_t)((j & 1) * NP), sH_a, sW_a, z, sgn, pair, &mbar[j & 1]);
+                issue_mmas<C8P, NP>(tmem, sH_a + (uint32_t)((j & 1) * G::kPlane * 16), sW_a, 2 - (p + 1) % 3, sgn, pair,
+                                    &mbar);
             }
-            // plane z + 2 goes to the slot of plane z - 2, which the MMAs of
-            // tile z - 1 were the last to read
-            if (z + 1 < ze) fetch(z + 2);
-            if (z > zb && !wait_tile(j - 1)) break;
-            if (z + 1 < ze) put(z + 2);
-            if (z > zb) {
-                epilogue<NP>(src, tmem + (uint32_t)(((j - 1) & 1) * NP), z - 1, ey, ex, N, bias, relu, osc, out);
-                tc_fence_before();
+            if (p < ze) {   // into the other slot, whose MMAs have completed
+                fetch(real(p + 1));
+                put(real(p + 1), (j + 1) & 1);
+            }
+            if (!wait_plane(j)) break;
+            const uint32_t acc = (uint32_t)((p + 2) % 3 * NP);   // output p - 1
+            if (p > zb) {
+                epilogue<NP>(src, tmem + acc, real(p - 1), ey, ex, N, bias, relu, osc, out);
+            } else {
+#pragma unroll
+                for (int c0 = 0; c0 < NP; c0 += 16) tmem_zero16(tlane + acc + (uint32_t)c0);
             }
         }
-        if (!ok || !wait_tile(j - 1)) break;
-        epilogue<NP>(src, tmem + (uint32_t)(((j - 1) & 1) * NP), ze - 1, ey, ex, N, bias, relu, osc, out);
-        tc_fence_before();
+        if (!ok) break;
+        tmem_st_wait();
     }
     cp_async_wait_all();   // no copy lands after the CTA has gone
     tc_fence_before();

@@ -42,6 +42,9 @@ cudaError_t launch_umma_nb(const ConvSrc& s, const UmmaW& u, int N, const float*
         occ = std::max(1, std::min(std::min(by_smem, by_regs), std::min(2048 / umma::kT, 512 / G::kCols)));
     }
     const int ntx = (s.W + umma::kX - 1) / umma::kX, nty = (s.H + umma::kY - 1) / umma::kY;
+    // as many CTAs as fit: they hide each other's staging and epilogues (a
+    // forward at 128x128x64 takes 833, 661, 599, 583 and 559 us with 1, 2, 3, 4
+    // and 6 an SM), although shorter runs multiply more planes twice
     const int grid = (int)std::min<long long>((long long)ntx * nty * s.D, (long long)num_sms() * occ);
     fn<<<grid, umma::kT, smem, st>>>(s, u.w, N, bias, relu, oscale, out, ntx, nty, status,
                                      umma_pair() ? u.wp : nullptr);
