@@ -933,7 +933,7 @@ static void launch_scales(mh3d_unet n, const float* in, float gain, cudaStream_t
 {
     using namespace mh3d::unet;
     k_sumsq_part<<<kScaleBlocks, kThreads, 0, st>>>(in, n->V[0], n->spart);
-    k_scales<<<1, 320, 0, st>>>(n->spart, kScaleBlocks, n->V[0], gain, n->scales);
+    k_scales<<<1, kScaleT, 0, st>>>(n->spart, kScaleBlocks, n->V[0], gain, n->scales);
 }
 
 mh3d_status mh3d_unet_loss_grad(mh3d_unet n, const float* in, const float* target, float* grad, double* loss,

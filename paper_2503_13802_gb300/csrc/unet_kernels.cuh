@@ -1574,18 +1574,23 @@ static __global__ void k_sumsq_part(const float* __restrict__ in, long long V, d
 }
 
 constexpr int kScaleMax = 304;   // most partial sums of the RMS
+constexpr int kScaleT = 512;     // k_scales' threads
 
-// r = RMS of the input from the partials (in block order); scales =
-// {1 / r, r gain, 1 / (r gain)} (r = 1 for an all-zero input).
-static __global__ void k_scales(const double* __restrict__ part, int nb, long long V, float gain, float* __restrict__ scales)
+// r = RMS of the input from the partials; scales = {1 / r, r gain, 1 / (r gain)}
+// (r = 1 for an all-zero input).  One block; the partials add up in a tree (one
+// after the other they are a chain of 304 FP64 additions: 13.1 us against 4.3).
+static __global__ void __launch_bounds__(kScaleT) k_scales(const double* __restrict__ part, int nb, long long V,
+                                                           float gain, float* __restrict__ scales)
 {
-    __shared__ double ps[kScaleMax];   // every partial in flight at once, then added in order
-    for (int b = threadIdx.x; b < nb; b += blockDim.x) ps[b] = part[b];
+    __shared__ double ps[kScaleT];
+    ps[threadIdx.x] = (int)threadIdx.x < nb ? part[threadIdx.x] : 0.0;
     __syncthreads();
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double s = 0.0;
-#pragma unroll 8
-    for (int b = 0; b < nb; ++b) s += ps[b];
+    for (int w = kScaleT / 2; w > 0; w >>= 1) {
+        if ((int)threadIdx.x < w) ps[threadIdx.x] += ps[threadIdx.x + w];
+        __syncthreads();
+    }
+    if (threadIdx.x != 0) return;
+    const double s = ps[0];
     double r = sqrt(s / (double)V);
     if (!(r > 0.0)) r = 1.0;
     scales[0] = (float)(1.0 / r);
