@@ -513,16 +513,22 @@ cudaError_t launch_normal(const Plan& P, int mode, const RegArgs& reg, const flo
     // was, so recomputing them is harmless (the epilogue pass checks the flag).
     XArgs xf = xpass_args(P);
     xf.vin = t2;
-    xf.dout = portrait;
-    if ((e = run_xfwd(xf, st)) != cudaSuccess) return e;
-    // a padded plan's data cover the field of view only: A^T A becomes
-    // A^T M A with M the field-of-view mask of the portraits (windowed passes
-    // exchange the field of view's portraits only)
-    if (P.padded && !P.windowed && (e = mask_portraits(P, portrait, st)) != cudaSuccess) return e;
-    XArgs xa = xpass_args(P);
-    xa.din = portrait;
-    xa.vout = t1;
-    if ((e = !P.windowed && xw_available(xa, false) ? run_xadj_w(xa, st) : run_xadj(xa, st)) != cudaSuccess) return e;
+    if (P.windowed && xwin_available(xf)) {
+        // A^T M A along the drive axis in one pass
+        xf.vout = t1;
+        if ((e = run_xwin(xf, st)) != cudaSuccess) return e;
+    } else {
+        xf.dout = portrait;
+        if ((e = run_xfwd(xf, st)) != cudaSuccess) return e;
+        // a padded plan's data cover the field of view only: A^T A becomes
+        // A^T M A with M the field-of-view mask of the portraits (windowed passes
+        // exchange the field of view's portraits only)
+        if (P.padded && !P.windowed && (e = mask_portraits(P, portrait, st)) != cudaSuccess) return e;
+        XArgs xa = xpass_args(P);
+        xa.din = portrait;
+        xa.vout = t1;
+        if ((e = !P.windowed && xw_available(xa, false) ? run_xadj_w(xa, st) : run_xadj(xa, st)) != cudaSuccess) return e;
+    }
     TArgs tz2 = tpass_args(P, 2, t1, t2, P.Zhat_adj);
     if (cg) tz2.cg = cgp;
     if ((e = run_tpass(tz2, tpass_outer(P, 2), st)) != cudaSuccess) return e;

@@ -276,8 +276,10 @@ struct XShape {
     size_t smem = 0;
     bool ok = false;
 };
-XShape x_rt_shape(const RadixPlan& rpx, const RadixPlan& rpm, int s, int K, int rows, bool adj)
+enum XKind { kXFwd, kXAdj, kXWin };
+XShape x_rt_shape(const RadixPlan& rpx, const RadixPlan& rpm, int s, int K, int rows, XKind kind)
 {
+    const bool adj = kind == kXAdj;
     XShape h;
     if (s < 1 || s > 4 || rpx.nst < 1 || rpm.nst < 1 || rpm.nst > 3) return h;
     const int nx = rpx.n, mx = rpm.n, R = rpm.radix[rpm.nst - 1], NB = mx / R;
@@ -287,6 +289,7 @@ XShape x_rt_shape(const RadixPlan& rpx, const RadixPlan& rpm, int s, int K, int 
     auto smem = [&](int lgP, int lgK) {
         const size_t P = (size_t)1 << lgP, KG = (size_t)1 << lgK, a = 2 * (size_t)nx * (P + 1);
         const size_t b = 2 * (size_t)mx * (KG * P + 1) + (adj ? 2 * KG * 2 * P * h.pitch : 0);
+        if (kind == kXWin) return sizeof(float2) * (nx + mx + 3 * KG * nx + a / 2 + std::max(a / 2, b));
         return sizeof(float2) * (nx + mx + (adj ? 2 : 3) * KG * nx + std::max(a, b));
     };
     while (h.lgP > 1 && xpass_blocks(rows, 1 << h.lgP) < 152) --h.lgP;
@@ -337,7 +340,7 @@ cudaError_t run_xfwd(const XArgs& a0, cudaStream_t st)
 {
     if (!a0.win.on && ct_xpass_available(a0.nx, a0.s, a0.pairs)) return run_xfwd_ct(a0, st);
     XArgs a = a0;
-    const XShape h = x_rt_shape(a.rpx, a.rpm, a.s, a.K, a.rows, false);
+    const XShape h = x_rt_shape(a.rpx, a.rpm, a.s, a.K, a.rows, kXFwd);
     if (h.ok) {
         a.lgP = h.lgP;
         a.lgK = h.lgK;
@@ -355,7 +358,7 @@ cudaError_t run_xadj(const XArgs& a0, cudaStream_t st)
 {
     if (!a0.win.on && ct_xpass_available(a0.nx, a0.s, a0.pairs)) return run_xadj_ct(a0, st);
     XArgs a = a0;
-    const XShape h = x_rt_shape(a.rpx, a.rpm, a.s, a.K, a.rows, true);
+    const XShape h = x_rt_shape(a.rpx, a.rpm, a.s, a.K, a.rows, kXAdj);
     a.pitch = h.pitch;
     if (h.ok) {
         a.lgP = h.lgP;
@@ -369,6 +372,24 @@ cudaError_t run_xadj(const XArgs& a0, cudaStream_t st)
     const size_t per = sizeof(float2) * 3 * (size_t)a.nx, fixed = sizeof(float2) * ((size_t)a.nx + a.mx);
     const int lgP = x_any_lgP(per, fixed);
     return launch_x(k_xadj, a, lgP, 256, fixed + per * ((1 << lgP) + 1), st);
+}
+// Both passes in one where the portrait length has two radices (other lengths
+// take them one after the other).
+bool xwin_available(const XArgs& a)
+{
+    return a.win.on && a.rpm.nst == 2 && x_rt_shape(a.rpx, a.rpm, a.s, a.K, a.rows, kXWin).ok;
+}
+cudaError_t run_xwin(const XArgs& a0, cudaStream_t st)
+{
+    XArgs a = a0;
+    const XShape h = x_rt_shape(a.rpx, a.rpm, a.s, a.K, a.rows, kXWin);
+    a.lgP = h.lgP;
+    a.lgK = h.lgK;
+    const int grid = xpass_blocks(a.rows, 1 << h.lgP);
+    if (a.s == 1) return XRt<1>::win(a, grid, h.threads, h.smem, st);
+    if (a.s == 2) return XRt<2>::win(a, grid, h.threads, h.smem, st);
+    if (a.s == 3) return XRt<3>::win(a, grid, h.threads, h.smem, st);
+    return XRt<4>::win(a, grid, h.threads, h.smem, st);
 }
 cudaError_t run_xnrm(const XArgs& a0, cudaStream_t st)
 {

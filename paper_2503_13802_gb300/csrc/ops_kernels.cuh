@@ -196,6 +196,8 @@ bool xpass_windowed(int nx, int mx, int s, int pairs);
 cudaError_t run_tpass(const TArgs& a, int nouter, cudaStream_t st);
 cudaError_t run_xfwd(const XArgs& a, cudaStream_t st);
 cudaError_t run_xadj(const XArgs& a, cudaStream_t st);
+bool xwin_available(const XArgs& a);
+cudaError_t run_xwin(const XArgs& a, cudaStream_t st);   // A^T M A along the drive axis (padded plans)
 cudaError_t run_xnrm(const XArgs& a, cudaStream_t st);
 int tpass_blocks(int nx, int cols, int nouter);
 

@@ -41,6 +41,7 @@ struct XRt {
     static cudaError_t set_attributes(int optin);
     static cudaError_t fwd(const XArgs& a, int grid, int threads, size_t smem, cudaStream_t st);
     static cudaError_t adj(const XArgs& a, int grid, int threads, size_t smem, cudaStream_t st);
+    static cudaError_t win(const XArgs& a, int grid, int threads, size_t smem, cudaStream_t st);
 };
 
 }  // namespace mh3d
@@ -345,6 +346,159 @@ __global__ void __launch_bounds__(256, 2) k_xadj_rt(const __grid_constant__ XArg
     rt_stage_any<true, false>(BufLd{src, ld}, out, stage_rev(a.rpx, nstx - 1), lgP, twx);
 }
 
+// The end of the inverse transform, the window and the start of the forward
+// one on a butterfly: radix[0] at j + r NB1 on both sides.
+template <int R>
+__device__ __forceinline__ void x_window(const float2* b0, float2* b1, int ldq, int lgP, int lgQ, int NB1, int m0, int len,
+                                         uint32_t rowmask, const float2* twm)
+{
+    for (int idx = threadIdx.x; idx < NB1 << lgQ; idx += blockDim.x) {
+        const int q = idx & ((1 << lgQ) - 1), j = idx >> lgQ, p = q & ((1 << lgP) - 1);
+        const bool h0 = (rowmask >> (2 * p)) & 1u, h1 = (rowmask >> (2 * p + 1)) & 1u;
+        float2 v[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = b0[(j + r * NB1) * ldq + q];
+#pragma unroll
+        for (int r = 1; r < R; ++r) v[r] = c_mulc(v[r], twm[r * j]);
+        dft<R, true>(v);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const bool in = (unsigned)(j + r * NB1 - m0) < (unsigned)len;
+            v[r] = make_float2(in && h0 ? v[r].x : 0.f, in && h1 ? v[r].y : 0.f);
+        }
+        dft<R, false>(v);
+#pragma unroll
+        for (int r = 0; r < R; ++r) b1[(j * R + r) * ldq + q] = v[r];
+    }
+}
+
+// The drive-axis part of A^T M A on a padded plan (M: the field of view) in
+// one pass, for portrait lengths of two radices: every harmonic's portrait
+// rows exist in shared memory only, real as they are before their phase
+// (which cancels), so that no portraits go through memory.  Rounds of KG
+// harmonics as in the two passes above, two barriers a round: fold and first
+// inverse radix; last inverse radix, window and first forward radix; last
+// forward radix and sum.  CTAs whose rows all lie outside the window write
+// zeros.
+// Measured, 144 x 144 x 72 of a 128 x 128 x 64 window, s = 2, K = 8: a normal
+// operator takes 43 us less than with the two passes (28 and 47 us with 33 MB of
+// portraits written and read between them).
+template <int S>
+__global__ void __launch_bounds__(256, 2) k_xwin_rt(const __grid_constant__ XArgs a)
+{
+    extern __shared__ float2 sm[];
+    const int nx = a.nx, mx = a.mx, lgP = a.lgP, P = 1 << lgP, ld = P + 1;
+    const int lgQ = lgP + a.lgK, KG = 1 << a.lgK, ldq = (1 << lgQ) + 1;
+    float2* twx = sm;
+    float2* twm = twx + nx;
+    float2* xs = twm + mx;                // three rounds' spectra [KG][nx]
+    float2* s0 = xs + 3 * KG * nx;        // the rows' spectrum; later the sum
+    float2* s1 = s0 + nx * ld;            // the transforms' other buffer, the rounds' buffers
+    float2 *b0 = s1, *b1 = s1 + mx * ldq;
+    const int row0 = blockIdx.x * 2 * P, nstx = a.rpx.nst;
+    const PortraitRows pr{row0, a.rows, mx, a.win};
+    uint32_t rowmask = 0;
+    for (int r = 0; r < 2 * P; ++r) rowmask |= (uint32_t)(pr.row(row0 + r) >= 0) << r;
+    if (!rowmask) {
+        const int n = min(2 * P, a.rows - row0) * nx;
+        for (int i = threadIdx.x; i < n; i += blockDim.x) a.vout[(long long)row0 * nx + i] = 0.f;
+        return;
+    }
+    cp_table(twx, a.twx, nx);
+    cp_table(twm, a.twm, mx);
+    stage_spectra(xs, a, 0, min(2 * KG, a.K));   // rounds 0 and 1
+    {
+        float2* sp = (nstx & 1) ? s0 : s1;       // the last stage writes s0
+        rt_stage_any<false, false>(RowPairLd{a.vin, nx, row0, a.rows}, BufSt{sp, ld}, stage_fwd(a.rpx, 0), lgP, twx);
+        cp_table_wait();
+        __syncthreads();
+        for (int s = 1; s < nstx; ++s) {
+            float2* dst = sp == s0 ? s1 : s0;
+            rt_stage_buf<false>(sp, dst, ld, stage_fwd(a.rpx, s), lgP, twx);
+            __syncthreads();
+            sp = dst;
+        }
+    }
+    const int RM = a.rpm.radix[1], NB = (int)a.rpm.dnb[1].d, R1 = a.rpm.radix[0], NB1 = (int)a.rpm.dnb[0].d;
+    const int m0 = pr.m0(), len = pr.len();
+    const XThread t(a);
+    const int q = (t.kk << lgP) + t.p;
+    float2 V[kXRegs];
+#pragma unroll
+    for (int i = 0; i < kXRegs; ++i) V[i] = make_float2(0.f, 0.f);
+    for (int k0 = 0, rd = 0; k0 < a.K; k0 += KG, ++rd) {
+        const bool act = t.act && k0 + t.kk < a.K;
+        const float2* xk = xs + (rd % 3 * KG + t.kk) * nx;
+        if (act) {
+            x_radix<S>(RM, [&](auto rc) {
+                constexpr int R = decltype(rc)::value;
+                float2 G[R];
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const int m = t.j + r * NB;
+                    float2 g = c_mul(s0[m * ld + t.p], xk[m]);
+#pragma unroll
+                    for (int al = 1; al < S; ++al) g = c_add(g, c_mul(s0[(m + al * mx) * ld + t.p], xk[m + al * mx]));
+                    G[r] = g;
+                }
+                dft<R, true>(G);
+#pragma unroll
+                for (int r = 0; r < R; ++r) b0[(t.j * R + r) * ldq + q] = G[r];
+            });
+        }
+        __syncthreads();
+        // the spectra two rounds on, over those read a round ago
+        if (k0 + 2 * KG < a.K) stage_spectra(xs + (rd + 2) % 3 * KG * nx, a, k0 + 2 * KG, min(KG, a.K - k0 - 2 * KG));
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        x_radix<1>(R1, [&](auto rc) {
+            x_window<decltype(rc)::value>(b0, b1, ldq, lgP, lgQ, NB1, m0, len, rowmask, twm);
+        });
+        asm volatile("cp.async.wait_group 1;" ::: "memory");   // the next round's spectra
+        __syncthreads();
+        if (act) {
+            x_radix<S>(RM, [&](auto rc) {
+                constexpr int R = decltype(rc)::value;
+                float2 v[R];
+#pragma unroll
+                for (int r = 0; r < R; ++r) v[r] = b1[(t.j + r * NB) * ldq + q];
+#pragma unroll
+                for (int r = 1; r < R; ++r) v[r] = c_mul(v[r], twm[r * t.j]);
+                dft<R, false>(v);
+#pragma unroll
+                for (int al = 0; al < S; ++al)
+#pragma unroll
+                    for (int r = 0; r < R; ++r)
+                        V[al * R + r] = c_add(V[al * R + r], c_mulc(v[r], xk[t.j + r * NB + al * mx]));
+            });
+        }
+    }
+    __syncthreads();   // the spectrum and the last round's buffers have been read
+    for (int g = 0; g < KG; ++g) {   // the KG threads' sums, in order
+        if (t.act && t.kk == g) {
+            x_radix<S>(RM, [&](auto rc) {
+                constexpr int R = decltype(rc)::value;
+#pragma unroll
+                for (int al = 0; al < S; ++al)
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        float2* d = s0 + (t.j + r * NB + al * mx) * ld + t.p;
+                        *d = g == 0 ? V[al * R + r] : c_add(*d, V[al * R + r]);
+                    }
+            });
+        }
+        __syncthreads();
+    }
+    const RowPairSt out{a.vout, nx, row0, a.rows};
+    float2* src = s0;
+    for (int s = 0; s + 1 < nstx; ++s) {
+        float2* dst = src == s0 ? s1 : s0;
+        rt_stage_buf<true>(src, dst, ld, stage_rev(a.rpx, s), lgP, twx);
+        __syncthreads();
+        src = dst;
+    }
+    rt_stage_any<true, false>(BufLd{src, ld}, out, stage_rev(a.rpx, nstx - 1), lgP, twx);
+}
+
 template <class F>
 static cudaError_t xrt_opt_in(F* f, int optin)
 {
@@ -356,8 +510,9 @@ static cudaError_t xrt_opt_in(F* f, int optin)
 template <int S>
 cudaError_t XRt<S>::set_attributes(int optin)
 {
-    const cudaError_t e = xrt_opt_in(k_xfwd_rt<S>, optin);
-    return e != cudaSuccess ? e : xrt_opt_in(k_xadj_rt<S>, optin);
+    cudaError_t e = xrt_opt_in(k_xfwd_rt<S>, optin);
+    if (e == cudaSuccess) e = xrt_opt_in(k_xadj_rt<S>, optin);
+    return e != cudaSuccess ? e : xrt_opt_in(k_xwin_rt<S>, optin);
 }
 template <int S>
 cudaError_t XRt<S>::fwd(const XArgs& a, int grid, int threads, size_t smem, cudaStream_t st)
@@ -369,6 +524,12 @@ template <int S>
 cudaError_t XRt<S>::adj(const XArgs& a, int grid, int threads, size_t smem, cudaStream_t st)
 {
     k_xadj_rt<S><<<grid, threads, smem, st>>>(a);
+    return cudaGetLastError();
+}
+template <int S>
+cudaError_t XRt<S>::win(const XArgs& a, int grid, int threads, size_t smem, cudaStream_t st)
+{
+    k_xwin_rt<S><<<grid, threads, smem, st>>>(a);
     return cudaGetLastError();
 }
 template struct XRt<MH3D_XRT_S>;
