@@ -563,13 +563,15 @@ struct PortraitKLd {
 __device__ __forceinline__ void stage_portraits(float2* raw, int pitch, const float2* __restrict__ d,
                                                 const PortraitRows& g, int P)
 {
-    const int lane = (int)threadIdx.x & 31, nw = (int)blockDim.x >> 5, len = g.len();
-    for (int rr = (int)threadIdx.x >> 5; rr < 2 * P; rr += nw) {
+    const int len = g.len();
+    // short rows share a warp: 2^lgw lanes a row
+    const int lgw = len >= 32 ? 5 : 32 - __clz(len - 1), lane = (int)threadIdx.x & ((1 << lgw) - 1);
+    for (int rr = (int)threadIdx.x >> lgw; rr < 2 * P; rr += (int)blockDim.x >> lgw) {
         const long long o = g.row(g.row0 + rr);
         if (o < 0) continue;
         const float2* src = d + o;
         const uint32_t dst = (uint32_t)__cvta_generic_to_shared(raw + rr * pitch + g.m0());
-        for (int m = lane; m < len; m += 32)
+        for (int m = lane; m < len; m += 1 << lgw)
             asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst + 8 * m), "l"(src + m) : "memory");
     }
 }
