@@ -77,7 +77,7 @@ struct SolveWork {
     int hist_cap = 0;
     size_t red_cap = 0;
     int* flags_host = nullptr;    // pinned
-    double* red_host = nullptr;   // pinned, red_cap doubles
+    double* red_host = nullptr;   // pinned: max(red_cap, 16) doubles, then a short solve's history
     void* base = nullptr;         // one allocation backing the vectors
 };
 
