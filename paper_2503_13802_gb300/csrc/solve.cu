@@ -704,7 +704,7 @@ static mh3d_status cg_solve(Plan& P, const float2* d, const mh3d_solve_opts& o, 
     if ((s = cg_suffix(P, o, st)) != MH3D_OK) return s;
     // the image and, where the pinned buffer holds it, the whole history behind
     // the suffix, so that one wait ends the solve
-    // (a second wait and its copies: 20 us of a 465 us solve at 128x128x64)
+    // (a second wait and its copies: 14 us of a 461 us solve at 128x128x64)
     SolveWork& w = P.w;
     const size_t nh = (size_t)o.max_iter + 1;
     const bool one_wait = nh <= kHistPinned;
