@@ -23,6 +23,7 @@
 #include <cuda_runtime.h>
 
 #include "fastdiv.h"
+#include "halo_index.h"
 
 namespace mh3d {
 namespace unet {
@@ -468,24 +469,26 @@ constexpr size_t conv_stream_smem()
 }
 
 // A thread's halo units: unit i of the block is 8 channels of a halo voxel.
-// rel: element offset from the block's first voxel's; pos: hx | hy << 8 |
-// hz << 16.
+// rel: voxels from the block's first voxel (halo_index.h); pos: hx | hy << 8 |
+// hz << 16; c8: the unit's first channel (kThreads is a multiple of C / 8, so
+// a thread's units share it).
 template <int C, int TY, int PER>
 struct HaloUnits {
     using G = HaloGeom<TY>;
     static constexpr int kItems = G::HV * (C / 8);
-    int rel[PER], pos[PER];
+    static_assert(kThreads % (C / 8) == 0, "a thread's units take the same channels");
+    int rel[PER], pos[PER], c8;
     // the units first + j kThreads (j < PER)
     __device__ __forceinline__ void init(const ConvSrc& s, int first)
     {
-        const int Ws = s.up ? s.W >> 1 : s.W, Hs = s.up ? s.H >> 1 : s.H, sh = s.up ? 1 : 0;
+        const int sh = s.up ? 1 : 0;
+        c8 = first % (C / 8) * 8;
 #pragma unroll
         for (int j = 0; j < PER; ++j) {
-            const int i = first + j * kThreads, hv = i / (C / 8), c8 = i % (C / 8);
+            const int i = first + j * kThreads, hv = i / (C / 8);
             const int hx = hv % G::HX, hy = (hv / G::HX) % G::HY, hz = hv / (G::HX * G::HY);
             pos[j] = i < kItems ? hx | hy << 8 | hz << 16 : -1;
-            // block origins are even, so halving commutes with the offset
-            rel[j] = ((((hz - 1) >> sh) * Hs + ((hy - 1) >> sh)) * Ws + ((hx - 1) >> sh)) * C + c8 * 8;
+            rel[j] = halo_rel(hx, hy, hz, sh, s.H >> sh, s.W >> sh);
         }
     }
 };
@@ -504,16 +507,18 @@ template <int C, int TY, int PER>
 __device__ __forceinline__ void halo_load(const ConvSrc& s, const HaloUnits<C, TY, PER>& u, int x0, int y0, int z0,
                                           uint4 (&v)[PER])
 {
-    const int sh = s.up ? 1 : 0, Ws = s.W >> sh, Hs = s.H >> sh;
-    const long long base = (((long long)(z0 >> sh) * Hs + (y0 >> sh)) * Ws + (x0 >> sh)) * C;
+    const int sh = s.up ? 1 : 0;
+    const long long base = halo_base(x0, y0, z0, sh, s.H >> sh, s.W >> sh);
+    const __nv_bfloat16 *a = s.a + halo_elem(base, 0, C, u.c8), *b = s.b ? s.b + halo_elem(base, 0, C, u.c8) : nullptr;
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
         v[j] = make_uint4(0, 0, 0, 0);
         if (u.pos[j] < 0) continue;
         const int x = x0 - 1 + (u.pos[j] & 255), y = y0 - 1 + ((u.pos[j] >> 8) & 255), z = z0 - 1 + (u.pos[j] >> 16);
         if ((unsigned)x >= (unsigned)s.W || (unsigned)y >= (unsigned)s.H || (unsigned)z >= (unsigned)s.D) continue;
-        v[j] = *reinterpret_cast<const uint4*>(s.a + base + u.rel[j]);
-        if (s.b) v[j] = add_bf16x8(v[j], *reinterpret_cast<const uint4*>(s.b + base + u.rel[j]));
+        const long long o = halo_elem(0, u.rel[j], C, 0);
+        v[j] = *reinterpret_cast<const uint4*>(a + o);
+        if (b) v[j] = add_bf16x8(v[j], *reinterpret_cast<const uint4*>(b + o));
     }
 }
 template <int C, int PER>
