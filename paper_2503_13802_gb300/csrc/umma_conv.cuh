@@ -198,7 +198,7 @@ __device__ __forceinline__ void epilogue(const ConvSrc& src, uint32_t acc, int z
 #pragma unroll
     for (int c0 = 0; c0 < NP; c0 += 16) {
         float a[16];
-        __syncwarp();   // (lanes outside the volume leave an iteration early)
+        __syncwarp();   // lanes outside the volume leave an iteration early; tcgen05.ld and .st are warp-wide
         tmem_ld16(acc + ((uint32_t)(32 * warp) << 16) + (uint32_t)c0, a);
         tmem_ld_wait();
         tmem_zero16(acc + ((uint32_t)(32 * warp) << 16) + (uint32_t)c0);
@@ -233,6 +233,7 @@ __device__ __forceinline__ void epilogue(const ConvSrc& src, uint32_t acc, int z
                 out[v * N + n] = a[j];
         }
     }
+    __syncwarp();   // the caller's next tcgen05 instruction is warp-wide
 }
 
 // The 9 x C8P / 2 MMAs of one plane into the three accumulators at column
@@ -410,6 +411,7 @@ __global__ void __launch_bounds__(kT) k_conv_umma(ConvSrc src, const __nv_bfloat
         put(real(zb - 1), j & 1);
         const int m = 32 * warp + (tid & 31), ex = x0 + m % kX, ey = y0 + m / kX;   // this thread's output voxel
         const uint32_t tlane = tmem + ((uint32_t)(32 * warp) << 16);
+        __syncwarp();   // (staging skips the units a lane does not have)
 #pragma unroll
         for (int c0 = 0; c0 < 3 * NP; c0 += 16) tmem_zero16(tlane + (uint32_t)c0);
         for (int p = zb - 1; p <= ze; ++p, ++j) {

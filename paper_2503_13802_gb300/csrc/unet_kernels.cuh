@@ -652,6 +652,7 @@ __global__ void __launch_bounds__(kThreads, C <= 16 && BN <= 32 ? 2 : 1)
         int nx0 = 0, ny0 = 0, nz0 = 0;
         if (next < ntiles) block_origin<TY>(src, next, nx0, ny0, nz0);
         if (PRE && next < ntiles) halo_load(src, hu, nx0, ny0, nz0, hv);
+        __syncwarp();   // (lanes load different units; ldmatrix and mma.sync are warp-wide)
         float acc[2][NT][4];
 #pragma unroll
         for (int i = 0; i < 2; ++i)
