@@ -298,6 +298,8 @@ XArgs xpass_args(const Plan& P)
     a.twm = P.am.tw;
     a.rpx = P.ax.rp;
     a.rpm = P.am.rp;
+    a.rpa[0] = P.adj_rp[0];
+    a.rpa[1] = P.adj_rp[1];
     a.nx = P.nx;
     a.mx = P.mx;
     a.s = P.s;
@@ -317,7 +319,6 @@ XArgs xpass_args(const Plan& P)
         a.win.dny = a.dny;
     }
     a.pairs = P.tile.xpass_pairs;
-    a.kg = P.tile.xpass_kgroup;
     a.vec4 = (P.nx % 4 == 0 && ((uintptr_t)P.sens % 16) == 0) ? 1 : 0;
     a.reg.nx = P.nx;
     a.reg.ny = P.ny;
@@ -643,7 +644,7 @@ mh3d_status mh3d_plan_create(const mh3d_geometry* g, void* stream, mh3d_plan* ou
     P->az.n = nz;
     P->am.n = mx;
     if (!radix_plan(nx, P->ax.rp) || !radix_plan(ny, P->ay.rp) || !radix_plan(nz, P->az.rp) ||
-        !radix_plan(mx, P->am.rp, xpass_max_last(P->s))) {
+        !radix_plan(mx, P->am.rp, xpass_max_last(P->s)) || !radix_plan(mx, P->adj_rp[0], kAdjMaxLast) || !radix_plan(mx, P->adj_rp[1], kAdjMaxLastLean)) {
         delete P;
         return MH3D_ERR_UNSUPPORTED_SIZE;
     }
@@ -652,7 +653,7 @@ mh3d_status mh3d_plan_create(const mh3d_geometry* g, void* stream, mh3d_plan* ou
     // run-time ones read and write the field of view's portraits directly
     // (144 x 144 x 72 with 128 x 128 x 64 inside, K = 8: the mask took 23 us
     // an application, padding 30 us, and the passes moved the padding too)
-    P->windowed = P->padded && xpass_windowed(nx, mx, P->s, P->tile.xpass_pairs);
+    P->windowed = P->padded && xpass_windowed(nx, P->s, P->tile.xpass_pairs);
     if (xfwd_smem_bytes(nx, mx, P->tile.xpass_pairs, P->tile.xpass_kgroup) > kSmemBudget ||
         tpass_smem_bytes(std::max(ny, nz), P->tile.tpass_cols) > kSmemBudget) {
         delete P;

@@ -588,7 +588,7 @@ int gen_lg_pencils(const RadixPlan& rp, long long np)
 {
     int nb = rp.n, lg = 3;
     for (int s = 0; s < rp.nst; ++s) nb = std::min(nb, rp.n / rp.radix[s]);
-    while ((1 << lg) < kGPMax && (nb << lg) < kGT && (np >> (lg + 1)) >= 152) ++lg;
+    while ((1 << lg) < kGPMax && (nb << lg) < kGT && (np >> (lg + 1)) >= num_sms()) ++lg;
     return lg;
 }
 

@@ -141,6 +141,7 @@ struct Plan {
     const float* sens = nullptr;  // borrowed device pointer (may be null)
 
     AxisPlan ax, ay, az, am;      // x (drive), y, z, portrait length mx
+    RadixPlan adj_rp[2]{};        // the portrait length's schedules in k_xadj
     TileChoice tile;
 
     // device tables (FP32 complex)
@@ -202,14 +203,22 @@ std::vector<cplx> drive_spectrum(int n, double dx, int k, double gamma, double g
 std::vector<cplx> transverse_spectrum(int n, double d, double gt);
 std::vector<cplx> twiddles(int n);
 double hermitian_lambda_max(const std::vector<cplx>& H, int s);
-// Largest last radix of the portrait length's schedule: the run-time
-// drive-axis passes keep the s aliases of a butterfly in registers (s R <= 24
-// complex values; 0: any, those passes do not run).
-inline int xpass_max_last(int s) { return s == 1 ? 16 : (s == 2 ? 12 : (s == 3 ? 8 : (s == 4 ? 6 : 0))); }
+// Largest last radix of the portrait length's schedule.  The run-time
+// drive-axis passes of s <= 4 keep the s aliases of a butterfly in registers
+// (s R <= 24 complex values); for s >= 5 the last radix carries the fold, s
+// products an element, on few butterflies (mx = 16 as 16: 38 us a forward at
+// 96 x 96 x 96, s = 6, K = 8; as 4 x 4: 29).
+inline int xpass_max_last(int s) { return s == 1 ? 16 : (s == 2 ? 12 : (s == 3 ? 8 : 6)); }
+// The same in k_xadj: one stage up to 12 samples, where the second costs more
+// than idle threads, two for 16 (16 x 144 x 96, s = 1, K = 11: 37 us as 16, 33 as 4 x 4);
+// in its lean form (x_any_shape) two from 8 on.
+constexpr int kAdjMaxLast = 12, kAdjMaxLastLean = 6;
 // max_last: largest radix of the schedule's last stage (0: any)
 bool radix_plan(int n, RadixPlan& pl, int max_last = 0);
 
-// ops.cu: operator launches (all asynchronous on `st`)
+// ops.cu
+int num_sms();   // SMs of the device
+// operator launches (all asynchronous on `st`)
 struct OpCtx;
 cudaError_t launch_forward(const Plan& P, const float* rho, float2* d, float* t1, float* t2, cudaStream_t st);
 cudaError_t launch_adjoint(const Plan& P, const float2* d, float* rho, float* t1, float* t2, cudaStream_t st);

@@ -150,18 +150,27 @@ cudaError_t run_tpass(const TArgs& a, int nouter, cudaStream_t st)
 // ---------------------------------------------------------------------------
 // X pass kernels (s = 1..4: ops_xrt.cuh)
 // ---------------------------------------------------------------------------
-// Any s and any length (one included), one harmonic at a time: the aliases
-// folded, or the harmonics summed, in shared memory.
-__global__ void __launch_bounds__(256) k_xfwd(const __grid_constant__ XArgs a)
+// Any s and any length (one included), rounds of KG harmonics whose pencils
+// are transformed together; the aliases folded, or the harmonics summed, in
+// shared memory.  They serve s >= 5 and the adjoint of portrait rows below 64
+// samples (kXAdjStaged), where a transform has few butterflies: what bounds
+// them is the latency of a round's stages, so a round takes up to eight
+// harmonics.  Measured, us a call: forward 96 x 96 x 96, s = 6, K = 8: 27.9
+// (79.6 with one harmonic a round); adjoint 24 x 128 x 128, s = 1, K = 12: 43.6
+// (74.3 on k_xadj_rt).
+// The pencils of a round of kn harmonics: P times the power of two from kn on.
+__device__ __forceinline__ int round_pencils(int kn, int P) { return P << (32 - __clz(kn - 1)); }
+
+__global__ void __launch_bounds__(256, 3) k_xfwd(const __grid_constant__ XArgs a)
 {
     extern __shared__ float2 sm[];
-    const int nx = a.nx, mx = a.mx, P = 1 << a.lgP, ld = P + 1;
+    const int nx = a.nx, mx = a.mx, P = 1 << a.lgP, ld = P + 1, KG = 1 << a.lgK, ldq = KG * P + 1;
     float2* twx = sm;
     float2* twm = twx + nx;
     float2* A0 = twm + mx;
     float2* A1 = A0 + nx * ld;
     float2* B0 = A1 + nx * ld;
-    float2* B1 = B0 + mx * ld;
+    float2* B1 = B0 + mx * ldq;
     for (int i = threadIdx.x; i < nx; i += blockDim.x) twx[i] = a.twx[i];
     for (int i = threadIdx.x; i < mx; i += blockDim.x) twm[i] = a.twm[i];
     __syncthreads();
@@ -169,38 +178,40 @@ __global__ void __launch_bounds__(256) k_xfwd(const __grid_constant__ XArgs a)
     const int res = fft_result_index(a.rpx.nst);
     float2* Ar = res ? A1 : A0;
     fft_run<false, false, true>(a.rpx, RowPairLd{a.vin, nx, row0, a.rows}, BufSt{Ar, ld}, A0, A1, ld, P, twx);
-    for (int k = 0; k < a.K; ++k)
-        fft_run<true, true, false>(a.rpm, FoldLd{Ar, ld, a.Xhat + (long long)k * nx, mx, a.s},
-                                   PortraitSt{a.dout + (long long)k * a.M, __ldg(a.phase + k),
-                                              PortraitRows{row0, a.rows, mx, a.win}},
-                                   B0, B1, ld, P, twm);
+    const PortraitRows pr{row0, a.rows, mx, a.win};
+    for (int k0 = 0; k0 < a.K; k0 += KG)
+        fft_run<true, true, false>(a.rpm, FoldLd{Ar, ld, a.Xhat + (long long)k0 * nx, nx, mx, a.s, a.lgP, a.K - k0},
+                                   RoundSt{a, pr, k0}, B0, B1, ldq, round_pencils(min(KG, a.K - k0), P), twm);
 }
 
-__global__ void __launch_bounds__(256) k_xadj(const __grid_constant__ XArgs a)
+// OCC: CTAs an SM holds by registers (4 spills where a radix is above 8).
+template <int OCC>
+__global__ void __launch_bounds__(256, OCC) k_xadj(const __grid_constant__ XArgs a)
 {
     extern __shared__ float2 sm[];
-    const int nx = a.nx, mx = a.mx, P = 1 << a.lgP, ld = P + 1;
+    const int nx = a.nx, mx = a.mx, P = 1 << a.lgP, ld = P + 1, KG = 1 << a.lgK, ldq = KG * P + 1;
     float2* twx = sm;
     float2* twm = twx + nx;
     float2* acc = twm + mx;            // [nx][ld]
-    float2* S0 = acc + nx * ld;        // two buffers of nx ld (the transforms of mx use their starts)
-    float2* S1 = S0 + nx * ld;
+    float2* S0 = acc + nx * ld;        // the inverse's buffers [nx][ld] or a round's [mx][ldq]
+    float2 *S1 = S0 + nx * ld, *B1 = S0 + mx * ldq;
     for (int i = threadIdx.x; i < nx; i += blockDim.x) twx[i] = a.twx[i];
     for (int i = threadIdx.x; i < mx; i += blockDim.x) twm[i] = a.twm[i];
     __syncthreads();
     const int row0 = blockIdx.x * 2 * P;
-    float2* Fr = fft_result_index(a.rpm.nst) ? S1 : S0;
-    for (int k = 0; k < a.K; ++k) {
-        fft_run<false, false, true>(a.rpm,
-                                    PortraitKLd{a.din + (long long)k * a.M, __ldg(a.phase + k),
-                                                PortraitRows{row0, a.rows, mx, a.win}},
-                                    BufSt{Fr, ld}, S0, S1, ld, P, twm);
-        // acc[w][p] (+)= conj(Xhat_k[w]) F[w mod mx][p]
+    float2* Fr = fft_result_index(a.rpm.nst) ? B1 : S0;
+    const PortraitRows pr{row0, a.rows, mx, a.win};
+    for (int k0 = 0; k0 < a.K; k0 += KG) {
+        const int kn = min(KG, a.K - k0);
+        fft_run<false, false, true>(a.rpm, RoundKLd{a, pr, k0}, BufSt{Fr, ldq}, S0, B1, ldq, round_pencils(kn, P), twm);
+        // acc[w][p] (+)= sum_kk conj(Xhat_k0+kk[w]) F_kk[w mod mx][p]
         for (int idx = threadIdx.x; idx < nx * P; idx += blockDim.x) {
             const int p = idx & (P - 1), w = idx >> a.lgP;
-            const int m = w % mx;
-            const float2 v = c_mulc(Fr[m * ld + p], __ldg(a.Xhat + (long long)k * nx + w));
-            acc[w * ld + p] = (k == 0) ? v : c_add(acc[w * ld + p], v);
+            const int m = w - (int)a.dmx.div((uint32_t)w) * mx;
+            const float2* x = a.Xhat + (long long)k0 * nx + w;
+            float2 v = k0 == 0 ? make_float2(0.f, 0.f) : acc[w * ld + p];
+            for (int kk = 0; kk < kn; ++kk) v = c_add(v, c_mulc(Fr[m * ldq + (kk << a.lgP) + p], __ldg(x + kk * nx)));
+            acc[w * ld + p] = v;
         }
         __syncthreads();
     }
@@ -260,6 +271,18 @@ __global__ void __launch_bounds__(256) k_xnrm(const __grid_constant__ XArgs a)
     if (a.count_iter) cg_count_iteration(a.cg);
 }
 
+int num_sms()
+{
+    static const int n = [] {
+        int dev = 0, v = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v < 1)
+            v = 1;
+        return v;
+    }();
+    return n;
+}
+
 int xpass_blocks(int rows, int pairs) { return (rows + 2 * pairs - 1) / (2 * pairs); }
 
 namespace {
@@ -274,7 +297,7 @@ constexpr size_t kXSmemMax = 200 * 1024;
 struct XShape {
     int lgP = 3, lgK = 0, threads = 0, pitch = 0;
     size_t smem = 0;
-    bool ok = false;
+    bool ok = false, lean = false;
 };
 enum XKind { kXFwd, kXAdj, kXWin };
 XShape x_rt_shape(const RadixPlan& rpx, const RadixPlan& rpm, int s, int K, int rows, XKind kind)
@@ -292,7 +315,7 @@ XShape x_rt_shape(const RadixPlan& rpx, const RadixPlan& rpm, int s, int K, int 
         if (kind == kXWin) return sizeof(float2) * (nx + mx + 3 * KG * nx + a / 2 + std::max(a / 2, b));
         return sizeof(float2) * (nx + mx + (adj ? 2 : 3) * KG * nx + std::max(a, b));
     };
-    while (h.lgP > 1 && xpass_blocks(rows, 1 << h.lgP) < 152) --h.lgP;
+    while (h.lgP > 1 && xpass_blocks(rows, 1 << h.lgP) < num_sms()) --h.lgP;
     while (h.lgP > 0 && ((NB << h.lgP) > 256 || smem(h.lgP, 0) > kXSmemMax)) --h.lgP;
     if ((NB << h.lgP) > 256 || smem(h.lgP, 0) > kXSmemMax) return h;
     while (h.lgK < 2 && (1 << h.lgK) < K && (NB << (h.lgP + h.lgK + 1)) <= 256 && smem(h.lgP, h.lgK + 1) <= kXSmemMax / 2) ++h.lgK;
@@ -303,29 +326,71 @@ XShape x_rt_shape(const RadixPlan& rpx, const RadixPlan& rpm, int s, int K, int 
     return h;
 }
 
-// Row pairs of the any-s kernels: as many as fit, at most 16.
-int x_any_lgP(size_t per_pair, size_t fixed)
+// Launch shape of the any-s kernels: up to 8 harmonics a round while two CTAs
+// fit an SM's shared memory; 16 row pairs a CTA, or 8 where that shortens the
+// SM's queue -- the row pairs of its CTAs, in whole turns of as many as it
+// holds at a time (three by their 80 registers) -- and every stage of a round
+// still has a butterfly for each thread (192 x 192 x 64, s = 6, K = 16, adjoint:
+// 101 us with 16, 81 with 8; 128 x 128 x 64, s = 8, K = 8: 31 and 37); fewer where
+// they leave SMs without a CTA.
+// The adjoint of short rows in more than one turn of CTAs is bound by its
+// throughput: the lean form holds four CTAs an SM, cuts 8, 9 and 12 samples
+// into two stages and takes 32 row pairs where that costs no harmonics (us a
+// call with three CTAs and 16 pairs, and so: 16 x 256 x 128, s = 2, K = 3 31.2 and
+// 27.2; 16 x 72 x 256, s = 1, K = 9 42 and 35; in one turn, 16 x 64 x 64, s = 2, K = 10,
+// 18 and 21).
+XShape x_any_shape(const XArgs& a, XKind kind)
 {
-    int lgP = 4;
-    while (lgP > 0 && fixed + per_pair * ((1 << lgP) + 1) > kXSmemMax) --lgP;
-    return lgP;
+    constexpr int kLgK = 3, kLeanRow = 24;
+    const int nx = a.nx, mx = a.mx, K = a.K, sms = num_sms();
+    XShape h;
+    auto ctas = [&](int lgP) { return (xpass_blocks(a.rows, 1 << lgP) + sms - 1) / sms; };
+    h.lean = kind == kXAdj && mx <= kLeanRow && ctas(4) > 3;
+    const int resident = h.lean ? 4 : 3;
+    auto smem = [&](int lgP, int lgK) {
+        const size_t x = (size_t)nx * ((1 << lgP) + 1), q = (size_t)mx * ((1 << (lgP + lgK)) + 1);
+        return sizeof(float2) * (nx + mx + (kind == kXAdj ? x + 2 * std::max(x, q) : 2 * x + 2 * q));
+    };
+    auto lg_harmonics = [&](int lgP) {
+        int k = 0;
+        while (k < kLgK && (1 << k) < K && smem(lgP, k + 1) <= std::max(kXSmemMax / 2, smem(lgP, k))) ++k;
+        return k;
+    };
+    auto queue = [&](int lgP) {
+        const int n = ctas(lgP);
+        const int r = std::max(1, std::min(resident, (int)(228 * 1024 / (smem(lgP, lg_harmonics(lgP)) + 1024))));
+        return (n <= r ? n : (n + r - 1) / r * r) << lgP;
+    };
+    const RadixPlan& rp = kind == kXAdj ? a.rpa[h.lean] : a.rpm;
+    int nb = mx;   // butterflies of the smallest stage
+    for (int s = 0; s < rp.nst; ++s) nb = std::min(nb, mx / rp.radix[s]);
+    h.lgP = 4;
+    if (h.lean) {
+        if (lg_harmonics(5) == lg_harmonics(4) && queue(5) <= queue(4)) h.lgP = 5;
+    } else if ((nb << (3 + lg_harmonics(3))) >= 256 && queue(3) < queue(4)) {
+        h.lgP = 3;
+    }
+    while (h.lgP > 1 && xpass_blocks(a.rows, 1 << h.lgP) < sms) --h.lgP;
+    while (h.lgP > 0 && smem(h.lgP, 0) > kXSmemMax) --h.lgP;
+    h.lgK = lg_harmonics(h.lgP);
+    h.threads = 256;
+    h.smem = smem(h.lgP, h.lgK);
+    h.ok = true;
+    return h;
 }
 
-template <class F>
-cudaError_t launch_x(F* f, XArgs& a, int lgP, int threads, size_t smem, cudaStream_t st)
-{
-    a.lgP = lgP;
-    f<<<xpass_blocks(a.rows, 1 << lgP), threads, smem, st>>>(a);
-    return cudaGetLastError();
-}
+// Portrait rows from which the adjoint stages them and keeps its sums in
+// registers (k_xadj_rt).  Shorter ones have too few butterflies a harmonic for
+// its 128 registers and a round of four harmonics; us a call on it and on
+// k_xadj: 24 samples (24 x 128 x 128, s = 1, K = 12) 74 and 44, 48 (48 x 216 x 64,
+// s = 1, K = 14) 84 and 57, 54 (162 x 108 x 81, s = 3, K = 5) 53 and 47; longer ones
+// gain: 108 (216 x 216 x 72, s = 2, K = 13) 207 and 219, 192 (192 x 64 x 64, s = 1, K = 5)
+// 37 and 42.
+constexpr int kXAdjStaged = 64;
 
 }  // namespace
 
-bool xpass_windowed(int nx, int mx, int s, int pairs)
-{
-    (void)mx;
-    return !ct_xpass_available(nx, s, pairs);
-}
+bool xpass_windowed(int nx, int s, int pairs) { return !ct_xpass_available(nx, s, pairs); }
 
 int xnrm_rt_pairs(const RadixPlan& rpx)
 {
@@ -350,17 +415,19 @@ cudaError_t run_xfwd(const XArgs& a0, cudaStream_t st)
         if (a.s == 3) return XRt<3>::fwd(a, grid, h.threads, h.smem, st);
         return XRt<4>::fwd(a, grid, h.threads, h.smem, st);
     }
-    const size_t per = sizeof(float2) * 2 * ((size_t)a.nx + a.mx), fixed = sizeof(float2) * ((size_t)a.nx + a.mx);
-    const int lgP = x_any_lgP(per, fixed);
-    return launch_x(k_xfwd, a, lgP, 256, fixed + per * ((1 << lgP) + 1), st);
+    const XShape g = x_any_shape(a, kXFwd);
+    a.lgP = g.lgP;
+    a.lgK = g.lgK;
+    k_xfwd<<<xpass_blocks(a.rows, 1 << g.lgP), g.threads, g.smem, st>>>(a);
+    return cudaGetLastError();
 }
 cudaError_t run_xadj(const XArgs& a0, cudaStream_t st)
 {
     if (!a0.win.on && ct_xpass_available(a0.nx, a0.s, a0.pairs)) return run_xadj_ct(a0, st);
     XArgs a = a0;
-    const XShape h = x_rt_shape(a.rpx, a.rpm, a.s, a.K, a.rows, kXAdj);
-    a.pitch = h.pitch;
+    const XShape h = a.mx >= kXAdjStaged ? x_rt_shape(a.rpx, a.rpm, a.s, a.K, a.rows, kXAdj) : XShape();
     if (h.ok) {
+        a.pitch = h.pitch;
         a.lgP = h.lgP;
         a.lgK = h.lgK;
         const int grid = xpass_blocks(a.rows, 1 << h.lgP);
@@ -369,9 +436,15 @@ cudaError_t run_xadj(const XArgs& a0, cudaStream_t st)
         if (a.s == 3) return XRt<3>::adj(a, grid, h.threads, h.smem, st);
         return XRt<4>::adj(a, grid, h.threads, h.smem, st);
     }
-    const size_t per = sizeof(float2) * 3 * (size_t)a.nx, fixed = sizeof(float2) * ((size_t)a.nx + a.mx);
-    const int lgP = x_any_lgP(per, fixed);
-    return launch_x(k_xadj, a, lgP, 256, fixed + per * ((1 << lgP) + 1), st);
+    const XShape g = x_any_shape(a, kXAdj);
+    a.rpm = a.rpa[g.lean];
+    a.lgP = g.lgP;
+    a.lgK = g.lgK;
+    a.dmx = FastDiv(a.mx);
+    const int grid = xpass_blocks(a.rows, 1 << g.lgP);
+    if (g.lean) k_xadj<4><<<grid, g.threads, g.smem, st>>>(a);
+    else k_xadj<3><<<grid, g.threads, g.smem, st>>>(a);
+    return cudaGetLastError();
 }
 // Both passes in one where the portrait length has two radices (other lengths
 // take them one after the other).
@@ -430,7 +503,8 @@ cudaError_t ops_set_attributes()
     if ((e = XRt<2>::set_attributes(optin)) != cudaSuccess) return e;
     if ((e = XRt<3>::set_attributes(optin)) != cudaSuccess) return e;
     if ((e = XRt<4>::set_attributes(optin)) != cudaSuccess) return e;
-    if ((e = opt_in_smem(k_xadj, optin)) != cudaSuccess) return e;
+    if ((e = opt_in_smem(k_xadj<3>, optin)) != cudaSuccess) return e;
+    if ((e = opt_in_smem(k_xadj<4>, optin)) != cudaSuccess) return e;
     if ((e = opt_in_smem(k_xnrm, optin)) != cudaSuccess) return e;
     if ((e = xw_set_attributes()) != cudaSuccess) return e;
     return ct_set_attributes(optin);

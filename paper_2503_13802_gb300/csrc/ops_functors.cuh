@@ -461,13 +461,14 @@ struct RowPairSt {
     }
 };
 
-// Forward: one harmonic's portrait spectrum at bin m =
-// sum_{j < s} A[m + j mx] Xhat_k[m + j mx]   (the fold that realises P).
+// Forward: the portrait spectrum of pencil q = kk P + p (harmonic kk of a
+// round) at bin m = sum_{j < s} A[m + j mx] Xhat_kk[m + j mx]   (the fold that
+// realises P).
 struct FoldLd {
     const float2* A;
     int ldA;
-    const float2* __restrict__ xk;   // Xhat + k nx
-    int mx, s;
+    const float2* __restrict__ xk;   // the round's first harmonic's spectrum
+    int nx, mx, s, lgP, left;        // left: harmonics from the round's first on
     struct At {
         const float2* A;
         int ldA;
@@ -483,7 +484,11 @@ struct FoldLd {
             return acc;
         }
     };
-    __device__ __forceinline__ At at(int p) const { return At{A + p, ldA, xk, mx, s}; }
+    // (a harmonic past the last folds with the last's spectrum and is not stored)
+    __device__ __forceinline__ At at(int q) const
+    {
+        return At{A + (q & ((1 << lgP) - 1)), ldA, xk + min(q >> lgP, left - 1) * nx, mx, s};
+    }
 };
 
 // One harmonic's portrait rows (row0 + 2p, row0 + 2p + 1) of a pencil.
@@ -553,6 +558,30 @@ struct PortraitKLd {
     {
         const long long i0 = g.row(g.row0 + 2 * p), i1 = g.row(g.row0 + 2 * p + 1);
         return At{i0 >= 0 ? d + i0 : nullptr, i1 >= 0 ? d + i1 : nullptr, ph, g.m0(), g.len()};
+    }
+};
+
+// A round's portraits: pencil q = kk P + p of harmonic k0 + kk.
+struct RoundSt {
+    const XArgs& a;
+    const PortraitRows& g;
+    int k0;
+    __device__ __forceinline__ PortraitSt::At at(int q) const
+    {
+        const int k = k0 + (q >> a.lgP);
+        if (k >= a.K) return PortraitSt::At{nullptr, nullptr, make_float2(0.f, 0.f), 0, 0};
+        return PortraitSt{a.dout + (long long)k * a.M, __ldg(a.phase + k), g}.at(q & ((1 << a.lgP) - 1));
+    }
+};
+struct RoundKLd {
+    const XArgs& a;
+    const PortraitRows& g;
+    int k0;
+    __device__ __forceinline__ PortraitKLd::At at(int q) const
+    {
+        const int k = k0 + (q >> a.lgP);
+        if (k >= a.K) return PortraitKLd::At{nullptr, nullptr, make_float2(0.f, 0.f), 0, 0};
+        return PortraitKLd{a.din + (long long)k * a.M, __ldg(a.phase + k), g}.at(q & ((1 << a.lgP) - 1));
     }
 };
 

@@ -125,11 +125,11 @@ struct XArgs {
     const float2* twx = nullptr;
     const float2* twm = nullptr;
     RadixPlan rpx{}, rpm{};
+    RadixPlan rpa[2]{};              // the portrait length's schedules in k_xadj
     int nx = 1, mx = 1, s = 1, K = 1;
     int rows = 1;
     long long M = 1;                 // rows * mx
     int pairs = 16;                  // row pairs per CTA
-    int kg = 4;                      // harmonics per transform batch
     int kpc = 0;                     // specialised forward: harmonics per CTA (grid.y groups; 0: all)
     int vec4 = 0;                    // nx % 4 == 0 and every vector 16-byte aligned
     // normal-mode epilogue
@@ -148,7 +148,7 @@ struct XArgs {
     int* status = nullptr;           // device status word for bounded-wait timeouts
     int ks = 0;                      // warp-centric passes: warps per row group (0: default)
     FastDiv dny;                     // by ny (rows are z ny + y)
-    FastDiv dmx;                     // by mx (run-time normal pass)
+    FastDiv dmx;                     // by mx (run-time normal pass, k_xadj)
     int lgP = 0;                     // run-time kernels: log2 of the row pairs per CTA
     int lgK = 0;                     // run-time passes: log2 of the harmonics per round
     int pitch = 0;                   // run-time adjoint: float2 between staged portrait rows
@@ -182,15 +182,10 @@ __host__ __forceinline__ size_t xadj_smem_bytes(int nx, int mx, int pairs, int k
     size_t a = 2 * (size_t)mx * (kg * pairs + 1), b = 2 * (size_t)nx * (pairs + 1);
     return sizeof(float2) * (size_t)(nx + mx + (size_t)nx * (pairs + 1) + (a > b ? a : b));
 }
-__host__ __forceinline__ size_t xnrm_smem_bytes(int nx, int pairs)
-{
-    return sizeof(float2) * (size_t)(nx + 2 * nx * (pairs + 1));
-}
-
 // Row pairs per CTA of the run-time normal pass.
 int xnrm_rt_pairs(const RadixPlan& rpx);
 // Whether the run-time drive-axis passes take a windowed (padded) mesh.
-bool xpass_windowed(int nx, int mx, int s, int pairs);
+bool xpass_windowed(int nx, int s, int pairs);
 
 // Launchers (ops.cu).
 cudaError_t run_tpass(const TArgs& a, int nouter, cudaStream_t st);

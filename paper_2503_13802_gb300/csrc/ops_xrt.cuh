@@ -1,4 +1,5 @@
-// Run-time drive-axis passes for s = 1..4 (any length 2^a 3^b), and helpers
+// Run-time drive-axis passes for s = 1..4 (any length 2^a 3^b; the adjoint from
+// portrait rows of kXAdjStaged samples on), and helpers
 // shared with the other run-time kernels (ops.cu).  Each S is compiled in a
 // file of its own (ops_x1.cu .. ops_x4.cu).
 #pragma once
@@ -122,18 +123,6 @@ __device__ __forceinline__ void stage_spectra(float2* dst, const XArgs& a, int k
                      : "memory");
 }
 
-// A round's portraits: pencil q = kk P + p of harmonic k0 + kk.
-struct RoundSt {
-    const XArgs& a;
-    const PortraitRows& g;
-    int k0;
-    __device__ __forceinline__ PortraitSt::At at(int q) const
-    {
-        const int k = k0 + (q >> a.lgP);
-        if (k >= a.K) return PortraitSt::At{nullptr, nullptr, make_float2(0.f, 0.f), 0, 0};
-        return PortraitSt{a.dout + (long long)k * a.M, __ldg(a.phase + k), g}.at(q & ((1 << a.lgP) - 1));
-    }
-};
 struct RoundLd {   // from the staged rows [kk][2 P][pitch]
     const XArgs& a;
     const float2* raw;

@@ -6,6 +6,7 @@
 #include <algorithm>
 #include <cstdlib>
 
+#include "mh3d_internal.h"
 #include "unet_kernels.cuh"
 
 namespace mh3d {
@@ -20,17 +21,6 @@ struct UmmaW {
     int c8p = 0, np = 0;
     int sgn = 1;                   // -1: the input-gradient (flipped) operand
 };
-
-inline int num_sms()
-{
-    static int v = -1;
-    if (v < 0) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v < 1) v = 1;
-    }
-    return v;
-}
 
 inline int smem_optin()
 {
