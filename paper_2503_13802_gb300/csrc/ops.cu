@@ -152,7 +152,7 @@ cudaError_t run_tpass(const TArgs& a, int nouter, cudaStream_t st)
 // ---------------------------------------------------------------------------
 // Any s and any length (one included), rounds of KG harmonics whose pencils
 // are transformed together; the aliases folded, or the harmonics summed, in
-// shared memory.  They serve s >= 5 and the adjoint of portrait rows below 64
+// shared memory.  They serve s >= 5 and the adjoint of portrait rows below 108
 // samples (kXAdjStaged), where a transform has few butterflies: what bounds
 // them is the latency of a round's stages, so a round takes up to eight
 // harmonics.  Measured, us a call: forward 96 x 96 x 96, s = 6, K = 8: 27.9
@@ -381,12 +381,12 @@ XShape x_any_shape(const XArgs& a, XKind kind)
 
 // Portrait rows from which the adjoint stages them and keeps its sums in
 // registers (k_xadj_rt).  Shorter ones have too few butterflies a harmonic for
-// its 128 registers and a round of four harmonics; us a call on it and on
+// its 128 registers and a round of four harmonics.  Us a call on it and on
 // k_xadj: 24 samples (24 x 128 x 128, s = 1, K = 12) 74 and 44, 48 (48 x 216 x 64,
-// s = 1, K = 14) 84 and 57, 54 (162 x 108 x 81, s = 3, K = 5) 53 and 47; longer ones
-// gain: 108 (216 x 216 x 72, s = 2, K = 13) 207 and 219, 192 (192 x 64 x 64, s = 1, K = 5)
-// 37 and 42.
-constexpr int kXAdjStaged = 64;
+// s = 1, K = 14) 84 and 57, 64 (256 x 128 x 64, s = 4, K = 8) 60 and 56, 96 (96 x 96 x
+// 64, s = 1, K = 6) 43 and 30; 108 (216 x 216 x 72, s = 2, K = 13) 210 and 270,
+// 192 (192 x 128 x 54, s = 1, K = 13) 130 and 172.
+constexpr int kXAdjStaged = 108;
 
 }  // namespace
 

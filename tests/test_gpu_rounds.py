@@ -1,6 +1,6 @@
 """The drive-axis passes of any subset factor, up to eight harmonics a round,
 against the FP64 oracle: one harmonic, rounds that are exactly full and last
-rounds of one and of several harmonics, portrait rows of 1 to 54 samples
+rounds of one and of several harmonics, portrait rows of 1 to 108 samples
 (none, one and two transform stages), 16 and 8 row pairs a CTA, row counts
 that leave a ragged last CTA.
 
@@ -26,6 +26,8 @@ CASES = {
     "short_k9": params((16, 81, 64), s=1, kmin=2, kmax=10),
     "short_k11": params((54, 27, 16), s=1, kmin=2, kmax=12),
     "short_s3": params((162, 9, 8), s=3, r=2, kmin=2, kmax=4),
+    "row96": params((96, 18, 16), s=1, kmin=2, kmax=6),
+    "row108": params((216, 9, 4), s=2, r=1, kmin=2, kmax=6),
     "short_s4": params((32, 36, 27), s=4, r=1, kmin=2, kmax=17),
     "short_ragged": params((18, 3, 9), s=2, r=1, kmin=2, kmax=6),
 }
