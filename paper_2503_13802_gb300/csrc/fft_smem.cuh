@@ -446,7 +446,10 @@ __device__ __forceinline__ void fft_run(const RadixPlan& pl, const LD& first, co
         } else if (isLast) {
             rt_stage_any<INV, LAST_PFAST>(BufLd{srcb, lds}, last, g, lgP, tw);
         } else {
-            rt_stage_buf<INV>(srcb, dstb, lds, g, lgP, tw);
+            // inlined: a call gives the kernel a stack, and its launch behind
+            // another one then takes 1 us longer (general model at 16 x 16 x 16,
+            // K = 3: a forward of nine launches 45 us with it, 38 so)
+            rt_stage_any<INV, true>(BufLd{srcb, lds}, BufSt{dstb, lds}, g, lgP, tw);
         }
         __syncthreads();
     }
