@@ -208,10 +208,16 @@ __global__ void __launch_bounds__(256, OCC) k_xadj(const __grid_constant__ XArgs
         for (int idx = threadIdx.x; idx < nx * P; idx += blockDim.x) {
             const int p = idx & (P - 1), w = idx >> a.lgP;
             const int m = w - (int)a.dmx.div((uint32_t)w) * mx;
-            const float2* x = a.Xhat + (long long)k0 * nx + w;
-            float2 v = k0 == 0 ? make_float2(0.f, 0.f) : acc[w * ld + p];
-            for (int kk = 0; kk < kn; ++kk) v = c_add(v, c_mulc(Fr[m * ldq + (kk << a.lgP) + p], __ldg(x + kk * nx)));
-            acc[w * ld + p] = v;
+            const float2 *x = a.Xhat + (long long)k0 * nx + w, *f = Fr + m * ldq + p;
+            float2 t[4];   // four short sums (at most 8 harmonics) round less than one
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                t[i] = i < kn ? c_mulc(f[i << a.lgP], __ldg(x + i * nx)) : make_float2(0.f, 0.f);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (4 + i < kn) t[i] = c_add(t[i], c_mulc(f[(4 + i) << a.lgP], __ldg(x + (4 + i) * nx)));
+            const float2 v = c_add(c_add(t[0], t[1]), c_add(t[2], t[3]));
+            acc[w * ld + p] = k0 == 0 ? v : c_add(acc[w * ld + p], v);
         }
         __syncthreads();
     }
@@ -341,7 +347,7 @@ XShape x_rt_shape(const RadixPlan& rpx, const RadixPlan& rpm, int s, int K, int 
 // 18 and 21).
 XShape x_any_shape(const XArgs& a, XKind kind)
 {
-    constexpr int kLgK = 3, kLeanRow = 24;
+    constexpr int kLgK = 3, kLeanRow = 24;   // (k_xadj sums at most 8 harmonics a round)
     const int nx = a.nx, mx = a.mx, K = a.K, sms = num_sms();
     XShape h;
     auto ctas = [&](int lgP) { return (xpass_blocks(a.rows, 1 << lgP) + sms - 1) / sms; };
