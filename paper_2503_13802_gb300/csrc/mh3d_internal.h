@@ -46,7 +46,7 @@ struct AxisPlan {
 struct TileChoice {
     int tpass_cols = 16;          // x columns per T-pass CTA (pencils = cols / 2)
     int xpass_pairs = 16;         // row pairs per X-pass CTA
-    int xpass_kgroup = 4;         // harmonics transformed together in the X pass
+    int xpass_kgroup = 4;         // harmonics a round in the acceptance rule (xfwd_smem_bytes)
     int threads = 256;
     // chosen by mh3d_plan_autotune (0 = the library's default; environment
     // switches of the same name still take precedence for A/B checks)
