@@ -30,11 +30,11 @@
  * [cout][3][3][3][cin] (taps dz, dy, dx), then b [cout].
  * Loss of mh3d_unet_loss_grad: sum((out - target)^2) / (2 V).
  *
- * The convolutions run on the tcgen05 tensor cores (accumulators in tensor
- * memory) where the source is bfloat16 with 8..32 channels in multiples of
- * 8 or the FP32 input, at most 64 outputs, and rows of 96 voxels or more;
- * on mma.sync tiles otherwise.  MH3D_UNET_UMMA=0 / 1 sends none / every
- * convolution it can take to the tcgen05 kernel.
+ * By default the convolutions of rows of 96 voxels or more run on the tcgen05
+ * tensor cores (accumulators in tensor memory), where the source is bfloat16
+ * with 8..32 channels in multiples of 8 or the FP32 input and there are at most
+ * 64 outputs; the others run on mma.sync.  The kernel itself takes rows of any
+ * length: MH3D_UNET_UMMA=1 sends every convolution it can take to it, 0 none.
  *
  * Sizes: nx, ny, nz multiples of 2^(L-1) (4 for mh3d_unet_create); channels
  * in 1..64 (mh3d_unet_create) or 1..128 (mh3d_unet_create_levels).  Volumes are
