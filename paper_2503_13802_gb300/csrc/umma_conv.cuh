@@ -36,12 +36,13 @@
 // multiplied while the next is staged (1.4 input voxels staged per output
 // voxel).  The columns' planes are one sequence, of which every CTA takes an
 // equal run; a run of R outputs multiplies R + 2 planes.
-// What bounds it: a K = 16 MMA with M = 128 takes 69 cycles for N = 16 and 76
-// for N = 64, whatever the operands' strides and alignment (two chunks of A
-// read from shared memory): with one MMA a tap, 27 a tile, 16 -> 16 channels at
-// 128x128x64 took 50 us, so the three dz of a plane share the read of A.
-// Issued from a branch on the thread index an MMA takes 133 cycles; from one on
-// elect.sync, 69.
+// What bounds it: the MMAs' reads of A from shared memory.  Back to back on one
+// CTA a K = 16 MMA with M = 128 takes 39, 44, 48, 56 and 96 cycles for N = 16, 48,
+// 64, 96 and 192 whatever its A offset, so the three dz of a plane in one MMA
+// cost little more than one; nine of them with their commit and wait, a
+// plane's chain, take 69, 72, 101 and 142 cycles each for N = 16, 48, 96 and 192.
+// Issued from a branch on the thread index instead of elect.sync: 45 and 79
+// for N = 16.
 // Measured, a whole forward of channels (16, 32, 64, 128) at 128x128x64: 650 us
 // with one MMA a tap, 559 with three.  Every output bit stays.
 // The wait on an mbarrier is bounded (%globaltimer): on expiry the CTA

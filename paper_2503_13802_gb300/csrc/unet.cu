@@ -249,12 +249,12 @@ int umma_c8p(int Cs, bool f32)
 int umma_np(int N) { return N <= 16 ? 16 : (N <= 32 ? 32 : (N <= 64 ? 64 : 0)); }
 
 // Which convolutions run on the tcgen05 kernel: those of rows of 96 voxels or
-// more (the FP32 single-channel input only with paired taps).  The line is
-// where the two tensor-core paths have always met: they accumulate a k16 step
-// differently in the last bit, which the bfloat16 activations turn into
-// 1e-4 of a trained step, so a layer does not change sides.  (At 128x128x64
-// 16 -> 16 channels take 50 us here and 78 on k_conv_halo; at 64x64x64 about
-// 13 against 20.)
+// more (the FP32 single-channel input only with paired taps).  Us a layer there
+// and on mma.sync: at 128x128x64 the input 1 -> 16 30 and 60, 16 -> 16 36 and 63,
+// upsampled 32 -> 16 58 and 122; at 64x64x64 16, 18 and 23 against 16, 18 and 34;
+// their coarse levels 32 -> 32 at 64x64x32 26 against 29, at 32x32x32 13 against 9.
+// The two accumulate a k16 step differently in the last bit, which the bfloat16
+// activations turn into 1e-4 of a trained step.
 // MH3D_UNET_UMMA=1 sends every convolution it can take to the tcgen05
 // kernel, 0 none.
 int umma_mode()
